@@ -211,6 +211,12 @@ cudaError_t launch_edge_records(int n, const T* eta, T* rec, cudaStream_t s);
 template <typename T>
 cudaError_t launch_stencil_edge(int mode, const LevelOp<T>& op, const StencilArgs<T>& a, cudaStream_t s, int zch_req);
 
+// Small levels (stencil_point.cu): eight lanes per vertex, on grids of up to
+// kPointMaxN cubes per axis (the reasons for the limit stand there)
+constexpr int kPointMaxN = 32;
+template <typename T>
+cudaError_t launch_stencil_point(int mode, const LevelOp<T>& op, const StencilArgs<T>& a, cudaStream_t s);
+
 // ------------------------------------------------------------ batched forms
 // One (problem, level) operator application inside a batched launch.
 template <typename TS, typename T>
@@ -231,6 +237,10 @@ cudaError_t launch_stencil_batch(int mode, bool coarse, const StencilTask<TS, T>
 template <typename T>
 cudaError_t launch_stencil_edge_batch(int mode, const StencilTask<T, T>* tasks, int ntasks, int64_t ntiles,
                                       cudaStream_t s);
+// small levels of a batch: max_n = cubes per axis of the largest task
+template <typename T>
+cudaError_t launch_stencil_point_batch(int mode, const StencilTask<T, T>* tasks, int ntasks, int max_n,
+                                       cudaStream_t s);
 // whether a step of this kind runs the edge form: every level of an FP64
 // context (its coefficient records exist on every level); the FP32 cycle and
 // the Stokes operator run the per-cube kernel
@@ -249,8 +259,7 @@ struct XferTask {
   int64_t count;        // work items of the task
   const void* src;
   void* dst;
-  const double* m1;     // coarsest solve: L^-1 column-major
-  const double* m2;     // coarsest solve: L^-1 row-major
+  const double* m1;     // coarsest solve: inverse of the coarsest matrix
   const double* sc;     // skip when sc[MS_DONE] != 0, or nullptr
 };
 enum XferKind { XK_RESTRICT = 0, XK_PROLONG_ADD, XK_D2F, XK_F2D, XK_COARSE, XK_PROLONG, XK_COPY64 };
@@ -288,16 +297,18 @@ cudaError_t launch_f2d(const float* in, double* out, int64_t n, cudaStream_t s);
 cudaError_t launch_coarse_assemble(const LevelOp<double>& op, double* dense, cudaStream_t s);
 cudaError_t launch_cholesky(double* a, int m, int* status, cudaStream_t s);
 cudaError_t launch_trinv(const double* l, int m, double* linv_cm, double* linv_rm, cudaStream_t s);
+cudaError_t launch_coarse_inverse(const double* linv_rm, int m, double* ainv, cudaStream_t s);
 template <typename T>
-cudaError_t launch_coarse_solve(int n, const double* linv_cm, const double* linv_rm, const T* r, T* z,
-                                cudaStream_t s);
+cudaError_t launch_coarse_solve(int n, const double* ainv, const T* r, T* z, cudaStream_t s);
 cudaError_t launch_pressure_mass(int np, const double* eta_f, double* pmass, double* pmass_inv, cudaStream_t s);
 // stencil storage of the flagged elements' Galerkin matrices (stencil_store.cu)
 cudaError_t launch_mark_vertices(int n, const uint8_t* flags, uint8_t* mark, cudaStream_t s);
 cudaError_t launch_stencil_assemble(int n, int64_t n_sv, const int32_t* slist, const int32_t* fidx, const double* gca,
                                     double* sten, cudaStream_t s);
 cudaError_t launch_stencil_to_f32(int64_t n_sv, const double* s64, float* s32, float* scale, cudaStream_t s);
-cudaError_t launch_masked_coef(int64_t E, const double* mean, const int32_t* fidx, double* coefm, cudaStream_t s);
+// DCA coefficient of a coarse level with the flagged elements zeroed, in FP64 or rounded to FP32
+template <typename T>
+cudaError_t launch_masked_coef(int64_t E, const double* mean, const int32_t* fidx, T* coefm, cudaStream_t s);
 cudaError_t launch_start_vector(int n, double* v, cudaStream_t s);
 
 // Stokes / Krylov kernels (krylov.cu)

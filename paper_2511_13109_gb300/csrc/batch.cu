@@ -67,14 +67,16 @@ __global__ void convert_batch_kernel(const XferTask* __restrict__ tasks) {
     out[i] = (TO)in[i];
 }
 
-// coarsest solves, one block per problem
+// coarsest solves, grid (row blocks of the largest, problems)
 template <typename T>
-__global__ void coarse_solve_batch_kernel(const XferTask* __restrict__ tasks) {
+__global__ void __launch_bounds__(32 * kCoarseWarps) coarse_solve_batch_kernel(const XferTask* __restrict__ tasks) {
   grid_dep_entry();
   extern __shared__ double sm[];
-  const XferTask tk = tasks[blockIdx.x];
+  const XferTask tk = tasks[blockIdx.y];
   if (skip(tk.sc)) return;
-  coarse_solve_block<T>(tk.nf, tk.m1, tk.m2, static_cast<const T*>(tk.src), static_cast<T*>(tk.dst), sm);
+  const int ni = tk.nf - 1, nb = (3 * ni * ni * ni + kCoarseWarps - 1) / kCoarseWarps;
+  if ((int)blockIdx.x >= nb) return;
+  coarse_solve_rows<T>(tk.nf, tk.m1, static_cast<const T*>(tk.src), static_cast<T*>(tk.dst), sm, blockIdx.x, nb);
 }
 
 // ------------------------------------------------------------------ Krylov
@@ -216,7 +218,8 @@ cudaError_t launch_xfer_batch(int kind, const XferTask* tasks, int ntasks, int64
       KL(launch_k(convert_batch_kernel<float, double>, gc, dim3(kBT), 0, s, tasks));
       break;
     case XK_COARSE:
-      KL(launch_k(coarse_solve_batch_kernel<T>, dim3(ntasks), dim3(1024), 2 * (size_t)max_m * sizeof(double), s, tasks));
+      KL(launch_k(coarse_solve_batch_kernel<T>, dim3(chunks(max_m, kCoarseWarps), (unsigned)ntasks),
+                  dim3(32 * kCoarseWarps), (size_t)max_m * sizeof(double), s, tasks));
       break;
     default: return cudaErrorInvalidValue;
   }

@@ -83,7 +83,7 @@ struct agca_ctx {
   size_t gs_bytes = 0, gs_need = 0;
   // coarsest
   int mc = 0;
-  double *cdense = nullptr, *cfac = nullptr, *linv_cm = nullptr, *linv_rm = nullptr;
+  double *cdense = nullptr, *cfac = nullptr, *ainv = nullptr, *linv = nullptr;
   // pressure
   int64_t Vp = 0;
   double *pmass = nullptr, *pmass_inv = nullptr, *qfine = nullptr, *sfine = nullptr;
@@ -221,8 +221,8 @@ void carve_workspace(agca_ctx* ctx, char* base) {
   const int64_t m2 = (int64_t)ctx->mc * ctx->mc;
   ctx->cdense = cv.take<double>(m2);
   ctx->cfac = cv.take<double>(m2);
-  ctx->linv_cm = cv.take<double>(m2);
-  ctx->linv_rm = cv.take<double>(m2);
+  ctx->ainv = cv.take<double>(m2);
+  ctx->linv = cv.take<double>(m2);
   ctx->pmass = cv.take<double>(ctx->Vp);
   ctx->pmass_inv = cv.take<double>(ctx->Vp);
   ctx->qfine = cv.take<double>(ctx->lev[ctx->L].V);
@@ -432,7 +432,7 @@ agca_status chebyshev(agca_ctx* ctx, int l, const T* b, bool from_zero, T** cur,
 template <typename T>
 agca_status cycle(agca_ctx* ctx, int l, const T* b, T* X, T* Tb, T** res, double* final64 = nullptr) {
   if (l == 1) {
-    LK(1, launch_coarse_solve<T>(ctx->lev[1].n, ctx->linv_cm, ctx->linv_rm, b, X, ctx->stream));
+    LK(1, launch_coarse_solve<T>(ctx->lev[1].n, ctx->ainv, b, X, ctx->stream));
     *res = X;
     return AGCA_OK;
   }
@@ -1074,7 +1074,7 @@ agca_status tune_level(agca_ctx* ctx, int l, int reps, std::map<std::string, Til
 // list, 2-D element-wise grids over (chunk, problem)), skipping converged
 // problems on the device.
 struct BatchStep {
-  int kind;        // 0 stencil, 1 xfer, 2 krylov
+  int kind;        // 0 stencil, 1 xfer, 2 krylov, 3 stencil on small levels (work = cubes per axis of the largest)
   int mode;        // stencil mode / xfer kind / krylov op
   int prec;        // 0: <double,double>, 1: <float,float>, 2: <double,float>
   bool coarse;
@@ -1159,6 +1159,18 @@ StencilTask<TS, T> make_task(agca_ctx* c, int l, int mode, const TS* x, const TS
 template <typename TS, typename T>
 void push_stencil(agca_batch* b, std::vector<BatchStep>& steps, int mode, bool coarse, std::vector<StencilTask<TS, T>> t,
                   int prec) {
+  if constexpr (std::is_same<TS, T>::value) {
+    if (mode != ST_STOKES) {  // small levels run the point kernel, as launch_stencil does
+      std::vector<StencilTask<TS, T>> small, large;
+      for (const auto& tk : t) (tk.op.n <= kPointMaxN ? small : large).push_back(tk);
+      if (!small.empty()) {
+        int64_t mx = 0;
+        for (const auto& tk : small) mx = std::max<int64_t>(mx, tk.op.n);
+        steps.push_back(BatchStep{3, mode, prec, coarse, push_tasks(b, small), (int)small.size(), mx, 0, 0});
+      }
+      t.swap(large);
+    }
+  }
   if (t.empty()) return;
   // one z-chunk for the whole step: about six waves of resident blocks over
   // all problems (the batch supplies the parallelism, so chunks stay long and
@@ -1265,8 +1277,7 @@ void build_cycle(agca_batch* b, std::vector<BatchStep>& steps, const std::vector
       x.count = 1;
       x.src = c->lev[1].vb;
       x.dst = c->lev[1].vx;
-      x.m1 = c->linv_cm;
-      x.m2 = c->linv_rm;
+      x.m1 = c->ainv;
       x.sc = sc_of(p);
       t.push_back(x);
     }
@@ -1439,6 +1450,14 @@ agca_status run_steps(agca_batch* b, const std::vector<BatchStep>& steps, int64_
         BCK(launch_stencil_batch<double, float>(st.mode, st.coarse, (const StencilTask<double, float>*)t, st.ntasks,
                                                 st.work, st.gca, s));
       *launches += (st.coarse && st.gca > 0) ? 2 : 1;
+    } else if (st.kind == 3) {
+      if (st.prec == 0)
+        BCK(launch_stencil_point_batch<double>(st.mode, (const StencilTask<double, double>*)t, st.ntasks, (int)st.work,
+                                               s));
+      else
+        BCK(launch_stencil_point_batch<float>(st.mode, (const StencilTask<float, float>*)t, st.ntasks, (int)st.work,
+                                              s));
+      *launches += 1;
     } else if (st.kind == 1) {
       if (st.prec == 1)
         BCK(launch_xfer_batch<float>(st.mode, (const XferTask*)t, st.ntasks, st.work, st.max_m, s));
@@ -1681,14 +1700,18 @@ agca_status agca_setup(agca_ctx* ctx) {
     if (mixed) {
       LK(1, launch_stencil_to_f32(lc.n_sv, lc.sten64, lc.sten32, lc.sscale32, s));
     } else {
-      LK(1, launch_masked_coef(lc.E, lc.mean, lc.fidx, lc.coefm, s));
+      LK(1, launch_masked_coef<double>(lc.E, lc.mean, lc.fidx, lc.coefm, s));
       LK(1, launch_edge_records(lc.n, lc.coefm, lc.hedge, s));
     }
   }
   for (int l = 1; l <= L; ++l) {
     Level& lv = ctx->lev[l];
     if (mixed) {
-      LK(1, launch_d2f(lv.mean, lv.mean32, lv.E, s));
+      // coarse levels: the flagged elements' part is in the stencils
+      if (l < L)
+        LK(1, launch_masked_coef<float>(lv.E, lv.mean, lv.fidx, lv.mean32, s));
+      else
+        LK(1, launch_d2f(lv.mean, lv.mean32, lv.E, s));
       if (l < L) LK(1, launch_gca_to_f32(lv.n_flag, lv.list, lv.mx, lv.gca64, lv.gca32, lv.gscale32, s));
     }
     LK(1, launch_diag(op64(ctx, l), lv.diag, lv.invD64, mixed ? lv.invD32 : nullptr, s));
@@ -1697,7 +1720,8 @@ agca_status agca_setup(agca_ctx* ctx) {
   LK(1, launch_coarse_assemble(op64(ctx, 1), ctx->cdense, s));
   CK(cudaMemcpyAsync(ctx->cfac, ctx->cdense, (size_t)ctx->mc * ctx->mc * sizeof(double), cudaMemcpyDeviceToDevice, s));
   LK(1, launch_cholesky(ctx->cfac, ctx->mc, ctx->status, s));
-  LK(1, launch_trinv(ctx->cfac, ctx->mc, ctx->linv_cm, ctx->linv_rm, s));
+  LK(1, launch_trinv(ctx->cfac, ctx->mc, ctx->ainv, ctx->linv, s));
+  LK(1, launch_coarse_inverse(ctx->linv, ctx->mc, ctx->ainv, s));
   CKS(check_status(ctx, "agca_setup"));
   for (int l = 2; l <= L; ++l) CKS(power_lambda(ctx, l, &ctx->lev[l].lambda));
   LK(1, launch_pressure_mass(ctx->lev[L].n / 2, ctx->lev[L].mean, ctx->pmass, ctx->pmass_inv, s));

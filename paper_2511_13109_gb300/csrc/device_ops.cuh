@@ -267,50 +267,41 @@ __device__ __forceinline__ T prolong_point(const int nf, const bool mask, const 
 }
 
 // ------------------------------------------------------------- coarsest solve
-// z = L^-T L^-1 r on the interior DoFs of the coarsest grid (n cubes), by one
-// thread block: one warp per row of each triangular product with coalesced
-// row reads (X row-major for t = X r, X column-major for z = X^T t); r, z are
-// full-grid vectors, sm holds 2 * 3 (n-1)^3 doubles.  Every row's sum is
-// formed by one warp in a fixed order, whatever the block size.
+// z = A_1^-1 r on the interior DoFs of the coarsest grid (n cubes) with the
+// explicit inverse ainv (m x m, m = 3 (n-1)^3, symmetric bit for bit): block
+// b of nb forms the rows b * 8 .. b * 8 + 7, one warp each, from a copy of r
+// in shared memory (sm: m doubles); r, z are full-grid vectors.  A row's sum is
+// formed by one warp in a fixed order, so the result depends on no grid shape.
+// One block doing both triangular products of L^-T L^-1 took 16 us at m = 81 and
+// 200 us for twelve problems of up to m = 648; the rows of the inverse are
+// independent, need half the passes and spread over the SMs.
+constexpr int kCoarseWarps = 8;
 template <typename T>
-__device__ __forceinline__ void coarse_solve_block(const int n, const double* __restrict__ xcm,
-                                                   const double* __restrict__ xrm, const T* r, T* z, double* sm) {
-  const int nv = n + 1, ni = n - 1;
-  const int64_t V = nverts(n);
+__device__ __forceinline__ void coarse_solve_rows(const int n, const double* __restrict__ ainv, const T* r, T* z,
+                                                  double* sm, const int b, const int nb) {
+  const int nv = n + 1, ni = n - 1, V = nv * nv * nv;
   const int nI = ni * ni * ni, m = 3 * nI;
-  double* rs = sm;
-  double* ts = sm + m;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int q = threadIdx.x; q < m; q += blockDim.x) {
-    const int c = q / nI, iv = q % nI;
-    const int i = 1 + iv % ni, j = 1 + (iv / ni) % ni, k = 1 + iv / (ni * ni);
-    rs[q] = (double)__ldg(r + c * V + i + (int64_t)nv * (j + (int64_t)nv * k));
+  auto grid_index = [&](int q) {
+    const int c = q / nI, iv = q - c * nI;
+    const int t = iv / ni, i = iv - t * ni, k = t / ni, j = t - k * ni;
+    return c * V + (1 + i) + nv * ((1 + j) + nv * (1 + k));
+  };
+  const int lane = threadIdx.x & 31, q = b * kCoarseWarps + (threadIdx.x >> 5);
+  for (int p = threadIdx.x; p < m; p += blockDim.x) sm[p] = (double)__ldg(r + grid_index(p));
+  // Dirichlet entries of z
+  for (int id = b * blockDim.x + threadIdx.x; id < 3 * V; id += nb * blockDim.x) {
+    const int v = id % V, t = v / nv, i = v - t * nv, k = t / nv, j = t - k * nv;
+    if (i == 0 || j == 0 || k == 0 || i == n || j == n || k == n) z[id] = T(0);
   }
   __syncthreads();
-  for (int q = warp; q < m; q += nw) {
-    double s = 0.0;
-    for (int p = lane; p <= q; p += 32) s = fma(xrm[(int64_t)q * m + p], rs[p], s);
+  if (q >= m) return;
+  const double* row = ainv + (int64_t)q * m;
+  double s = 0.0;
+#pragma unroll 4
+  for (int p = lane; p < m; p += 32) s = fma(row[p], sm[p], s);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-    if (lane == 0) ts[q] = s;
-  }
-  __syncthreads();
-  for (int q = warp; q < m; q += nw) {
-    double s = 0.0;
-    for (int p = q + lane; p < m; p += 32) s = fma(xcm[(int64_t)q * m + p], ts[p], s);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-    if (lane == 0) rs[q] = s;
-  }
-  __syncthreads();
-  for (int id = threadIdx.x; id < 3 * (int)V; id += blockDim.x) {
-    const int c = id / (int)V, v = id - c * (int)V;
-    const int t = v / nv, i = v - t * nv, k = t / nv, j = t - k * nv;
-    const bool inner = i > 0 && j > 0 && k > 0 && i < n && j < n && k < n;
-    T out = T(0);
-    if (inner) out = (T)rs[c * nI + (i - 1) + ni * ((j - 1) + ni * (k - 1))];
-    z[id] = out;
-  }
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if (lane == 0) z[grid_index(q)] = (T)s;
 }
 
 }  // namespace agca

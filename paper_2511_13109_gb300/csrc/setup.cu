@@ -384,6 +384,7 @@ __global__ void cholesky_kernel(double* a, int m, int* status) {
 }
 
 // X = L^-1 (lower), one thread per column; writes column- and row-major copies
+// (the column-major one is scratch: the inverse takes its place)
 __global__ void trinv_kernel(const double* l, int m, double* xcm, double* xrm) {
   grid_dep_entry();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -401,13 +402,24 @@ __global__ void trinv_kernel(const double* l, int m, double* xcm, double* xrm) {
   }
 }
 
-// z = L^-T L^-1 r on the interior DoFs of level 1, one block; r, z full-grid.
+// ainv = X^T X for X = L^-1 row-major (lower): entry (i, j) and entry (j, i)
+// add the same products in the same order
+__global__ void coarse_inverse_kernel(const double* __restrict__ x, int m, double* __restrict__ ainv) {
+  grid_dep_entry();
+  const int j = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+  if (j >= m) return;
+  double s = 0.0;
+  for (int k = max(i, j); k < m; ++k) s = fma(x[(int64_t)k * m + i], x[(int64_t)k * m + j], s);
+  ainv[(int64_t)i * m + j] = s;
+}
+
+// z = A_1^-1 r on the interior DoFs of level 1; r, z full-grid.
 template <typename T>
-__global__ void coarse_solve_kernel(int n, const double* __restrict__ xcm, const double* __restrict__ xrm,
-                                    const T* __restrict__ r, T* __restrict__ z) {
+__global__ void __launch_bounds__(32 * kCoarseWarps)
+    coarse_solve_kernel(int n, const double* __restrict__ ainv, const T* __restrict__ r, T* __restrict__ z) {
   grid_dep_entry();
   extern __shared__ double sm[];
-  coarse_solve_block<T>(n, xcm, xrm, r, z, sm);
+  coarse_solve_rows<T>(n, ainv, r, z, sm, blockIdx.x, gridDim.x);
 }
 
 __global__ void pressure_mass_kernel(const RefineTables rt, int np, const double* __restrict__ eta_f, double* pmass, double* pmass_inv) {
@@ -543,17 +555,20 @@ cudaError_t launch_trinv(const double* l, int m, double* linv_cm, double* linv_r
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_coarse_solve(int n, const double* linv_cm, const double* linv_rm, const T* r, T* z,
-                                cudaStream_t s) {
-  const int ni = n - 1, m = 3 * ni * ni * ni;
-  const size_t smem = 2 * (size_t)m * sizeof(double);
-  KL(launch_k(coarse_solve_kernel<T>, dim3(1), dim3(1024), smem, s, n, linv_cm, linv_rm, r, z));
+cudaError_t launch_coarse_inverse(const double* linv_rm, int m, double* ainv, cudaStream_t s) {
+  KL(launch_k(coarse_inverse_kernel, dim3(blocks_for(m, 128), (unsigned)m), dim3(128), 0, s, linv_rm, m, ainv));
   return cudaGetLastError();
 }
-template cudaError_t launch_coarse_solve<float>(int, const double*, const double*, const float*, float*, cudaStream_t);
-template cudaError_t launch_coarse_solve<double>(int, const double*, const double*, const double*, double*,
-                                                 cudaStream_t);
+
+template <typename T>
+cudaError_t launch_coarse_solve(int n, const double* ainv, const T* r, T* z, cudaStream_t s) {
+  const int ni = n - 1, m = 3 * ni * ni * ni;
+  KL(launch_k(coarse_solve_kernel<T>, dim3(blocks_for(m, kCoarseWarps)), dim3(32 * kCoarseWarps),
+              (size_t)m * sizeof(double), s, n, ainv, r, z));
+  return cudaGetLastError();
+}
+template cudaError_t launch_coarse_solve<float>(int, const double*, const float*, float*, cudaStream_t);
+template cudaError_t launch_coarse_solve<double>(int, const double*, const double*, double*, cudaStream_t);
 
 cudaError_t launch_pressure_mass(int np, const double* eta_f, double* pmass, double* pmass_inv, cudaStream_t s) {
   const int64_t V = nverts(np);

@@ -725,6 +725,10 @@ template <typename TS, typename T>
 cudaError_t launch_stencil(int mode, const LevelOp<T>& op, const StencilArgs<TS>& a, cudaStream_t s,
                            const TileCfg* cfg) {
   const int by = cfg ? cfg->by : 8, zch = cfg ? cfg->zch : 0;
+  if constexpr (std::is_same<TS, T>::value) {
+    if (op.n <= kPointMaxN && mode != ST_STOKES && mode != ST_STOKES_B)
+      return launch_stencil_point<T>(mode, op, a, s);
+  }
   if constexpr (std::is_same<TS, double>::value && std::is_same<T, double>::value) {
     // FP64 levels run the edge form (their coefficient records exist in FP64 contexts)
     if (op.hedge && mode != ST_STOKES && mode != ST_STOKES_B) return launch_stencil_edge<T>(mode, op, a, s, zch);

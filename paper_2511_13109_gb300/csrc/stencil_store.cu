@@ -104,12 +104,13 @@ __global__ void stencil_to_f32_kernel(const int64_t n_sv, const double* __restri
 }
 
 // DCA coefficient with the flagged elements zeroed (their part is in the stencils)
+template <typename T>
 __global__ void masked_coef_kernel(const int64_t E, const double* __restrict__ mean, const int32_t* __restrict__ fidx,
-                                   double* __restrict__ coefm) {
+                                   T* __restrict__ coefm) {
   grid_dep_entry();
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= E) return;
-  coefm[e] = fidx[e] >= 0 ? 0.0 : mean[e];
+  coefm[e] = fidx[e] >= 0 ? T(0) : (T)mean[e];
 }
 
 unsigned nblocks(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
@@ -136,9 +137,13 @@ cudaError_t launch_stencil_to_f32(int64_t n_sv, const double* s64, float* s32, f
   return cudaGetLastError();
 }
 
-cudaError_t launch_masked_coef(int64_t E, const double* mean, const int32_t* fidx, double* coefm, cudaStream_t s) {
-  KL(launch_k(masked_coef_kernel, dim3(nblocks(E, 256)), dim3(256), 0, s, E, mean, fidx, coefm));
+template <typename T>
+cudaError_t launch_masked_coef(int64_t E, const double* mean, const int32_t* fidx, T* coefm, cudaStream_t s) {
+  KL(launch_k(masked_coef_kernel<T>, dim3(nblocks(E, 256)), dim3(256), 0, s, E, mean, fidx, coefm));
   return cudaGetLastError();
 }
+
+template cudaError_t launch_masked_coef<double>(int64_t, const double*, const int32_t*, double*, cudaStream_t);
+template cudaError_t launch_masked_coef<float>(int64_t, const double*, const int32_t*, float*, cudaStream_t);
 
 }  // namespace agca

@@ -1,0 +1,64 @@
+"""The eight-lanes-per-vertex kernel of the small levels and the coarsest solve
+by the explicit inverse, at the edges of their ranges: grids of 2 to 5 cubes
+per axis, odd sizes, and the largest size (32 cubes) and the first tiled ones
+against the other precision on the same grid.  Tolerances as in test_gpu_parity.py: 1e-12 (FP64) and
+1e-5 (FP32) of the largest entry for an apply, 1e-9 and 1e-4 for a cycle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import agca as oagca
+from synth import random_vector
+
+pytestmark = pytest.mark.gpu
+
+pkg = pytest.importorskip("paper_2511_13109_gb300")
+DEV = torch.device("cuda:0")
+
+
+def _eta(N, seed):
+    m = 6 * (2 * N) ** 3
+    return np.exp(np.random.default_rng(seed).uniform(-2, 2, m) * np.log(10.0))
+
+
+# (N, levels): finest / coarsest cubes per axis 4/2, 10/5, 12/3, 18/9 (1,536 coarsest unknowns)
+@pytest.mark.parametrize("N,L", [(2, 2), (5, 2), (6, 3), (9, 2)])
+@pytest.mark.parametrize("nu", [10.0, 1e9])  # nearly all elements flagged, none
+def test_small_levels_match_oracle(N, L, nu):
+    eta = _eta(N, N)
+    H = oagca.Hierarchy(N, L, eta, nu)
+    c64 = pkg.Context(N, L, pkg.FP64, device=DEV)
+    c32 = pkg.Context(N, L, pkg.MIXED, device=DEV)
+    for c in (c64, c32):
+        c.prepare(torch.from_numpy(eta).to(DEV), nu)
+    for l in range(1, L + 1):
+        x = random_vector(3 * c64.V[l], 40 + l)  # boundary entries are not zero: they are ignored
+        ref = H.A[l] @ (x * H.mask[l])
+        big = np.abs(ref).max()
+        xd = torch.from_numpy(x).to(DEV)
+        for c in (c64, c32):  # FP64 with coefficient records, and from the element coefficients
+            assert np.abs(c.apply(l, xd).cpu().numpy() - ref).max() <= 1e-12 * big, l
+        x32 = x.astype(np.float32)
+        ref = H.A[l] @ (x32.astype(np.float64) * H.mask[l])
+        got = c32.apply(l, torch.from_numpy(x32).to(DEV), dtype=pkg.F32).cpu().numpy()
+        assert np.abs(got - ref).max() <= 1e-5 * np.abs(ref).max(), l
+    r = random_vector(3 * c64.V[L], 50)
+    ref = H.vcycle(r * H.mask[L])
+    for c, tol in ((c64, 1e-9), (c32, 1e-4)):
+        z = c.vcycle(torch.from_numpy(r).to(DEV)).cpu().numpy()
+        assert np.abs(z - ref).max() <= tol * np.abs(ref).max()
+        assert np.abs(z * (1 - H.mask[L])).max() == 0.0
+
+
+@pytest.mark.parametrize("N", [16, 18, 24])  # 32 cubes per axis: the last point level; 36 and 48: tiles over point levels
+def test_point_kernel_meets_tile_kernel(N):
+    eta = torch.from_numpy(_eta(N, N)).to(DEV)
+    c64, c32 = (pkg.Context(N, None, p, device=DEV) for p in (pkg.FP64, pkg.MIXED))
+    c64.prepare(eta, 10.0)
+    c32.prepare(eta, 10.0)
+    for l in (c64.L, c64.L - 1):
+        x = torch.from_numpy(random_vector(3 * c64.V[l], l).astype(np.float32)).to(DEV)
+        ref = c64.apply(l, x.double())
+        big = float(ref.abs().max())
+        assert float((c32.apply(l, x.double()) - ref).abs().max()) <= 1e-12 * big
+        assert float((c32.apply(l, x, dtype=pkg.F32).double() - ref).abs().max()) <= 1e-5 * big
