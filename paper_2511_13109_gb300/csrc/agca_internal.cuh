@@ -103,12 +103,14 @@ struct LevelOp {
   const T* gscale;     // per flagged element scale (mixed) or nullptr
   const int32_t* list; // flagged element ids (coarse levels)
   int64_t n_flag;      // number of flagged elements
-  T* ye;               // n_flag * 12 scratch: s_e A_e x_e of the flagged elements
+  T* ye;               // n_flag * 12 scratch: the stored-Galerkin part at the touched vertices (launch_gather)
   const T* hedge;      // FP64 levels: per-vertex coefficient records [EREC][V] of the edge form, or nullptr
   const T* coefm;      // FP64 coarse levels: DCA coefficient with flagged elements zeroed (edge form), or nullptr
   // stored-Galerkin part as per-vertex stencils (Remark 5): stencil index of a
   // vertex or -1, 15 x 3 x 3 couplings per touched vertex, FP32 scale (mixed)
   const int32_t* sidx;
+  const int32_t* slist;  // touched vertices, ascending
+  int64_t n_sv;          // number of them
   const T* sten;
   const T* sscale;
 };
@@ -157,6 +159,9 @@ cudaError_t launch_k(void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, 
   } while (0)
 
 // ---------------------------------------------------------------- launchers
+// ST_CHEB_PRE, the Chebyshev step from x0 = 0: the small levels form the first
+// iterate x1 = (s2 D^-1) b on the fly; the tile kernels find it in a.x, written
+// by the kernel that wrote b (launch_restrict, launch_d2f) or by launch_x1
 enum StencilMode { ST_APPLY = 0, ST_RESID = 1, ST_CHEB_FIRST = 2, ST_CHEB_STEP = 3, ST_CHEB_PRE = 4, ST_STOKES = 5 };
 // internal (FP64 contexts, not tunable): the pressure coupling of the Stokes
 // operator added to a.b = A u from the edge form, out = a.b - B_f^T q,
@@ -211,11 +216,22 @@ cudaError_t launch_edge_records(int n, const T* eta, T* rec, cudaStream_t s);
 template <typename T>
 cudaError_t launch_stencil_edge(int mode, const LevelOp<T>& op, const StencilArgs<T>& a, cudaStream_t s, int zch_req);
 
+// FP32 levels of more than kPointMaxN cubes per axis (stencil_f32.cu): modes
+// APPLY, RESID and the Chebyshev steps; tile grid with per_z() * gz tiles
+TileGrid f32_tiles(int n, int zch_req, int slots = 0);
+cudaError_t launch_stencil_f32(int mode, const LevelOp<float>& op, const StencilArgs<float>& a, cudaStream_t s,
+                               int zch_req);
+
 // Small levels (stencil_point.cu): eight lanes per vertex, on grids of up to
 // kPointMaxN cubes per axis (the reasons for the limit stand there)
 constexpr int kPointMaxN = 32;
 template <typename T>
 cudaError_t launch_stencil_point(int mode, const LevelOp<T>& op, const StencilArgs<T>& a, cudaStream_t s);
+
+// stored-Galerkin part of a coarse level for the tile kernels: op.ye <- sum_o
+// S[o] x(v + o) at the touched vertices (x: the operator input)
+template <typename T>
+cudaError_t launch_gather(const LevelOp<T>& op, const T* x, cudaStream_t s);
 
 // ------------------------------------------------------------ batched forms
 // One (problem, level) operator application inside a batched launch.
@@ -227,12 +243,10 @@ struct StencilTask {
   int64_t tile0;        // first tile of this task in the flattened work list
   const double* sc;     // MINRES scalars of the problem (skip when sc[MS_DONE] != 0) or nullptr
 };
-// tasks: device array, ntiles = total tiles of all tasks; coarse launches
-// first run the stored-Galerkin products of every task (max_gca_rows = the
-// largest n_flag * 12)
+// tasks: device array, ntiles = total tiles of all tasks (FP64 vectors)
 template <typename TS, typename T>
 cudaError_t launch_stencil_batch(int mode, bool coarse, const StencilTask<TS, T>* tasks, int ntasks, int64_t ntiles,
-                                 int64_t max_gca_rows, cudaStream_t s);
+                                 cudaStream_t s);
 // the edge form for a batch of tasks (tiles from edge_tiles)
 template <typename T>
 cudaError_t launch_stencil_edge_batch(int mode, const StencilTask<T, T>* tasks, int ntasks, int64_t ntiles,
@@ -241,6 +255,12 @@ cudaError_t launch_stencil_edge_batch(int mode, const StencilTask<T, T>* tasks, 
 template <typename T>
 cudaError_t launch_stencil_point_batch(int mode, const StencilTask<T, T>* tasks, int ntasks, int max_n,
                                        cudaStream_t s);
+// stored-Galerkin parts of a batch of tile steps (max_sv: the largest n_sv)
+template <typename T>
+cudaError_t launch_gather_batch(const StencilTask<T, T>* tasks, int ntasks, int64_t max_sv, cudaStream_t s);
+// FP32 tiles of a batch (from f32_tiles); sten: every task has stored-Galerkin stencils, or none has
+cudaError_t launch_stencil_f32_batch(int mode, bool sten, const StencilTask<float, float>* tasks, int ntasks,
+                                     int64_t ntiles, cudaStream_t s);
 // whether a step of this kind runs the edge form: every level of an FP64
 // context (its coefficient records exist on every level); the FP32 cycle and
 // the Stokes operator run the per-cube kernel
@@ -260,16 +280,29 @@ struct XferTask {
   const void* src;
   void* dst;
   const double* m1;     // coarsest solve: inverse of the coarsest matrix
+  const void* invD;     // restriction, XK_D2F, XK_X1: first Chebyshev iterate x1 = (s2 D^-1) b
+  void* x1;             // beside the right-hand side written (nullptr: none)
+  double s2;
   const double* sc;     // skip when sc[MS_DONE] != 0, or nullptr
 };
-enum XferKind { XK_RESTRICT = 0, XK_PROLONG_ADD, XK_D2F, XK_F2D, XK_COARSE, XK_PROLONG, XK_COPY64 };
+enum XferKind { XK_RESTRICT = 0, XK_PROLONG_ADD, XK_D2F, XK_F2D, XK_COARSE, XK_PROLONG, XK_COPY64, XK_X1 };
 template <typename T>
 cudaError_t launch_xfer_batch(int kind, const XferTask* tasks, int ntasks, int64_t max_count, int max_m,
                               cudaStream_t s);
 
 // grid transfers (transfer.cu)
+// the first Chebyshev iterate x1 = (s2 D^-1) b, written beside a right-hand side b
 template <typename T>
-cudaError_t launch_restrict(int nf, int ncomp, bool mask, T scale, const T* rf, T* rc, cudaStream_t s);
+struct FirstIterate {
+  const T* invD = nullptr;
+  T* x1 = nullptr;  // nullptr: none
+  T s2 = T(0);
+};
+template <typename T>
+cudaError_t launch_restrict(int nf, int ncomp, bool mask, T scale, const T* rf, T* rc, cudaStream_t s,
+                            const FirstIterate<T>& fi = {});
+// x1 from a right-hand side in place; n = 3 V entries (D^-1 is 0 on Dirichlet entries, where b is ignored)
+cudaError_t launch_x1(const double* b, const FirstIterate<double>& fi, int64_t n, cudaStream_t s);
 template <typename T>
 cudaError_t launch_prolong(int nf, int ncomp, bool mask, bool add, const T* ec, T* xf, cudaStream_t s);
 
@@ -292,7 +325,7 @@ cudaError_t launch_galerkin(int nc, int64_t n_flag, const int32_t* list, int nf,
 cudaError_t launch_diag(const LevelOp<double>& op, double* diag, double* invD64, float* invD32, cudaStream_t s);
 cudaError_t launch_gca_to_f32(int64_t n_flag, const int32_t* list, const double* mx, const double* gca64,
                               float* gca32, float* scale32, cudaStream_t s);
-cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s);
+cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s, const FirstIterate<float>& fi = {});
 cudaError_t launch_f2d(const float* in, double* out, int64_t n, cudaStream_t s);
 cudaError_t launch_coarse_assemble(const LevelOp<double>& op, double* dense, cudaStream_t s);
 cudaError_t launch_cholesky(double* a, int m, int* status, cudaStream_t s);

@@ -31,8 +31,12 @@ __global__ void restrict_batch_kernel(const XferTask* __restrict__ tasks) {
   const T* rf = static_cast<const T*>(tk.src);
   T* rc = static_cast<T*>(tk.dst);
   const int t = id / nvc, I = id - t * nvc, K = t / nvc, J = t - K * nvc;
-  for (int c = 0; c < tk.ncomp; ++c)
-    rc[c * Vc + id] = restrict_point<T>(nf, tk.mask, (T)tk.scale, rf + c * Vf, I, J, K);
+  T* x1 = static_cast<T*>(tk.x1);
+  for (int c = 0; c < tk.ncomp; ++c) {
+    const T v = restrict_point<T>(nf, tk.mask, (T)tk.scale, rf + c * Vf, I, J, K);
+    rc[c * Vc + id] = v;
+    if (x1) x1[c * Vc + id] = (T)tk.s2 * __ldg(static_cast<const T*>(tk.invD) + c * Vc + id) * v;
+  }
 }
 
 template <typename T, bool ADD>
@@ -65,6 +69,24 @@ __global__ void convert_batch_kernel(const XferTask* __restrict__ tasks) {
   TO* out = static_cast<TO*>(tk.dst);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tk.count; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = (TO)in[i];
+}
+
+// FP32 right-hand sides (XK_D2F) or the FP64 ones in place (XK_X1, WRITE false), with the first Chebyshev iterate
+template <typename TO, bool WRITE>
+__global__ void rhs_batch_kernel(const XferTask* __restrict__ tasks) {
+  grid_dep_entry();
+  const XferTask tk = tasks[blockIdx.y];
+  if (skip(tk.sc)) return;
+  const double* in = static_cast<const double*>(tk.src);
+  TO* out = static_cast<TO*>(tk.dst);
+  TO* x1 = static_cast<TO*>(tk.x1);
+  const TO* invD = static_cast<const TO*>(tk.invD);
+  const TO s2 = (TO)tk.s2;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tk.count; i += (int64_t)gridDim.x * blockDim.x) {
+    const TO v = (TO)in[i];
+    if (WRITE) out[i] = v;
+    if (x1) x1[i] = s2 * __ldg(invD + i) * v;
+  }
 }
 
 // coarsest solves, grid (row blocks of the largest, problems)
@@ -212,7 +234,10 @@ cudaError_t launch_xfer_batch(int kind, const XferTask* tasks, int ntasks, int64
       KL(launch_k(convert_batch_kernel<double, double>, gc, dim3(kBT), 0, s, tasks));
       break;
     case XK_D2F:
-      KL(launch_k(convert_batch_kernel<double, float>, gc, dim3(kBT), 0, s, tasks));
+      KL(launch_k(rhs_batch_kernel<float, true>, gc, dim3(kBT), 0, s, tasks));
+      break;
+    case XK_X1:
+      KL(launch_k(rhs_batch_kernel<double, false>, gc, dim3(kBT), 0, s, tasks));
       break;
     case XK_F2D:
       KL(launch_k(convert_batch_kernel<float, double>, gc, dim3(kBT), 0, s, tasks));

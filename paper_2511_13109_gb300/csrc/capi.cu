@@ -261,6 +261,8 @@ LevelOp<double> op64(const agca_ctx* ctx, int l) {
   if (l < ctx->L) {
     op.coefm = lv.coefm;
     op.sidx = lv.sidx;
+    op.slist = lv.slist;
+    op.n_sv = lv.n_sv;
     op.sten = lv.n_sv > 0 ? lv.sten64 : nullptr;
     op.fidx = lv.fidx;
     op.gca = lv.gca64;
@@ -280,6 +282,8 @@ LevelOp<float> op32(const agca_ctx* ctx, int l) {
   op.coef = lv.mean32;
   if (l < ctx->L) {
     op.sidx = lv.sidx;
+    op.slist = lv.slist;
+    op.n_sv = lv.n_sv;
     op.sten = lv.n_sv > 0 ? lv.sten32 : nullptr;
     op.sscale = lv.n_sv > 0 ? lv.sscale32 : nullptr;
     op.fidx = lv.fidx;
@@ -381,7 +385,8 @@ agca_status stencil(agca_ctx* ctx, int mode, int l, const T* x, const T* b, cons
   const bool timed = ctx->prof && l == ctx->L && ctx->ev_used + 2 <= ctx->ev.size();
   if (timed) CK(cudaEventRecord(ctx->ev[ctx->ev_used], ctx->stream));
   const TileCfg* cfg = (mode >= 0 && mode < 6) ? &ctx->tune[l][mode] : nullptr;
-  LK((l < ctx->L && lv.n_flag > 0) ? 2 : 1, launch_stencil<T, T>(mode, level_op<T>(ctx, l), a, ctx->stream, cfg));
+  if (lv.n > kPointMaxN && l < ctx->L && lv.n_sv > 0) LK(1, launch_gather<T>(level_op<T>(ctx, l), x, ctx->stream));
+  LK(1, launch_stencil<T, T>(mode, level_op<T>(ctx, l), a, ctx->stream, cfg));
   if (timed) {
     CK(cudaEventRecord(ctx->ev[ctx->ev_used + 1], ctx->stream));
     ctx->ev_used += 2;
@@ -394,8 +399,22 @@ agca_status stencil(agca_ctx* ctx, int mode, int l, const T* x, const T* b, cons
   return AGCA_OK;
 }
 
+// The levels of tile kernels take the first iterate of a Chebyshev step from
+// zero as a vector (see ST_CHEB_PRE): x1 (the level's second iterate buffer)
+// for the right-hand side written there, or none.
+template <typename T>
+FirstIterate<T> first_iterate(const agca_ctx* ctx, int l, T* x1) {
+  FirstIterate<T> fi;
+  if (ctx->cheb_degree != 2 || l < 2 || ctx->lev[l].n <= kPointMaxN) return fi;
+  fi.invD = invD_of<T>(ctx->lev[l]);
+  fi.x1 = x1;
+  fi.s2 = (T)(1.0 / cheb_params(ctx, l).theta);
+  return fi;
+}
+
 // Chebyshev smoothing of A_l x = b (Section 4).  from_zero: start at x = 0
-// (the result of the first step is staged on the fly); otherwise start at
+// (degree 2: the first iterate is in *other on the levels of tile kernels and
+// formed on the fly on the small ones); otherwise start at
 // *cur.  cur/other are the two iterate buffers; returns the result buffer.
 // final64: if set, the last step writes its result there, widened to FP64,
 // instead of to the iterate buffers (the end of a mixed-precision cycle).
@@ -408,7 +427,7 @@ agca_status chebyshev(agca_ctx* ctx, int l, const T* b, bool from_zero, T** cur,
   int step = 1;
   if (from_zero && k == 2) {
     const double rn = 1.0 / (2.0 * c.sigma - rho);
-    CKS(stencil<T>(ctx, ST_CHEB_PRE, l, nullptr, b, nullptr, *cur, rn * rho, 2.0 * rn / c.delta, 1.0 / c.theta));
+    CKS(stencil<T>(ctx, ST_CHEB_PRE, l, *other, b, nullptr, *cur, rn * rho, 2.0 * rn / c.delta, 1.0 / c.theta));
     return AGCA_OK;
   }
   if (from_zero) CK(cudaMemsetAsync(*cur, 0, 3 * ctx->lev[l].V * sizeof(T), ctx->stream));
@@ -444,7 +463,8 @@ agca_status cycle(agca_ctx* ctx, int l, const T* b, T* X, T* Tb, T** res, double
   T* r = static_cast<T*>(lv.vr);
   CKS(stencil<T>(ctx, ST_RESID, l, cur, b, nullptr, r, 0, 0, 0));
   T* bc = static_cast<T*>(lc.vb);
-  LK(1, launch_restrict<T>(lv.n, 3, true, T(1), r, bc, ctx->stream));
+  LK(1, launch_restrict<T>(lv.n, 3, true, T(1), r, bc, ctx->stream,
+                           first_iterate<T>(ctx, l - 1, static_cast<T*>(lc.vt))));
   T* ec = nullptr;
   CKS(cycle<T>(ctx, l - 1, bc, static_cast<T*>(lc.vx), static_cast<T*>(lc.vt), &ec));
   LK(1, launch_prolong<T>(lv.n, 3, true, true, ec, cur, ctx->stream));
@@ -459,11 +479,13 @@ agca_status vcycle_direct(agca_ctx* ctx, const double* r, double* z) {
   const int64_t n3 = 3 * lf.V;
   if (ctx->prec == AGCA_FP64) {
     double* res = nullptr;
+    const auto fi = first_iterate<double>(ctx, L, static_cast<double*>(lf.vt));
+    if (fi.x1) LK(1, launch_x1(r, fi, n3, ctx->stream));
     CKS(cycle<double>(ctx, L, r, z, static_cast<double*>(lf.vt), &res));
     if (res != z) CK(cudaMemcpyAsync(z, res, n3 * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
   } else {
     float* b32 = static_cast<float*>(lf.vb);
-    LK(1, launch_d2f(r, b32, n3, ctx->stream));
+    LK(1, launch_d2f(r, b32, n3, ctx->stream, first_iterate<float>(ctx, L, static_cast<float*>(lf.vt))));
     float* res = nullptr;
     CKS(cycle<float>(ctx, L, b32, static_cast<float*>(lf.vx), static_cast<float*>(lf.vt), &res, z));
   }
@@ -983,7 +1005,8 @@ agca_status tune_level(agca_ctx* ctx, int l, int reps, std::map<std::string, Til
   const bool f32 = sizeof(T) == 4;
   // the edge form (every FP64 level) has one tile shape
   const bool edge = !f32;
-  std::vector<int> bys = edge ? std::vector<int>{8} : std::vector<int>{8, 12, 16};
+  const std::vector<int> bys = {8};  // the tile kernels have one tile shape; the small levels no tiles
+  auto tiles = [&](int zr, int slots) { return edge ? edge_tiles(lv.n, zr, slots) : f32_tiles(lv.n, zr, slots); };
   const int nv = lv.n + 1;
   int dev = 0, sms = 152;
   CK(cudaGetDevice(&dev));
@@ -993,10 +1016,10 @@ agca_status tune_level(agca_ctx* ctx, int l, int reps, std::map<std::string, Til
   // partly filled last wave)
   auto candidates = [&](int by) {
     std::vector<int> zs = {0, 1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
-    const int per_sm = edge ? 2 : (by <= 8 ? 3 : (by <= 12 ? 2 : 1));
-    const int per_z = edge ? edge_tiles(lv.n, 1).per_z() : stencil_tiles(lv.n, by, 1).per_z();
+    (void)by;
+    const int per_z = tiles(1, 0).per_z();
     for (int k = 1; k <= 16; ++k) {
-      const int gz = std::max(1, k * sms * per_sm / per_z);
+      const int gz = std::max(1, 2 * k * sms / per_z);
       zs.push_back((nv + gz - 1) / gz);
     }
     std::sort(zs.begin() + 1, zs.end());
@@ -1022,7 +1045,7 @@ agca_status tune_level(agca_ctx* ctx, int l, int reps, std::map<std::string, Til
       int last_zch = -1;
       for (int zr : candidates(by)) {
         if (zr > nv) continue;
-        const int zch = edge ? edge_tiles(lv.n, zr, 2 * sms).zch : stencil_tiles(lv.n, by, zr).zch;
+        const int zch = tiles(zr, 2 * sms).zch;
         if (zch == last_zch) continue;
         last_zch = zch;
         TileCfg c;
@@ -1035,7 +1058,7 @@ agca_status tune_level(agca_ctx* ctx, int l, int reps, std::map<std::string, Til
         T* R = static_cast<T*>(lv.vr);
         auto once = [&]() -> agca_status {
           switch (mode) {
-            case ST_CHEB_PRE: return stencil<T>(ctx, mode, l, nullptr, Bv, nullptr, X, 0.5, 0.5, 0.5);
+            case ST_CHEB_PRE: return stencil<T>(ctx, mode, l, Tb, Bv, nullptr, X, 0.5, 0.5, 0.5);
             case ST_RESID: return stencil<T>(ctx, mode, l, X, Bv, nullptr, R, 0, 0, 0);
             case ST_CHEB_FIRST: return stencil<T>(ctx, mode, l, X, Bv, nullptr, Tb, 0.5, 0, 0);
             default: return stencil<T>(ctx, mode, l, Tb, Bv, X, X, 0.5, 0.5, 0);
@@ -1074,14 +1097,16 @@ agca_status tune_level(agca_ctx* ctx, int l, int reps, std::map<std::string, Til
 // list, 2-D element-wise grids over (chunk, problem)), skipping converged
 // problems on the device.
 struct BatchStep {
-  int kind;        // 0 stencil, 1 xfer, 2 krylov, 3 stencil on small levels (work = cubes per axis of the largest)
+  // 0 stencil, 1 xfer, 2 krylov, 3 stencil on small levels (work = cubes per
+  // axis of the largest), 4 FP32 tiles (coarse: every task has stored-Galerkin
+  // stencils), 5 stored-Galerkin parts of the next step's tasks (work = most touched vertices)
+  int kind;
   int mode;        // stencil mode / xfer kind / krylov op
-  int prec;        // 0: <double,double>, 1: <float,float>, 2: <double,float>
+  int prec;        // 0: FP64, 1: FP32, 2: FP64 vectors with FP32 arithmetic
   bool coarse;
   size_t off;      // byte offset of the task array in the task table
   int ntasks;
   int64_t work;    // tiles (stencil), max count (xfer), max n (krylov)
-  int64_t gca;     // max gca rows (coarse stencil)
   int max_m;       // coarsest solve size
 };
 
@@ -1156,6 +1181,14 @@ StencilTask<TS, T> make_task(agca_ctx* c, int l, int mode, const TS* x, const TS
   return tk;
 }
 
+// the stored-Galerkin parts of tile steps whose task table is at off
+template <typename T>
+void push_gather(std::vector<BatchStep>& steps, const std::vector<StencilTask<T, T>>& t, size_t off, int prec) {
+  int64_t mx = 0;
+  for (const auto& tk : t) mx = std::max(mx, tk.op.sten ? tk.op.n_sv : 0);
+  if (mx > 0) steps.push_back(BatchStep{5, 0, prec, true, off, (int)t.size(), mx, 0});
+}
+
 template <typename TS, typename T>
 void push_stencil(agca_batch* b, std::vector<BatchStep>& steps, int mode, bool coarse, std::vector<StencilTask<TS, T>> t,
                   int prec) {
@@ -1166,10 +1199,45 @@ void push_stencil(agca_batch* b, std::vector<BatchStep>& steps, int mode, bool c
       if (!small.empty()) {
         int64_t mx = 0;
         for (const auto& tk : small) mx = std::max<int64_t>(mx, tk.op.n);
-        steps.push_back(BatchStep{3, mode, prec, coarse, push_tasks(b, small), (int)small.size(), mx, 0, 0});
+        steps.push_back(BatchStep{3, mode, prec, coarse, push_tasks(b, small), (int)small.size(), mx, 0});
       }
       t.swap(large);
     }
+  }
+  if constexpr (std::is_same<TS, float>::value && std::is_same<T, float>::value) {
+    for (const bool sten : {false, true}) {
+      std::vector<StencilTask<TS, T>> u;
+      for (const auto& tk : t)
+        if ((tk.op.sten != nullptr) == sten) u.push_back(tk);
+      if (u.empty()) continue;
+      // one z-chunk for the whole step: the least modelled time, as in f32_tiles
+      int max_n = 0;
+      for (const auto& tk : u) max_n = std::max(max_n, tk.op.n);
+      int zch = 1;
+      double best = 1e300;
+      for (int z = max_n; z >= 1; --z) {
+        int64_t tiles = 0;
+        for (const auto& tk : u) {
+          const TileGrid g = f32_tiles(tk.op.n, z);
+          tiles += (int64_t)g.per_z() * g.gz;
+        }
+        const double cost = (double)((tiles + 2 * b->sms - 1) / (2 * b->sms)) * (z + 2.0);
+        if (cost < best - 1e-9) {
+          best = cost;
+          zch = z;
+        }
+      }
+      int64_t tiles = 0;
+      for (auto& tk : u) {
+        tk.tg = f32_tiles(tk.op.n, zch);
+        tk.tile0 = tiles;
+        tiles += (int64_t)tk.tg.per_z() * tk.tg.gz;
+      }
+      const size_t off = push_tasks(b, u);
+      push_gather(steps, u, off, prec);
+      steps.push_back(BatchStep{4, mode, prec, sten, off, (int)u.size(), tiles, 0});
+    }
+    return;
   }
   if (t.empty()) return;
   // one z-chunk for the whole step: about six waves of resident blocks over
@@ -1179,14 +1247,17 @@ void push_stencil(agca_batch* b, std::vector<BatchStep>& steps, int mode, bool c
   for (const auto& tk : t) cols += (int64_t)stencil_tiles(tk.op.n, 8, 0).per_z() * (tk.op.n + 1);
   const int64_t slots = 6 * (int64_t)b->sms * 3;
   const int zch = (int)std::min<int64_t>(32, std::max<int64_t>(4, (cols + slots - 1) / slots));
-  int64_t tiles = 0, gca = 0;
+  int64_t tiles = 0;
   for (auto& tk : t) {
     tk.tg = edge_form_step<TS, T>(mode, coarse) ? edge_tiles(tk.op.n, zch) : stencil_tiles(tk.op.n, 8, zch);
     tk.tile0 = tiles;
     tiles += (int64_t)tk.tg.per_z() * tk.tg.gz;
-    gca = std::max<int64_t>(gca, tk.op.sten ? 0 : tk.op.n_flag * 12);  // stencils need no product launch
   }
-  BatchStep st{0, mode, prec, coarse, push_tasks(b, t), (int)t.size(), tiles, coarse ? gca : 0, 0};
+  const size_t off = push_tasks(b, t);
+  if constexpr (std::is_same<TS, T>::value) {
+    if (coarse) push_gather(steps, t, off, prec);
+  }
+  BatchStep st{0, mode, prec, coarse, off, (int)t.size(), tiles, 0};
   steps.push_back(st);
 }
 
@@ -1198,7 +1269,7 @@ void push_xfer(agca_batch* b, std::vector<BatchStep>& steps, int kind, const std
     mx = std::max(mx, tk.count);
     if (kind == XK_COARSE) mm = std::max(mm, 3 * (tk.nf - 1) * (tk.nf - 1) * (tk.nf - 1));
   }
-  BatchStep st{1, kind, prec, false, push_tasks(b, t), (int)t.size(), mx, 0, mm};
+  BatchStep st{1, kind, prec, false, push_tasks(b, t), (int)t.size(), mx, mm};
   steps.push_back(st);
 }
 
@@ -1206,7 +1277,7 @@ void push_krylov(agca_batch* b, std::vector<BatchStep>& steps, int op, const std
   if (t.empty()) return;
   int64_t mx = 0;
   for (auto& tk : t) mx = std::max(mx, tk.n);
-  BatchStep st{2, op, 0, false, push_tasks(b, t), (int)t.size(), mx, 0, 0};
+  BatchStep st{2, op, 0, false, push_tasks(b, t), (int)t.size(), mx, 0};
   steps.push_back(st);
 }
 
@@ -1224,7 +1295,13 @@ void build_cycle(agca_batch* b, std::vector<BatchStep>& steps, const std::vector
     agca_ctx* c = b->ctx[p];
     return mixed ? static_cast<const T*>(c->lev[c->L].vb) : reinterpret_cast<const T*>(r[p]);
   };
-  if (mixed) {
+  auto set_x1 = [&](XferTask& x, agca_ctx* c, int l) {
+    const auto fi = first_iterate<T>(c, l, static_cast<T*>(c->lev[l].vt));
+    x.invD = fi.invD;
+    x.x1 = fi.x1;
+    x.s2 = (double)fi.s2;
+  };
+  {
     std::vector<XferTask> t;
     for (int p : b->members) {
       agca_ctx* c = b->ctx[p];
@@ -1233,9 +1310,10 @@ void build_cycle(agca_batch* b, std::vector<BatchStep>& steps, const std::vector
       x.src = r[p];
       x.dst = c->lev[c->L].vb;
       x.sc = sc_of(p);
-      t.push_back(x);
+      set_x1(x, c, c->L);
+      if (mixed || x.x1) t.push_back(x);
     }
-    push_xfer(b, steps, XK_D2F, t, 1);
+    push_xfer(b, steps, mixed ? XK_D2F : XK_X1, t, pr);
   }
   // down-sweep by depth below each problem's finest level
   for (int d = 0; d <= maxL - 2; ++d) {
@@ -1250,7 +1328,7 @@ void build_cycle(agca_batch* b, std::vector<BatchStep>& steps, const std::vector
       T* X = static_cast<T*>(lv.vx);
       const Cheb ch = cheb_params(c, l);
       const double rho = 1.0 / ch.sigma, rn = 1.0 / (2.0 * ch.sigma - rho);
-      pre.push_back(make_task<T, T>(c, l, ST_CHEB_PRE, nullptr, bl, nullptr, X, rn * rho, 2.0 * rn / ch.delta,
+      pre.push_back(make_task<T, T>(c, l, ST_CHEB_PRE, static_cast<const T*>(lv.vt), bl, nullptr, X, rn * rho, 2.0 * rn / ch.delta,
                                     1.0 / ch.theta, sc_of(p)));
       res.push_back(make_task<T, T>(c, l, ST_RESID, X, bl, nullptr, static_cast<T*>(lv.vr), 0, 0, 0, sc_of(p)));
       XferTask x{};
@@ -1262,6 +1340,7 @@ void build_cycle(agca_batch* b, std::vector<BatchStep>& steps, const std::vector
       x.src = lv.vr;
       x.dst = c->lev[l - 1].vb;
       x.sc = sc_of(p);
+      set_x1(x, c, l - 1);
       rst.push_back(x);
     }
     push_stencil<T, T>(b, steps, ST_CHEB_PRE, d > 0, pre, pr);
@@ -1442,14 +1521,11 @@ agca_status run_steps(agca_batch* b, const std::vector<BatchStep>& steps, int64_
     if (st.kind == 0) {
       if (st.prec == 0)
         BCK(launch_stencil_batch<double, double>(st.mode, st.coarse, (const StencilTask<double, double>*)t, st.ntasks,
-                                                 st.work, st.gca, s));
-      else if (st.prec == 1)
-        BCK(launch_stencil_batch<float, float>(st.mode, st.coarse, (const StencilTask<float, float>*)t, st.ntasks,
-                                               st.work, st.gca, s));
+                                                 st.work, s));
       else
         BCK(launch_stencil_batch<double, float>(st.mode, st.coarse, (const StencilTask<double, float>*)t, st.ntasks,
-                                                st.work, st.gca, s));
-      *launches += (st.coarse && st.gca > 0) ? 2 : 1;
+                                                st.work, s));
+      *launches += 1;
     } else if (st.kind == 3) {
       if (st.prec == 0)
         BCK(launch_stencil_point_batch<double>(st.mode, (const StencilTask<double, double>*)t, st.ntasks, (int)st.work,
@@ -1457,6 +1533,15 @@ agca_status run_steps(agca_batch* b, const std::vector<BatchStep>& steps, int64_
       else
         BCK(launch_stencil_point_batch<float>(st.mode, (const StencilTask<float, float>*)t, st.ntasks, (int)st.work,
                                               s));
+      *launches += 1;
+    } else if (st.kind == 5) {
+      if (st.prec == 0)
+        BCK(launch_gather_batch<double>((const StencilTask<double, double>*)t, st.ntasks, st.work, s));
+      else
+        BCK(launch_gather_batch<float>((const StencilTask<float, float>*)t, st.ntasks, st.work, s));
+      *launches += 1;
+    } else if (st.kind == 4) {
+      BCK(launch_stencil_f32_batch(st.mode, st.coarse, (const StencilTask<float, float>*)t, st.ntasks, st.work, s));
       *launches += 1;
     } else if (st.kind == 1) {
       if (st.prec == 1)

@@ -139,90 +139,6 @@ __device__ __forceinline__ void cube_stokes_b(const T (&Xl)[4][4], const T (&Xh)
   }
 }
 
-// Flagged elements of a coarse level: y_e = s_e A_e x_e (Eq. 2.9, stored
-// Galerkin part), one thread per (element, row), written to op.ye for the
-// stencil kernel to scatter.  x follows the stencil's input convention
-// (boundary entries are zero; CHEB_PRE stages x = s2 D^-1 b).  A separate
-// launch spreads the clustered flagged elements over the whole GPU; inside
-// the stencil they would serialise in the few warps whose cubes hold them.
-// xval(d, v): the operator input (component d, vertex v) on an interior vertex
-template <typename T, typename XF>
-__device__ __forceinline__ void gca_row_of(const LevelOp<T>& op, const int64_t id, XF xval) {
-  const int64_t f = id / 12;
-  const int r = (int)(id - f * 12);
-  const int e = op.list[f];
-  const int cube = e / 6, t = e - cube * 6;
-  const int n = op.n, nv = n + 1;
-  const int q0 = cube / n, ci = cube - q0 * n, ck = q0 / n, cj = q0 - ck * n;
-  const T* M = op.gca + f * 144 + r * 12;
-  T acc = T(0);
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int q = tet_corner(t, b);
-    const int i = ci + (q & 1), j = cj + ((q >> 1) & 1), k = ck + ((q >> 2) & 1);
-    const bool inner = i > 0 && j > 0 && k > 0 && i < n && j < n && k < n;
-    const int v = i + nv * (j + nv * k);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const T xv = inner ? (T)xval(d, v) : T(0);
-      acc = fma(M[d * 4 + b], xv, acc);
-    }
-  }
-  op.ye[f * 12 + r] = op.gscale ? op.gscale[f] * acc : acc;
-}
-
-template <typename TS, typename T, bool PRE>
-__device__ __forceinline__ void gca_row(const LevelOp<T>& op, const StencilArgs<TS>& a, const int64_t id) {
-  const int V = (op.n + 1) * (op.n + 1) * (op.n + 1);
-  gca_row_of<T>(op, id, [&](int d, int v) -> TS {
-    if (PRE) return a.s2 * __ldg(a.invD + d * V + v) * __ldg(a.b + d * V + v);
-    return __ldg(a.x + d * V + v);
-  });
-}
-
-// Stored-Galerkin part of a coarse operator at interior vertex (i, j, k) of a
-// grid with n cubes per axis (Remark 5): g += sum_o S[o] x(v + o) over the 15
-// Kuhn offsets, S = op.sten + 135 s for the vertex's stencil index s; Dirichlet
-// neighbours contribute nothing.  xval(d, v'): operator input (component d,
-// vertex v').  Fixed order: offset, then component.
-template <typename T, typename XF>
-__device__ __forceinline__ void stencil_gather(const LevelOp<T>& op, const int s, const int i, const int j, const int k,
-                                               XF xval, T (&g)[3]) {
-  const int n = op.n, nv = n + 1;
-  const T* S = op.sten + (int64_t)s * 135;
-  T acc[3] = {T(0), T(0), T(0)};
-#pragma unroll
-  for (int o = 0; o < 15; ++o) {
-    const int a = i + kuhn_offset_comp(o, 0), b = j + kuhn_offset_comp(o, 1), c = k + kuhn_offset_comp(o, 2);
-    if (a <= 0 || b <= 0 || c <= 0 || a >= n || b >= n || c >= n) continue;
-    const int w = a + nv * (b + nv * c);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const T xv = (T)xval(d, w);
-#pragma unroll
-      for (int r = 0; r < 3; ++r) acc[r] = fma(S[o * 9 + r * 3 + d], xv, acc[r]);
-    }
-  }
-  const T sc = op.sscale ? op.sscale[s] : T(1);
-#pragma unroll
-  for (int r = 0; r < 3; ++r) g[r] = op.sscale ? sc * acc[r] : acc[r];
-}
-
-// Result of a fused stencil mode at one vertex from the operator value y =
-// (A x)_v, the vertex's own iterate xo, rhs eb, inverse diagonal ed and
-// previous iterate ep (Chebyshev steps of Sec. 4; CHEB_PRE starts from x0 = 0
-// with xo = x1 = s2 D^-1 b).
-template <int MODE, typename TS>
-__device__ __forceinline__ TS stencil_epilogue(const TS xo, const TS y, const TS eb, const TS ed, const TS ep,
-                                               const TS s0, const TS s1) {
-  if (MODE == ST_APPLY || MODE == ST_STOKES) return y;
-  if (MODE == ST_STOKES_B) return eb + y;
-  if (MODE == ST_RESID) return eb - y;
-  if (MODE == ST_CHEB_FIRST) return xo + s0 * ed * (eb - y);
-  if (MODE == ST_CHEB_STEP) return xo + s0 * (xo - ep) + s1 * ed * (eb - y);
-  return xo + s0 * xo + s1 * ed * (eb - y);  // ST_CHEB_PRE
-}
-
 // ------------------------------------------------------------------ transfers
 // Linear interpolation between Kuhn grids and its transpose (Sec. 2.1).  Every
 // fine vertex is either 2i (a coarse vertex) or the midpoint 2i + d of the

@@ -308,10 +308,19 @@ __global__ void gca_to_f32_kernel(int64_t n_flag, const int32_t* list, const dou
   if (id % 144 == 0) scale32[f] = (float)s;
 }
 
-__global__ void d2f_kernel(const double* in, float* out, int64_t n) {
+__global__ void d2f_kernel(const double* __restrict__ in, float* __restrict__ out, int64_t n,
+                           const FirstIterate<float> fi) {
+  grid_dep_entry();
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const float v = (float)in[i];
+    out[i] = v;
+    if (fi.x1) fi.x1[i] = fi.s2 * __ldg(fi.invD + i) * v;
+  }
+}
+__global__ void x1_kernel(const double* __restrict__ b, const FirstIterate<double> fi, int64_t n) {
   grid_dep_entry();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = (float)in[i];
+    fi.x1[i] = fi.s2 * __ldg(fi.invD + i) * b[i];
 }
 __global__ void f2d_kernel(const float* in, double* out, int64_t n) {
   grid_dep_entry();
@@ -530,8 +539,12 @@ cudaError_t launch_gca_to_f32(int64_t n_flag, const int32_t* list, const double*
   return cudaGetLastError();
 }
 
-cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s) {
-  KL(launch_k(d2f_kernel, dim3(1216), dim3(256), 0, s, in, out, n));
+cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s, const FirstIterate<float>& fi) {
+  KL(launch_k(d2f_kernel, dim3(1216), dim3(256), 0, s, in, out, n, fi));
+  return cudaGetLastError();
+}
+cudaError_t launch_x1(const double* b, const FirstIterate<double>& fi, int64_t n, cudaStream_t s) {
+  KL(launch_k(x1_kernel, dim3(1216), dim3(256), 0, s, b, fi, n));
   return cudaGetLastError();
 }
 cudaError_t launch_f2d(const float* in, double* out, int64_t n, cudaStream_t s) {

@@ -23,10 +23,16 @@
 //
 // GB300 runs one FP64 fused multiply-add per 64 FP32 ones, so FP64
 // arithmetic bounds the operator; the records are formed once per viscosity
-// (edge_record_kernel) and read by each vertex's own thread.  (The FP32
-// cycle keeps the per-cube kernel: an FP32 instance of this kernel, records
-// formed in-kernel from staged cube rows, issued about 1,600 instructions per
-// vertex, mostly integer, and ran 2.3x slower.)
+// (edge_record_kernel) and read by each vertex's own thread.  (The FP32 cycle
+// is bound by memory instead and forms the weights from the element
+// coefficients: stencil_f32.cu.)
+//
+// The Chebyshev step from zero takes its first iterate x1 as the input vector:
+// formed while staging it cost 1.6 D^-1 b products per vertex and a second ring
+// (110 KB a block); at 256^3 cubes the step took 4.28 ms against 3.07 ms as a
+// first step plus 0.2 ms for x1.  The stored-Galerkin part comes from
+// launch_gather (at 128^3 cubes with 8 spheres one thread walking a vertex's 135
+// values held its block up: FP64 cycle at 64^3 pressure cubes 3.18 -> 2.62 ms).
 //
 // Tiling: a CTA of 32 x 8 threads, thread (tx, ty) <-> vertex column
 // (x0 - 1 + tx, y0 - 1 + ty), marches a chunk of z-planes.  Per plane k it
@@ -65,10 +71,9 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;
 
 template <typename T, int MODE>
 __host__ __device__ constexpr size_t edge_smem_elems() {
-  // x ring [3][3][XT] (+ D^-1 ring for the step from zero), difference ring
-  // [3][6][DT], y-flux exchange [3][ENT]: in FP64 82 KB, or 110 KB with the
-  // D^-1 ring
-  return (size_t)(MODE == ST_CHEB_PRE ? 2 : 1) * 3 * 3 * XT + (size_t)3 * 6 * DT + (size_t)3 * ENT;
+  // x ring [3][3][XT], difference ring [3][6][DT], y-flux exchange [3][ENT]:
+  // 82 KB in FP64
+  return (size_t)3 * 3 * XT + (size_t)3 * 6 * DT + (size_t)3 * ENT;
 }
 // resident CTAs per SM (shared memory and the 128-register budget)
 template <typename T, int MODE>
@@ -136,8 +141,7 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
   constexpr bool PRE = MODE == ST_CHEB_PRE;
 
   T* xs = sm;                                    // [3][3][XT]
-  T* xa = xs + 3 * 3 * XT;                       // PRE: D^-1 ring [3][3][XT]
-  T* ds = xa + (PRE ? 3 * 3 * XT : 0);           // [3][6][DT]
+  T* ds = xs + 3 * 3 * XT;                       // [3][6][DT]
   T* fy = ds + 3 * 6 * DT;                       // [3][ENT]
 
   const int zs = za - 2;  // planes zs + i use ring slot i mod 3
@@ -147,11 +151,10 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
   // last XW - 32 lanes): interior in x?  Dirichlet and outside vertices read 0
   const bool inx0 = x0 - 2 + tx > 0 && x0 - 2 + tx < n;
   const bool inx1 = tx < XW - 32 && x0 + 30 + tx > 0 && x0 + 30 + tx < n;
-  // stage x plane p (PRE: b and D^-1): warp ty copies the rows r = ty, ty + 8, ..
+  // stage x plane p: warp ty copies the rows r = ty, ty + 8, ..
   // of the [3][XH] rows of the tile
   auto issue_x = [&](int p) {
     T* dst = xs + slot(p) * 3 * XT;
-    T* dsa = xa + slot(p) * 3 * XT;
     const bool zin = p > 0 && p < n;
     for (int r = ty; r < 3 * XH; r += NWARP) {
       const int c = r / XH, j = r - c * XH;
@@ -161,30 +164,8 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
       const int e = c * XT + j * XW + tx;
       const bool ok0 = rin && inx0, ok1 = rin && inx1;
       const int g0 = ok0 ? g + tx : 0, g1 = ok1 ? g + 32 + tx : 0;
-      if (PRE) {
-        cpT(dst + e, a.b + g0, ok0);
-        cpT(dsa + e, a.invD + g0, ok0);
-        if (tx < XW - 32) {
-          cpT(dst + e + 32, a.b + g1, ok1);
-          cpT(dsa + e + 32, a.invD + g1, ok1);
-        }
-      } else {
-        cpT(dst + e, a.x + g0, ok0);
-        if (tx < XW - 32) cpT(dst + e + 32, a.x + g1, ok1);
-      }
-    }
-  };
-  // PRE: the first Chebyshev iterate x1 = (s2 D^-1) b of the entries this
-  // thread staged (the same operations as the per-tetrahedron kernel)
-  auto convert_x = [&](int p) {
-    if (!PRE) return;
-    T* dst = xs + slot(p) * 3 * XT;
-    const T* dsa = xa + slot(p) * 3 * XT;
-    for (int r = ty; r < 3 * XH; r += NWARP) {
-      const int c = r / XH, j = r - c * XH;
-      const int e = c * XT + j * XW + tx;
-      dst[e] = a.s2 * dsa[e] * dst[e];
-      if (tx < XW - 32) dst[e + 32] = a.s2 * dsa[e + 32] * dst[e + 32];
+      cpT(dst + e, a.x + g0, ok0);
+      if (tx < XW - 32) cpT(dst + e + 32, a.x + g1, ok1);
     }
   };
   // edge differences of plane p from x planes p, p + 1: difference-tile
@@ -230,9 +211,6 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
   issue_x(zs + 2);
   cp_commit();
   cp_wait_all();
-  convert_x(zs);
-  convert_x(zs + 1);
-  convert_x(zs + 2);
   __syncthreads();
   T dcur[3][3], dnext[3][3];
   compute_d(zs, dnext);
@@ -246,7 +224,6 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
 
   for (int k = za - 1; k < zb; ++k) {
     cp_wait_all();
-    convert_x(k + 2);
     __syncthreads();  // x plane k+2 staged; ring slots of k-2 free
     compute_d(k + 1, dnext);
     __syncthreads();  // differences of plane k+1 visible; x slot of plane k free
@@ -267,7 +244,7 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
         if (MODE != ST_APPLY) eb[c] = __ldg(a.b + c * V + vo);
         if (MODE == ST_CHEB_FIRST || MODE == ST_CHEB_STEP || MODE == ST_CHEB_PRE) ed[c] = __ldg(a.invD + c * V + vo);
         if (MODE == ST_CHEB_STEP) ep[c] = a.xprev[c * V + vo];
-        if (MODE == ST_CHEB_FIRST || MODE == ST_CHEB_STEP) xo[c] = __ldg(a.x + c * V + vo);
+        if (MODE == ST_CHEB_FIRST || MODE == ST_CHEB_STEP || PRE) xo[c] = __ldg(a.x + c * V + vo);
       }
     }
 
@@ -314,14 +291,13 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
       fy[c * ENT + tid] = Fy[c];
     }
     __syncthreads();  // y fluxes of the tile visible
-    T gs[3] = {T(0), T(0), T(0)};  // stored-Galerkin part (coarse levels)
+    T gs[3] = {T(0), T(0), T(0)};  // stored-Galerkin part (coarse levels, launch_gather)
     if (op.sten && inner) {
-      const int sv = op.sidx[vo];
-      if (sv >= 0)
-        stencil_gather<T>(op, sv, gx, gy, k, [&](int d, int w) -> T {
-          if (PRE) return a.s2 * __ldg(a.invD + d * V + w) * __ldg(a.b + d * V + w);
-          return __ldg(a.x + d * V + w);
-        }, gs);
+      const int sv = __ldg(op.sidx + vo);
+      if (sv >= 0) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) gs[c] = __ldg(op.ye + 3 * (int64_t)sv + c);
+      }
     }
     if (out_k) {
 #pragma unroll
@@ -339,10 +315,7 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
             if (MODE == ST_RESID) o = r;
             if (MODE == ST_CHEB_FIRST) o = fma(a.s0, ed[c] * r, xo[c]);
             if (MODE == ST_CHEB_STEP) o = fma(a.s1, ed[c] * r, fma(a.s0, xo[c] - ep[c], xo[c]));
-            if (MODE == ST_CHEB_PRE) {
-              const T x1 = a.s2 * ed[c] * eb[c];
-              o = fma(a.s1, ed[c] * r, fma(a.s0, x1, x1));
-            }
+            if (PRE) o = fma(a.s1, ed[c] * r, fma(a.s0, xo[c], xo[c]));  // a.x holds the first iterate
           }
         }
         if (a.out64)

@@ -37,6 +37,47 @@ constexpr int PT = 128;  // threads per block: 16 vertices, so that small levels
 // coefficient sources of a level
 enum PointCoef { PC_PLAIN = 0, PC_MASK = 1, PC_RECORD = 2 };  // op.coef, op.coef with flagged elements zero, op.hedge
 
+// Stored-Galerkin part of a coarse operator at vertex (vi, vj, vk) with stencil
+// index sv (Remark 5), by the eight lanes e of the vertex (lanes without a
+// stencil pass sv < 0): g = sum_o S[o] x(v + o) over the 15 Kuhn offsets,
+// offsets e and e + 8 in lane e, added by shuffles so that every lane holds g.
+// Dirichlet neighbours contribute nothing.  All lanes of the warp call it.
+template <typename T, typename XF>
+__device__ __forceinline__ void gather_lanes(const LevelOp<T>& op, const int sv, const int vi, const int vj,
+                                             const int vk, const int e, XF xat, T (&g)[3]) {
+  const int n = op.n, nv = n + 1;
+  if (sv >= 0) {
+    const T* St = op.sten + (int64_t)sv * 135;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int o = e + 8 * r;
+      // offset pair (o - 1) / 2 of x, y, z, xy, xz, yz, xyz; odd o: +, even o: -
+      const int p = o > 0 ? (o - 1) >> 1 : 0, sg = o == 0 ? 0 : ((o & 1) ? 1 : -1);
+      const int bits = (int)((0x7653421u >> (4 * p)) & 7u);
+      const int i = vi + sg * (bits & 1), j = vj + sg * ((bits >> 1) & 1), k = vk + sg * (bits >> 2);
+      if (o < 15 && i > 0 && j > 0 && k > 0 && i < n && j < n && k < n) {
+        const int wv = i + nv * (j + nv * k);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          const T xv = xat(d, wv, true);
+#pragma unroll
+          for (int q = 0; q < 3; ++q) g[q] = fma(__ldg(St + o * 9 + q * 3 + d), xv, g[q]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+#pragma unroll
+    for (int off = 1; off < 8; off <<= 1) g[q] += __shfl_xor_sync(0xffffffffu, g[q], off);
+  }
+  if (sv >= 0 && op.sscale) {
+    const T s = op.sscale[sv];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) g[q] *= s;
+  }
+}
+
 template <typename T, int MODE, int COEF>
 __device__ __forceinline__ void stencil_point(const LevelOp<T>& op, const StencilArgs<T>& a, const int64_t id) {
   const int n = op.n, nv = n + 1, V = nv * nv * nv;
@@ -135,43 +176,11 @@ __device__ __forceinline__ void stencil_point(const LevelOp<T>& op, const Stenci
     for (int off = 1; off < 8; off <<= 1) F[q] += __shfl_xor_sync(0xffffffffu, F[q], off);
   }
 
-  // stored-Galerkin part of a touched vertex: offsets e and e + 8 of the 15
+  // stored-Galerkin part of a touched vertex
   T g[3] = {T(0), T(0), T(0)};
   if (op.sten) {
     const int sv = inner ? op.sidx[v] : -1;
-    if (__any_sync(0xffffffffu, sv >= 0)) {
-      if (sv >= 0) {
-        const T* St = op.sten + (int64_t)sv * 135;
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const int o = e + 8 * r;
-          // offset pair (o - 1) / 2 of x, y, z, xy, xz, yz, xyz; odd o: +, even o: -
-          const int p = o > 0 ? (o - 1) >> 1 : 0, sg = o == 0 ? 0 : ((o & 1) ? 1 : -1);
-          const int bits = (int)((0x7653421u >> (4 * p)) & 7u);
-          const int oi = sg * (bits & 1), oj = sg * ((bits >> 1) & 1), ok = sg * (bits >> 2);
-          const int i = vi + oi, j = vj + oj, k2 = vk + ok;
-          if (o < 15 && i > 0 && j > 0 && k2 > 0 && i < n && j < n && k2 < n) {
-            const int wv = v + oi + nv * (oj + nv * ok);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-              const T xv = xat(d, wv, true);
-#pragma unroll
-              for (int q = 0; q < 3; ++q) g[q] = fma(__ldg(St + o * 9 + q * 3 + d), xv, g[q]);
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-#pragma unroll
-        for (int off = 1; off < 8; off <<= 1) g[q] += __shfl_xor_sync(0xffffffffu, g[q], off);
-      }
-      if (sv >= 0 && op.sscale) {
-        const T s = op.sscale[sv];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) g[q] *= s;
-      }
-    }
+    if (__any_sync(0xffffffffu, sv >= 0)) gather_lanes<T>(op, sv, vi, vj, vk, e, xat, g);
   }
   if (!out_lane) return;
   const T sum = e == 0 ? F[0] : (e == 1 ? F[1] : F[2]);
@@ -195,6 +204,40 @@ __device__ __forceinline__ void stencil_point(const LevelOp<T>& op, const Stenci
     a.out64[vo] = (double)o;  // the mixed cycle's result, widened
   else
     a.out[vo] = o;
+}
+
+// The stored-Galerkin part alone, for the tile kernels: op.ye[3 s + c] for the
+// vertex with stencil index s (its room is the 12 values per flagged element,
+// and an element has four vertices).  Inside a tile one thread would walk its
+// vertex's 135 stencil values alone while the block waits: that made the coarse
+// levels of a twelve-problem batch eight times slower per vertex.
+template <typename T>
+__device__ __forceinline__ void gather_point(const LevelOp<T>& op, const T* __restrict__ x, const int64_t id) {
+  const int nv = op.n + 1, V = nv * nv * nv;
+  const int e = (int)(id & 7);
+  const int64_t s64 = id >> 3;
+  const bool exists = s64 < op.n_sv;
+  const int v = exists ? __ldg(op.slist + s64) : 0;
+  const int vk = v / (nv * nv), vr = v - vk * nv * nv, vj = vr / nv, vi = vr - vj * nv;
+  T g[3] = {T(0), T(0), T(0)};
+  gather_lanes<T>(op, exists ? (int)s64 : -1, vi, vj, vk, e,
+                  [&](int d, int w, bool) -> T { return __ldg(x + d * V + w); }, g);
+  if (exists && e < 3) op.ye[3 * s64 + e] = e == 0 ? g[0] : (e == 1 ? g[1] : g[2]);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(PT) gather_kernel(const LevelOp<T> op, const T* __restrict__ x) {
+  grid_dep_entry();
+  gather_point<T>(op, x, blockIdx.x * (int64_t)PT + threadIdx.x);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(PT) gather_batch_kernel(const StencilTask<T, T>* __restrict__ tasks) {
+  grid_dep_entry();
+  const StencilTask<T, T>& tk = tasks[blockIdx.y];
+  if (tk.sc && tk.sc[MS_DONE] != 0.0) return;  // converged problem
+  if (blockIdx.x * (int64_t)(PT / 8) >= tk.op.n_sv) return;
+  gather_point<T>(tk.op, tk.a.x, blockIdx.x * (int64_t)PT + threadIdx.x);
 }
 
 template <typename T, int MODE, int COEF>
@@ -264,6 +307,23 @@ cudaError_t launch_stencil_point_batch(int mode, const StencilTask<T, T>* tasks,
   return cudaGetLastError();
 }
 
+template <typename T>
+cudaError_t launch_gather(const LevelOp<T>& op, const T* x, cudaStream_t s) {
+  if (!op.sten || op.n_sv <= 0) return cudaSuccess;
+  return launch_k(gather_kernel<T>, dim3((unsigned)((op.n_sv * 8 + PT - 1) / PT)), dim3(PT), 0, s, op, x);
+}
+
+template <typename T>
+cudaError_t launch_gather_batch(const StencilTask<T, T>* tasks, int ntasks, int64_t max_sv, cudaStream_t s) {
+  if (ntasks <= 0 || max_sv <= 0) return cudaSuccess;
+  return launch_k(gather_batch_kernel<T>, dim3((unsigned)((max_sv * 8 + PT - 1) / PT), (unsigned)ntasks), dim3(PT), 0,
+                  s, tasks);
+}
+
+template cudaError_t launch_gather<float>(const LevelOp<float>&, const float*, cudaStream_t);
+template cudaError_t launch_gather<double>(const LevelOp<double>&, const double*, cudaStream_t);
+template cudaError_t launch_gather_batch<float>(const StencilTask<float, float>*, int, int64_t, cudaStream_t);
+template cudaError_t launch_gather_batch<double>(const StencilTask<double, double>*, int, int64_t, cudaStream_t);
 template cudaError_t launch_stencil_point<float>(int, const LevelOp<float>&, const StencilArgs<float>&, cudaStream_t);
 template cudaError_t launch_stencil_point<double>(int, const LevelOp<double>&, const StencilArgs<double>&,
                                                   cudaStream_t);

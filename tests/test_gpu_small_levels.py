@@ -1,8 +1,10 @@
 """The eight-lanes-per-vertex kernel of the small levels and the coarsest solve
 by the explicit inverse, at the edges of their ranges: grids of 2 to 5 cubes
-per axis, odd sizes, and the largest size (32 cubes) and the first tiled ones
-against the other precision on the same grid.  Tolerances as in test_gpu_parity.py: 1e-12 (FP64) and
-1e-5 (FP32) of the largest entry for an apply, 1e-9 and 1e-4 for a cycle."""
+per axis, odd sizes, and the largest size (32 cubes); the first tiled sizes
+(tiles cut in x and y, one and two tiled levels, nearly every coarse element
+flagged) against the other precision on the same grid.  Tolerances as in
+test_gpu_parity.py: 1e-12 (FP64) and 1e-5 (FP32) of the largest entry for an
+apply, 1e-9 and 1e-4 for a cycle."""
 import numpy as np
 import pytest
 import torch
@@ -50,7 +52,8 @@ def test_small_levels_match_oracle(N, L, nu):
         assert np.abs(z * (1 - H.mask[L])).max() == 0.0
 
 
-@pytest.mark.parametrize("N", [16, 18, 24])  # 32 cubes per axis: the last point level; 36 and 48: tiles over point levels
+# finest cubes per axis 32: the last point level; 36, 40, 48: tiles over point levels; 72: two tiled levels
+@pytest.mark.parametrize("N", [16, 18, 20, 24, 36])
 def test_point_kernel_meets_tile_kernel(N):
     eta = torch.from_numpy(_eta(N, N)).to(DEV)
     c64, c32 = (pkg.Context(N, None, p, device=DEV) for p in (pkg.FP64, pkg.MIXED))
@@ -62,3 +65,6 @@ def test_point_kernel_meets_tile_kernel(N):
         big = float(ref.abs().max())
         assert float((c32.apply(l, x.double()) - ref).abs().max()) <= 1e-12 * big
         assert float((c32.apply(l, x, dtype=pkg.F32).double() - ref).abs().max()) <= 1e-5 * big
+    r = torch.from_numpy(random_vector(3 * c64.V[c64.L], 7)).to(DEV)
+    ref = c64.vcycle(r)
+    assert float((c32.vcycle(r) - ref).abs().max()) <= 1e-4 * float(ref.abs().max())
