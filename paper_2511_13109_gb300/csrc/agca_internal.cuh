@@ -99,13 +99,11 @@ struct LevelOp {
   T hq;                // h^2 / 6 (divergence terms, finest level)
   const T* coef;       // per-element coefficient: eta (finest) or child mean (coarse)
   const int32_t* fidx; // compact Galerkin index per element or -1; nullptr on finest
-  const T* gca;        // stored Galerkin matrices (n_flag * 144)
-  const T* gscale;     // per flagged element scale (mixed) or nullptr
+  const T* gca;        // stored Galerkin matrices (n_flag * 144, FP64)
   const int32_t* list; // flagged element ids (coarse levels)
   int64_t n_flag;      // number of flagged elements
   T* ye;               // n_flag * 12 scratch: the stored-Galerkin part at the touched vertices (launch_gather)
   const T* hedge;      // FP64 levels: per-vertex coefficient records [EREC][V] of the edge form, or nullptr
-  const T* coefm;      // FP64 coarse levels: DCA coefficient with flagged elements zeroed (edge form), or nullptr
   // stored-Galerkin part as per-vertex stencils (Remark 5): stencil index of a
   // vertex or -1, 15 x 3 x 3 couplings per touched vertex, FP32 scale (mixed)
   const int32_t* sidx;
@@ -163,10 +161,8 @@ cudaError_t launch_k(void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, 
 // iterate x1 = (s2 D^-1) b on the fly; the tile kernels find it in a.x, written
 // by the kernel that wrote b (launch_restrict, launch_d2f) or by launch_x1
 enum StencilMode { ST_APPLY = 0, ST_RESID = 1, ST_CHEB_FIRST = 2, ST_CHEB_STEP = 3, ST_CHEB_PRE = 4, ST_STOKES = 5 };
-// internal (FP64 contexts, not tunable): the pressure coupling of the Stokes
-// operator added to a.b = A u from the edge form, out = a.b - B_f^T q,
-// out2 = B_f u
-constexpr int ST_STOKES_B = 6;
+// internal: D^-1 A x, a step of the power iteration (FP64 edge form and small levels)
+constexpr int ST_POWER = 6;
 
 template <typename T>
 struct StencilArgs {
@@ -211,8 +207,9 @@ constexpr int EREC = 27;
 // tile grid of the edge form; zch_req 0 picks the z-chunk for `slots`
 // resident blocks (0: 304)
 TileGrid edge_tiles(int n, int zch_req, int slots = 0);
+// (fidx: flagged elements, whose coefficient counts as zero, or nullptr)
 template <typename T>
-cudaError_t launch_edge_records(int n, const T* eta, T* rec, cudaStream_t s);
+cudaError_t launch_edge_records(int n, const T* eta, const int32_t* fidx, T* rec, cudaStream_t s);
 template <typename T>
 cudaError_t launch_stencil_edge(int mode, const LevelOp<T>& op, const StencilArgs<T>& a, cudaStream_t s, int zch_req);
 
@@ -285,7 +282,7 @@ struct XferTask {
   double s2;
   const double* sc;     // skip when sc[MS_DONE] != 0, or nullptr
 };
-enum XferKind { XK_RESTRICT = 0, XK_PROLONG_ADD, XK_D2F, XK_F2D, XK_COARSE, XK_PROLONG, XK_COPY64, XK_X1 };
+enum XferKind { XK_RESTRICT = 0, XK_PROLONG_ADD, XK_D2F, XK_F2D, XK_COARSE, XK_PROLONG, XK_COPY64, XK_X1, XK_GRADIENT, XK_DIVERGENCE };
 template <typename T>
 cudaError_t launch_xfer_batch(int kind, const XferTask* tasks, int ntasks, int64_t max_count, int max_m,
                               cudaStream_t s);
@@ -323,8 +320,6 @@ cudaError_t launch_galerkin(int nc, int64_t n_flag, const int32_t* list, int nf,
                             const double* coef_f, const int32_t* fidx_f, const double* gca_f, double* gca_c,
                             cudaStream_t s);
 cudaError_t launch_diag(const LevelOp<double>& op, double* diag, double* invD64, float* invD32, cudaStream_t s);
-cudaError_t launch_gca_to_f32(int64_t n_flag, const int32_t* list, const double* mx, const double* gca64,
-                              float* gca32, float* scale32, cudaStream_t s);
 cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s, const FirstIterate<float>& fi = {});
 cudaError_t launch_f2d(const float* in, double* out, int64_t n, cudaStream_t s);
 cudaError_t launch_coarse_assemble(const LevelOp<double>& op, double* dense, cudaStream_t s);
@@ -333,16 +328,27 @@ cudaError_t launch_trinv(const double* l, int m, double* linv_cm, double* linv_r
 cudaError_t launch_coarse_inverse(const double* linv_rm, int m, double* ainv, cudaStream_t s);
 template <typename T>
 cudaError_t launch_coarse_solve(int n, const double* ainv, const T* r, T* z, cudaStream_t s);
-cudaError_t launch_pressure_mass(int np, const double* eta_f, double* pmass, double* pmass_inv, cudaStream_t s);
+// work: 6 np^3 doubles of scratch
+cudaError_t launch_pressure_mass(int np, const double* eta_f, double* work, double* pmass, double* pmass_inv,
+                                 cudaStream_t s);
 // stencil storage of the flagged elements' Galerkin matrices (stencil_store.cu)
 cudaError_t launch_mark_vertices(int n, const uint8_t* flags, uint8_t* mark, cudaStream_t s);
 cudaError_t launch_stencil_assemble(int n, int64_t n_sv, const int32_t* slist, const int32_t* fidx, const double* gca,
                                     double* sten, cudaStream_t s);
 cudaError_t launch_stencil_to_f32(int64_t n_sv, const double* s64, float* s32, float* scale, cudaStream_t s);
-// DCA coefficient of a coarse level with the flagged elements zeroed, in FP64 or rounded to FP32
+// DCA coefficient of a coarse level with the flagged elements zeroed, rounded to T (FP32)
 template <typename T>
 cudaError_t launch_masked_coef(int64_t E, const double* mean, const int32_t* fidx, T* coefm, cudaStream_t s);
 cudaError_t launch_start_vector(int n, double* v, cudaStream_t s);
+
+// pressure coupling of the FP64 Stokes operator (stokes.cu): y += -B_f^T q on
+// the interior vertices of the velocity grid (n cubes per axis), y = B u on the
+// pressure grid (np cubes per axis; boundary entries of u are ignored).  Batched:
+// tasks with nf = velocity cubes per axis, src, dst
+cudaError_t launch_gradient(int n, const double* q, double* y, cudaStream_t s);
+cudaError_t launch_divergence(int np, const double* u, double* y, cudaStream_t s);
+cudaError_t launch_gradient_batch(const XferTask* tasks, int ntasks, int64_t max_count, cudaStream_t s);
+cudaError_t launch_divergence_batch(const XferTask* tasks, int ntasks, int64_t max_count, cudaStream_t s);
 
 // Stokes / Krylov kernels (krylov.cu)
 // device-resident MINRES scalar slots

@@ -236,6 +236,8 @@ cudaError_t launch_xfer_batch(int kind, const XferTask* tasks, int ntasks, int64
     case XK_D2F:
       KL(launch_k(rhs_batch_kernel<float, true>, gc, dim3(kBT), 0, s, tasks));
       break;
+    case XK_GRADIENT: return launch_gradient_batch(tasks, ntasks, max_count, s);
+    case XK_DIVERGENCE: return launch_divergence_batch(tasks, ntasks, max_count, s);
     case XK_X1:
       KL(launch_k(rhs_batch_kernel<double, false>, gc, dim3(kBT), 0, s, tasks));
       break;

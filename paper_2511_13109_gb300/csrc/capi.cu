@@ -35,7 +35,6 @@ struct Level {
   int64_t n_flag = 0;
   double* gca64 = nullptr;
   double* hedge = nullptr;  // FP64 contexts: per-vertex coefficient records [EREC][V] of the edge form
-  double* coefm = nullptr;  // FP64 coarse levels: DCA coefficient with flagged elements zeroed (edge form)
   // stencil storage of the flagged elements' Galerkin matrices (Remark 5)
   uint8_t* vmark = nullptr;   // vertex touched by a flagged element
   int32_t* sidx = nullptr;    // stencil index of a vertex or -1
@@ -49,8 +48,6 @@ struct Level {
   // FP32 copies (mixed)
   float* mean32 = nullptr;
   float* invD32 = nullptr;
-  float* gca32 = nullptr;
-  float* gscale32 = nullptr;
   // s_e A_e x_e of the flagged elements (coarse-apply scratch)
   double* ye64 = nullptr;
   float* ye32 = nullptr;
@@ -198,7 +195,6 @@ void carve_workspace(agca_ctx* ctx, char* base) {
     }
     if (mixed) lv.mean32 = cv.take<float>(lv.E);
     if (!mixed) lv.hedge = cv.take<double>(EREC * lv.V);
-    if (!mixed && l < ctx->L) lv.coefm = cv.take<double>(lv.E);
     if (l < ctx->L) {
       lv.vmark = cv.take<uint8_t>(lv.V);
       lv.sidx = cv.take<int32_t>(lv.V);
@@ -241,8 +237,6 @@ void carve_gca(agca_ctx* ctx, char* base) {
     lv.sten64 = cv.take<double>(std::max<int64_t>(1, lv.n_sv * 135));
     if (mixed) {
       lv.ye32 = cv.take<float>(std::max<int64_t>(1, lv.n_flag * 12));
-      lv.gca32 = cv.take<float>(std::max<int64_t>(1, lv.n_flag * 144));
-      lv.gscale32 = cv.take<float>(std::max<int64_t>(1, lv.n_flag));
       lv.sten32 = cv.take<float>(std::max<int64_t>(1, lv.n_sv * 135));
       lv.sscale32 = cv.take<float>(std::max<int64_t>(1, lv.n_sv));
     }
@@ -259,7 +253,6 @@ LevelOp<double> op64(const agca_ctx* ctx, int l) {
   op.coef = lv.mean;
   op.hedge = lv.hedge;
   if (l < ctx->L) {
-    op.coefm = lv.coefm;
     op.sidx = lv.sidx;
     op.slist = lv.slist;
     op.n_sv = lv.n_sv;
@@ -287,8 +280,6 @@ LevelOp<float> op32(const agca_ctx* ctx, int l) {
     op.sten = lv.n_sv > 0 ? lv.sten32 : nullptr;
     op.sscale = lv.n_sv > 0 ? lv.sscale32 : nullptr;
     op.fidx = lv.fidx;
-    op.gca = lv.gca32;
-    op.gscale = lv.gscale32;
     op.list = lv.list;
     op.n_flag = lv.n_flag;
     op.ye = lv.ye32;
@@ -552,22 +543,18 @@ agca_status stokes_impl(agca_ctx* ctx, const double* x, double* y) {
   LK(1, launch_prolong<double>(lf.n, 1, false, false, x + n3, ctx->qfine, ctx->stream));
   StencilArgs<double> a{};
   a.x = x;
-  a.q = ctx->qfine;
   a.out = y;
-  a.out2 = ctx->sfine;
-  if (std::is_same<TC, double>::value && lf.hedge) {
-    // FP64 context: the viscous block in edge form (A u into y), then the
-    // pressure coupling per cube added to it (y = A u - B_f^T q, B_f u)
-    StencilArgs<double> e{};
-    e.x = x;
-    e.out = y;
-    LK(1, launch_stencil<double, double>(ST_APPLY, op64(ctx, L), e, ctx->stream));
-    a.b = y;
-    LK(1, launch_stencil<double, double>(ST_STOKES_B, op64(ctx, L), a, ctx->stream));
+  if (std::is_same<TC, double>::value) {
+    // FP64: the viscous block, then the pressure coupling (y_u += B^T p, y_p = B u)
+    LK(1, launch_stencil<double, double>(ST_APPLY, op64(ctx, L), a, ctx->stream));
+    LK(1, launch_gradient(lf.n, ctx->qfine, y, ctx->stream));
+    LK(1, launch_divergence(ctx->N, x, y + n3, ctx->stream));
   } else {
-    LK(1, launch_stencil<double, TC>(ST_STOKES, level_op<TC>(ctx, L), a, ctx->stream));
+    a.q = ctx->qfine;
+    a.out2 = ctx->sfine;
+    LK(1, launch_stencil<double, float>(ST_STOKES, op32(ctx, L), a, ctx->stream));
+    LK(1, launch_restrict<double>(lf.n, 1, false, -1.0, ctx->sfine, y + n3, ctx->stream));
   }
-  LK(1, launch_restrict<double>(lf.n, 1, false, -1.0, ctx->sfine, y + n3, ctx->stream));
   return AGCA_OK;
 }
 
@@ -966,28 +953,47 @@ agca_status check_status(agca_ctx* ctx, const char* where) {
   return AGCA_OK;
 }
 
-agca_status power_lambda(agca_ctx* ctx, int l, double* lam) {
-  const Level& lv = ctx->lev[l];
+// Power iteration on D^-1 A_l from the start vector, then the two inner
+// products of the Rayleigh quotient (v^T A v) / (v^T D v) into
+// sc[kRaySlot + 2 l], sc[kRaySlot + 2 l + 1].  The quotient does not depend on
+// the length of v, so v is normalised only every 16 steps, against overflow.
+// Tiled levels run the edge form; a mixed context, which keeps no coefficient
+// records, forms the level's in the Krylov vectors the iteration leaves free
+// (27 V values in 10 vectors of 3 V and more; the per-cube kernel it would
+// otherwise run takes 1047 against 412 us at 128^3 cubes).
+constexpr int kRaySlot = 24;
+static_assert(kRaySlot >= MS_COUNT && kRaySlot + 2 * 12 + 2 <= 64, "scalar slots for up to 12 levels");
+agca_status power_lambda(agca_ctx* ctx, int l) {
+  Level& lv = ctx->lev[l];
   const int64_t n3 = 3 * lv.V;
   cudaStream_t s = ctx->stream;
+  const bool scratch = lv.hedge == nullptr && lv.n > kPointMaxN;
+  if (scratch) {
+    lv.hedge = ctx->kv[KV_Z];
+    const cudaError_t e = launch_edge_records(lv.n, lv.mean, l < ctx->L ? lv.fidx : nullptr, lv.hedge, s);
+    if (e != cudaSuccess) lv.hedge = nullptr;
+    LK(1, e);
+  }
   double* v = ctx->kv[KV_VOLD];
   double* w = ctx->kv[KV_V];
-  LK(1, launch_start_vector(lv.n, v, s));
-  for (int it = 0; it < ctx->power_iters; ++it) {
+  auto run = [&]() -> agca_status {
+    LK(1, launch_start_vector(lv.n, v, s));
+    for (int it = 0; it < ctx->power_iters; ++it) {
+      CKS(stencil<double>(ctx, ST_POWER, l, v, nullptr, nullptr, w, 0, 0, 0));
+      std::swap(v, w);
+      if (it % 16 == 15) {
+        CKS(dot1(ctx, v, v, n3, ctx->sc + MS_TMP0));
+        LK(1, launch_vec_op(VOP_SCALE_RSQRT, n3, v, v, nullptr, nullptr, ctx->sc + MS_TMP0, s));
+      }
+    }
     CKS(stencil<double>(ctx, ST_APPLY, l, v, nullptr, nullptr, w, 0, 0, 0));
-    LK(1, launch_vec_op(VOP_MUL, n3, w, w, lv.invD64, nullptr, nullptr, s));
-    CKS(dot1(ctx, w, w, n3, ctx->sc + MS_TMP0));
-    LK(1, launch_vec_op(VOP_SCALE_RSQRT, n3, v, w, nullptr, nullptr, ctx->sc + MS_TMP0, s));
-  }
-  CKS(stencil<double>(ctx, ST_APPLY, l, v, nullptr, nullptr, w, 0, 0, 0));
-  CKS(dot1(ctx, v, w, n3, ctx->sc + MS_TMP0));
-  LK(1, launch_vec_op(VOP_MUL, n3, w, v, lv.diag, nullptr, nullptr, s));
-  CKS(dot1(ctx, v, w, n3, ctx->sc + MS_TMP1));
-  double num = 0.0, den = 0.0;
-  CKS(read_scalar(ctx, ctx->sc + MS_TMP0, &num));
-  CKS(read_scalar(ctx, ctx->sc + MS_TMP1, &den));
-  *lam = num / den;
-  return AGCA_OK;
+    CKS(dot1(ctx, v, w, n3, ctx->sc + kRaySlot + 2 * l));
+    LK(1, launch_vec_op(VOP_MUL, n3, w, v, lv.diag, nullptr, nullptr, s));
+    return dot1(ctx, v, w, n3, ctx->sc + kRaySlot + 2 * l + 1);
+  };
+  const agca_status st = run();
+  if (scratch) lv.hedge = nullptr;
+  return st;
 }
 
 bool valid_level(const agca_ctx* ctx, int l) { return l >= 1 && l <= ctx->L; }
@@ -1409,8 +1415,7 @@ void build_cycle(agca_batch* b, std::vector<BatchStep>& steps, const std::vector
 // K x for every problem (x_p, y_p: Stokes vectors), FP32 compute when low
 void build_stokes(agca_batch* b, std::vector<BatchStep>& steps, const std::vector<const double*>& x,
                   const std::vector<double*>& y, bool low, bool skip_done) {
-  const int P = b->n;
-  std::vector<XferTask> pro, rst;
+  std::vector<XferTask> pro, grad, div;
   std::vector<StencilTask<double, double>> t64;
   std::vector<StencilTask<double, float>> t32;
   for (int p : b->members) {
@@ -1418,15 +1423,18 @@ void build_stokes(agca_batch* b, std::vector<BatchStep>& steps, const std::vecto
     const Level& lf = c->lev[c->L];
     const int64_t n3 = 3 * lf.V;
     const double* sc = skip_done ? c->sc : nullptr;
-    XferTask a{};
-    a.nf = lf.n;
-    a.ncomp = 1;
-    a.mask = 0;
-    a.count = lf.V;
-    a.src = x[p] + n3;
-    a.dst = c->qfine;
-    a.sc = sc;
-    pro.push_back(a);
+    auto xfer = [&](int ncomp, int64_t count, const void* src, void* dst) {
+      XferTask a{};
+      a.nf = lf.n;
+      a.ncomp = ncomp;
+      a.mask = 0;
+      a.count = count;
+      a.src = src;
+      a.dst = dst;
+      a.sc = sc;
+      return a;
+    };
+    pro.push_back(xfer(1, lf.V, x[p] + n3, c->qfine));
     if (low) {
       StencilTask<double, float> tk{};
       tk.op = op32(c, c->L);
@@ -1436,33 +1444,28 @@ void build_stokes(agca_batch* b, std::vector<BatchStep>& steps, const std::vecto
       tk.a.out2 = c->sfine;
       tk.sc = sc;
       t32.push_back(tk);
+      div.push_back(xfer(1, c->Vp, c->sfine, y[p] + n3));
+      div.back().scale = -1.0;
     } else {
       StencilTask<double, double> tk{};
       tk.op = op64(c, c->L);
       tk.a.x = x[p];
-      tk.a.q = c->qfine;
       tk.a.out = y[p];
-      tk.a.out2 = c->sfine;
       tk.sc = sc;
       t64.push_back(tk);
+      grad.push_back(xfer(3, lf.V, c->qfine, y[p]));
+      div.push_back(xfer(3, c->Vp, x[p], y[p] + n3));
     }
-    XferTask r{};
-    r.nf = lf.n;
-    r.ncomp = 1;
-    r.mask = 0;
-    r.scale = -1.0;
-    r.count = c->Vp;
-    r.src = c->sfine;
-    r.dst = y[p] + n3;
-    r.sc = sc;
-    rst.push_back(r);
   }
   push_xfer(b, steps, XK_PROLONG, pro, 0);
-  if (low)
+  if (low) {
     push_stencil<double, float>(b, steps, ST_STOKES, false, t32, 2);
-  else
-    push_stencil<double, double>(b, steps, ST_STOKES, false, t64, 0);
-  push_xfer(b, steps, XK_RESTRICT, rst, 0);
+    push_xfer(b, steps, XK_RESTRICT, div, 0);
+  } else {
+    push_stencil<double, double>(b, steps, ST_APPLY, false, t64, 0);
+    push_xfer(b, steps, XK_GRADIENT, grad, 0);
+    push_xfer(b, steps, XK_DIVERGENCE, div, 0);
+  }
 }
 
 // One MINRES iteration for every problem at buffer parity par (see minres_impl).
@@ -1672,7 +1675,7 @@ agca_status agca_set_viscosity(agca_ctx* ctx, const double* eta_dev) {
   if (!ctx->ws) return ctx->fail(AGCA_ESTATE, "bind the workspace first");
   Level& lf = ctx->lev[ctx->L];
   CK(cudaMemcpyAsync(lf.mean, eta_dev, lf.E * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
-  if (lf.hedge) LK(1, launch_edge_records(lf.n, lf.mean, lf.hedge, ctx->stream));
+  if (lf.hedge) LK(1, launch_edge_records(lf.n, lf.mean, nullptr, lf.hedge, ctx->stream));
   ctx->have_eta = true;
   ctx->flagged = ctx->setup_done = false;
   return AGCA_OK;
@@ -1785,8 +1788,7 @@ agca_status agca_setup(agca_ctx* ctx) {
     if (mixed) {
       LK(1, launch_stencil_to_f32(lc.n_sv, lc.sten64, lc.sten32, lc.sscale32, s));
     } else {
-      LK(1, launch_masked_coef<double>(lc.E, lc.mean, lc.fidx, lc.coefm, s));
-      LK(1, launch_edge_records(lc.n, lc.coefm, lc.hedge, s));
+      LK(1, launch_edge_records(lc.n, lc.mean, lc.fidx, lc.hedge, s));
     }
   }
   for (int l = 1; l <= L; ++l) {
@@ -1797,7 +1799,6 @@ agca_status agca_setup(agca_ctx* ctx) {
         LK(1, launch_masked_coef<float>(lv.E, lv.mean, lv.fidx, lv.mean32, s));
       else
         LK(1, launch_d2f(lv.mean, lv.mean32, lv.E, s));
-      if (l < L) LK(1, launch_gca_to_f32(lv.n_flag, lv.list, lv.mx, lv.gca64, lv.gca32, lv.gscale32, s));
     }
     LK(1, launch_diag(op64(ctx, l), lv.diag, lv.invD64, mixed ? lv.invD32 : nullptr, s));
   }
@@ -1808,9 +1809,12 @@ agca_status agca_setup(agca_ctx* ctx) {
   LK(1, launch_trinv(ctx->cfac, ctx->mc, ctx->ainv, ctx->linv, s));
   LK(1, launch_coarse_inverse(ctx->linv, ctx->mc, ctx->ainv, s));
   CKS(check_status(ctx, "agca_setup"));
-  for (int l = 2; l <= L; ++l) CKS(power_lambda(ctx, l, &ctx->lev[l].lambda));
-  LK(1, launch_pressure_mass(ctx->lev[L].n / 2, ctx->lev[L].mean, ctx->pmass, ctx->pmass_inv, s));
+  for (int l = 2; l <= L; ++l) CKS(power_lambda(ctx, l));
+  LK(2, launch_pressure_mass(ctx->lev[L].n / 2, ctx->lev[L].mean, ctx->kv[KV_Z], ctx->pmass, ctx->pmass_inv, s));
+  double ray[64];
+  CK(cudaMemcpyAsync(ray, ctx->sc, sizeof(ray), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  for (int l = 2; l <= L; ++l) ctx->lev[l].lambda = ray[kRaySlot + 2 * l] / ray[kRaySlot + 2 * l + 1];
   ctx->setup_done = true;
   return AGCA_OK;
 }

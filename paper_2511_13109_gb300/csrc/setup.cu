@@ -5,6 +5,8 @@
 // vector.  All arithmetic here is FP64.
 #include <math.h>
 
+#include <algorithm>
+
 #include "agca_internal.cuh"
 #include "device_ops.cuh"
 
@@ -206,56 +208,79 @@ __global__ void compact_scatter_kernel(const uint8_t* flags, int64_t n, const in
   }
 }
 
-// One block per flagged parent; thread r*12+s computes entry (r, s) of
-// A_parent = sum_k (I3 x p_k)^T C_k (I3 x p_k).
-__global__ void galerkin_kernel(const RefineTables rt, int nc, const int32_t* __restrict__ list, int nf, int child_finest,
-                                const double* __restrict__ coef_f, const int32_t* __restrict__ fidx_f,
-                                const double* __restrict__ gca_f, double* __restrict__ gca_c) {
+// Galerkin matrices A_parent = sum_k (I3 x p_k)^T C_k (I3 x p_k) of the flagged
+// parents, entry (r, s) by thread r*12+s of a block that walks the list.  The
+// weights p are 0, 1/2 or 1 and the rediscretised child matrix is w_k K' with
+// an integer K', so such a child needs one integer (4 P^T K' P)(r, s), one table
+// lookup and one FP64 multiply-add; a stored child one multiply-add per pair of
+// non-zero weights.  Converting those integers to FP64 in the loop (conversions
+// issue at the FP64 rate) took 2.78 + 2.08 ms for the 15,635 + 11,291 parents of
+// the two finest coarse levels of 8 spheres at 64^3.
+__global__ void galerkin_kernel(const RefineTables rt, int nc, int64_t n_flag, const int32_t* __restrict__ list, int nf,
+                                int child_finest, const double* __restrict__ coef_f,
+                                const int32_t* __restrict__ fidx_f, const double* __restrict__ gca_f,
+                                double* __restrict__ gca_c) {
   grid_dep_entry();
-  __shared__ int8_t kp[6][144];
+  constexpr int R = 128;  // |4 P^T K' P| <= 4 * 16 * max |K'| is far below
+  __shared__ int8_t kp[6][144], pk[6][8][16], ct[6][8];
+  __shared__ double quarter[2 * R + 1];  // i / 4
   __shared__ double w[8];
   __shared__ int32_t kf[8];
-  const int fpar = blockIdx.x;
-  const int64_t e = list[fpar];
-  const int t = (int)(e % 6);
-  const int64_t cube = e / 6;
-  const int I = (int)(cube % nc), J = (int)((cube / nc) % nc), K = (int)(cube / ((int64_t)nc * nc));
   const double h6f = 1.0 / (6.0 * nf);
-  for (int i = threadIdx.x; i < 6 * 144; i += blockDim.x) kp[i / 144][i % 144] = 0;
-  __syncthreads();
+  for (int i = threadIdx.x; i < 2 * R + 1; i += blockDim.x) quarter[i] = 0.25 * (double)(i - R);
+  for (int i = threadIdx.x; i < 6 * 8 * 16; i += blockDim.x) {
+    const int t = i / 128, k = (i / 16) % 8, q = i % 16;
+    pk[t][k][q] = rt.pk2[t][k][q / 4][q % 4];
+    if (q == 0) ct[t][k] = rt.child[t][k][3];
+  }
   if (threadIdx.x < 144) {
     const int r = threadIdx.x / 12, s = threadIdx.x % 12;
 #pragma unroll
     for (int tt = 0; tt < 6; ++tt) kp[tt][threadIdx.x] = (int8_t)kuhn_kprime(tt, r, s);
   }
-  if (threadIdx.x < 8) {
-    const int k = threadIdx.x;
-    const int64_t f = child_id(rt, nf, I, J, K, t, k);
-    w[k] = coef_f[f] * h6f;
-    kf[k] = (child_finest || fidx_f == nullptr) ? -1 : fidx_f[f];
-  }
-  __syncthreads();
-  if (threadIdx.x >= 144) return;
   const int r = threadIdx.x / 12, s = threadIdx.x % 12;
   const int c = r >> 2, a = r & 3, d = s >> 2, b = s & 3;
-  double acc = 0.0;
-  for (int k = 0; k < 8; ++k) {
-    const int tc = rt.child[t][k][3];
-    const int8_t* p = &rt.pk2[t][k][0][0];  // p[i*4 + j] = 2 lambda_j at child vertex i
-    const double* M = kf[k] >= 0 ? gca_f + (int64_t)kf[k] * 144 : nullptr;
-    for (int i = 0; i < 4; ++i) {
-      const int pia = p[i * 4 + a];
-      if (pia == 0) continue;
-      for (int j = 0; j < 4; ++j) {
-        const int pjb = p[j * 4 + b];
-        if (pjb == 0) continue;
-        const int rr = c * 4 + i, ss = d * 4 + j;
-        const double cv = M ? M[rr * 12 + ss] : w[k] * (double)kp[tc][rr * 12 + ss];
-        acc = fma(0.25 * (double)(pia * pjb), cv, acc);
+  for (int64_t fpar = blockIdx.x; fpar < n_flag; fpar += gridDim.x) {
+    const int64_t e = list[fpar];
+    const int t = (int)(e % 6);
+    __syncthreads();  // tables written; w and kf of the last parent read
+    if (threadIdx.x < 8) {
+      const int64_t cube = e / 6;
+      const int I = (int)(cube % nc), J = (int)((cube / nc) % nc), K = (int)(cube / ((int64_t)nc * nc));
+      const int64_t f = child_id(rt, nf, I, J, K, t, threadIdx.x);
+      w[threadIdx.x] = coef_f[f] * h6f;
+      kf[threadIdx.x] = (child_finest || fidx_f == nullptr) ? -1 : fidx_f[f];
+    }
+    __syncthreads();
+    if (threadIdx.x >= 144) continue;
+    double acc = 0.0;
+    for (int k = 0; k < 8; ++k) {
+      const int8_t* p = pk[t][k];  // p[i*4 + j] = 2 lambda_j at child vertex i
+      int pa[4], pb[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        pa[i] = p[i * 4 + a];
+        pb[i] = p[i * 4 + b];
+      }
+      if (kf[k] < 0) {
+        const int8_t* M = kp[ct[t][k]] + c * 4 * 12 + d * 4;
+        int m = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) m += pa[i] * pb[j] * M[i * 12 + j];
+        acc = fma(quarter[m + R], w[k], acc);
+      } else {
+        const double* M = gca_f + (int64_t)kf[k] * 144 + c * 4 * 12 + d * 4;
+        for (int i = 0; i < 4; ++i) {
+          if (pa[i] == 0) continue;
+          for (int j = 0; j < 4; ++j)
+            if (pb[j] != 0) acc = fma(quarter[pa[i] * pb[j] + R], M[i * 12 + j], acc);
+        }
       }
     }
+    gca_c[fpar * 144 + threadIdx.x] = acc;
   }
-  gca_c[(int64_t)fpar * 144 + threadIdx.x] = acc;
 }
 
 __global__ void diag_kernel(const LevelOp<double> op, double* diag, double* invD64, float* invD32) {
@@ -266,7 +291,8 @@ __global__ void diag_kernel(const LevelOp<double> op, double* diag, double* invD
   if (v >= V) return;
   const int i = (int)(v % nv), j = (int)((v / nv) % nv), k = (int)(v / ((int64_t)nv * nv));
   const bool inner = i > 0 && j > 0 && k > 0 && i < n && j < n && k < n;
-  double dg[3] = {0.0, 0.0, 0.0};
+  // the entries of K' are small integers: one multiply-add per tetrahedron and component, h/6 once
+  double dg[3] = {0.0, 0.0, 0.0}, gg[3] = {0.0, 0.0, 0.0};
   if (inner) {
 #pragma unroll
     for (int o = 0; o < 8; ++o) {
@@ -278,16 +304,18 @@ __global__ void diag_kernel(const LevelOp<double> op, double* diag, double* invD
         if (a < 0) continue;
         const int64_t e = 6 * cube + t;
         const int32_t f = op.fidx ? op.fidx[e] : -1;
+        if (f >= 0) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const int r = c * 4 + a;
-          if (f >= 0)
-            dg[c] += op.gca[(int64_t)f * 144 + r * 13];
-          else
-            dg[c] += op.coef[e] * op.h6 * (double)kuhn_kprime(t, r, r);
+          for (int c = 0; c < 3; ++c) gg[c] += op.gca[(int64_t)f * 144 + (c * 4 + a) * 13];
+        } else {
+          const double q = op.coef[e];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) dg[c] = fma(q, (double)kuhn_kprime(t, c * 4 + a, c * 4 + a), dg[c]);
         }
       }
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) dg[c] = fma(op.h6, dg[c], gg[c]);
   }
   for (int c = 0; c < 3; ++c) {
     diag[c * V + v] = dg[c];
@@ -295,17 +323,6 @@ __global__ void diag_kernel(const LevelOp<double> op, double* diag, double* invD
     invD64[c * V + v] = inv;
     if (invD32) invD32[c * V + v] = (float)inv;
   }
-}
-
-__global__ void gca_to_f32_kernel(int64_t n_flag, const int32_t* list, const double* mx, const double* gca64,
-                                  float* gca32, float* scale32) {
-  grid_dep_entry();
-  const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (id >= n_flag * 144) return;
-  const int64_t f = id / 144;
-  const double s = mx[list[f]];
-  gca32[id] = (float)(gca64[id] / s);
-  if (id % 144 == 0) scale32[f] = (float)s;
 }
 
 __global__ void d2f_kernel(const double* __restrict__ in, float* __restrict__ out, int64_t n,
@@ -431,7 +448,23 @@ __global__ void __launch_bounds__(32 * kCoarseWarps)
   coarse_solve_rows<T>(n, ainv, r, z, sm, blockIdx.x, gridDim.x);
 }
 
-__global__ void pressure_mass_kernel(const RefineTables rt, int np, const double* __restrict__ eta_f, double* pmass, double* pmass_inv) {
+// mean of 1/eta over the 8 children of each pressure element (np cubes per axis)
+__global__ void inverse_viscosity_kernel(const RefineTables rt, int np, const double* __restrict__ eta_f,
+                                         double* __restrict__ w) {
+  grid_dep_entry();
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= nelems(np)) return;
+  const int t = (int)(e % 6);
+  const int64_t cube = e / 6;
+  const int I = (int)(cube % np), J = (int)((cube / np) % np), K = (int)(cube / ((int64_t)np * np));
+  double q[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) q[k] = 1.0 / eta_f[child_id(rt, 2 * np, I, J, K, t, k)];
+  w[e] = (((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]))) * 0.125;
+}
+
+// lumped pressure mass from the element weights w of inverse_viscosity_kernel
+__global__ void pressure_mass_kernel(int np, const double* __restrict__ w, double* pmass, double* pmass_inv) {
   grid_dep_entry();
   const int nv = np + 1;
   const int64_t V = nverts(np);
@@ -439,17 +472,16 @@ __global__ void pressure_mass_kernel(const RefineTables rt, int np, const double
   if (v >= V) return;
   const int i = (int)(v % nv), j = (int)((v / nv) % nv), k = (int)(v / ((int64_t)nv * nv));
   const double vol4 = 1.0 / (24.0 * (double)np * np * np);  // |T| / 4
-  const int nf = 2 * np;
   double acc = 0.0;
+#pragma unroll
   for (int o = 0; o < 8; ++o) {
     const int ci = i - (o & 1), cj = j - ((o >> 1) & 1), ck = k - ((o >> 2) & 1);
     if (ci < 0 || cj < 0 || ck < 0 || ci >= np || cj >= np || ck >= np) continue;
+    const int64_t cube = ci + (int64_t)np * (cj + (int64_t)np * ck);
+#pragma unroll
     for (int t = 0; t < 6; ++t) {
       if (corner_local(t, o) < 0) continue;
-      double q[8];
-      for (int kk = 0; kk < 8; ++kk) q[kk] = 1.0 / eta_f[child_id(rt, nf, ci, cj, ck, t, kk)];
-      const double w = (((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]))) * 0.125;
-      acc += w * vol4;
+      acc += __ldg(w + 6 * cube + t) * vol4;
     }
   }
   pmass[v] = acc;
@@ -520,22 +552,14 @@ cudaError_t launch_galerkin(int nc, int64_t n_flag, const int32_t* list, int nf,
                             const double* coef_f, const int32_t* fidx_f, const double* gca_f, double* gca_c,
                             cudaStream_t s) {
   if (n_flag == 0) return cudaSuccess;
-  KL(launch_k(galerkin_kernel, dim3((unsigned)n_flag), dim3(160), 0, s,
-     refine_tables(), nc, list, nf, child_finest ? 1 : 0, coef_f, fidx_f, gca_f, gca_c));
+  KL(launch_k(galerkin_kernel, dim3((unsigned)std::min<int64_t>(n_flag, 12 * 152)), dim3(160), 0, s,
+     refine_tables(), nc, n_flag, list, nf, child_finest ? 1 : 0, coef_f, fidx_f, gca_f, gca_c));
   return cudaGetLastError();
 }
 
 cudaError_t launch_diag(const LevelOp<double>& op, double* diag, double* invD64, float* invD32, cudaStream_t s) {
   const int64_t V = nverts(op.n);
   KL(launch_k(diag_kernel, dim3(blocks_for(V, 128)), dim3(128), 0, s, op, diag, invD64, invD32));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gca_to_f32(int64_t n_flag, const int32_t* list, const double* mx, const double* gca64,
-                              float* gca32, float* scale32, cudaStream_t s) {
-  if (n_flag == 0) return cudaSuccess;
-  KL(launch_k(gca_to_f32_kernel, dim3(blocks_for(n_flag * 144, 256)), dim3(256), 0, s,
-     n_flag, list, mx, gca64, gca32, scale32));
   return cudaGetLastError();
 }
 
@@ -583,10 +607,12 @@ cudaError_t launch_coarse_solve(int n, const double* ainv, const T* r, T* z, cud
 template cudaError_t launch_coarse_solve<float>(int, const double*, const float*, float*, cudaStream_t);
 template cudaError_t launch_coarse_solve<double>(int, const double*, const double*, double*, cudaStream_t);
 
-cudaError_t launch_pressure_mass(int np, const double* eta_f, double* pmass, double* pmass_inv, cudaStream_t s) {
-  const int64_t V = nverts(np);
-  KL(launch_k(pressure_mass_kernel, dim3(blocks_for(V, 128)), dim3(128), 0, s,
-     refine_tables(), np, eta_f, pmass, pmass_inv));
+cudaError_t launch_pressure_mass(int np, const double* eta_f, double* work, double* pmass, double* pmass_inv,
+                                 cudaStream_t s) {
+  KL(launch_k(inverse_viscosity_kernel, dim3(blocks_for(nelems(np), 256)), dim3(256), 0, s, refine_tables(), np, eta_f,
+              work));
+  KL(launch_k(pressure_mass_kernel, dim3(blocks_for(nverts(np), 128)), dim3(128), 0, s, np, (const double*)work, pmass,
+              pmass_inv));
   return cudaGetLastError();
 }
 

@@ -5,13 +5,13 @@
 // caching allocator or a fixed pool they must not bypass), or code in a loop
 // where an allocation's latency or possible failure is not acceptable.  For
 // them agca_stokes_apply_static computes y = K x on the finest grid without a
-// context, a workspace or any allocation: the two fine-grid scratch fields the
-// operator needs (the prolongated pressure P p and the divergence B_f u) live
-// in a fixed file-scope device array that every GPU loading this library
-// holds until the process exits.
+// context, a workspace or any allocation: the fine-grid scratch field the
+// operator needs (the prolongated pressure P p) lives in a fixed file-scope
+// device array that every GPU loading this library holds until the process
+// exits.
 //
 // Limit: N <= kStaticMaxN pressure cubes per axis (the scratch holds
-// 2 * (2N+1)^3 doubles, 4.4 MB at the limit).
+// (2N+1)^3 doubles, 2.2 MB at the limit).
 #include <cuda.h>  // driver types only: the two driver calls are resolved at run time
 
 #include <mutex>
@@ -23,8 +23,8 @@ namespace {
 constexpr int kStaticMaxN = 32;
 constexpr int64_t kStaticMaxV = (int64_t)(2 * kStaticMaxN + 1) * (2 * kStaticMaxN + 1) * (2 * kStaticMaxN + 1);
 
-// [0, V): fine-grid pressure P p; [kStaticMaxV, kStaticMaxV + V): B_f u
-static __device__ __align__(256) double g_stokes_scratch[2 * kStaticMaxV];
+// [0, V): fine-grid pressure P p
+static __device__ __align__(256) double g_stokes_scratch[kStaticMaxV];
 
 // The scratch array's device address belongs to a CUDA context (a module is
 // loaded per context), so it is cached per context, keyed by the context's
@@ -122,21 +122,18 @@ extern "C" agca_status agca_stokes_apply_static(int N, const double* eta_dev, co
   const int n = 2 * N;
   const int64_t V = nverts(n);
   double* qfine = scratch;
-  double* sfine = scratch + kStaticMaxV;
-  // the same three launches as agca_stokes_apply, with the scratch above;
-  // every scratch entry used is written before it is read
+  // the launches of agca_stokes_apply, with the scratch above; every scratch
+  // entry used is written before it is read
   if (launch_prolong<double>(n, 1, false, false, x_dev + 3 * V, qfine, s) != cudaSuccess) return AGCA_ECUDA;
   LevelOp<double> op{};
   op.n = n;
   op.h6 = 1.0 / (6.0 * n);
-  op.hq = 1.0 / (6.0 * (double)n * n);
   op.coef = eta_dev;
   StencilArgs<double> a{};
   a.x = x_dev;
-  a.q = qfine;
   a.out = y_dev;
-  a.out2 = sfine;
-  if (launch_stencil<double, double>(ST_STOKES, op, a, s) != cudaSuccess) return AGCA_ECUDA;
-  if (launch_restrict<double>(n, 1, false, -1.0, sfine, y_dev + 3 * V, s) != cudaSuccess) return AGCA_ECUDA;
+  if (launch_stencil<double, double>(ST_APPLY, op, a, s) != cudaSuccess) return AGCA_ECUDA;
+  if (launch_gradient(n, qfine, y_dev, s) != cudaSuccess) return AGCA_ECUDA;
+  if (launch_divergence(N, x_dev, y_dev + 3 * V, s) != cudaSuccess) return AGCA_ECUDA;
   return AGCA_OK;
 }

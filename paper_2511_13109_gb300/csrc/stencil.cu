@@ -1,8 +1,8 @@
 // Matrix-free operator application on a Kuhn cube grid, one cube per thread:
-// the Stokes operator (FP64 vectors; FP64 or FP32 arithmetic) and its pressure
-// coupling, and the FP64 operator of mixed contexts, which keep no coefficient
-// records (levels of more than kPointMaxN cubes per axis); the per-cube element
-// action (cube_dca) is in device_ops.cuh.  The dispatch of launch_stencil at
+// the Stokes operator on FP64 vectors with FP32 arithmetic, and the FP64
+// operator of mixed contexts, which keep no coefficient records (levels of more
+// than kPointMaxN cubes per axis); the per-cube element actions are in
+// device_ops.cuh.  The dispatch of launch_stencil at
 // the end of the file sends every other operator application to its kernel.
 //
 // Tiling (GB300): a CTA of BX x BY threads owns a (BX-1) x (BY-1) column of
@@ -144,7 +144,6 @@ __device__ __forceinline__ void stencil_block(const LevelOp<T>& op, const Stenci
     }
   };
   auto issue_coef = [&](int kc) {
-    if (MODE == ST_STOKES_B) return;  // no viscous part: the coefficients are not read
     T* dst = cfs + (((kc - zs) & 1) * NT + tid) * 6;
     const bool ok = cube_xy && kc >= 0 && kc < n;
     const T* src = op.coef + (ok ? 6 * (cube_col + kc * n * n) : 0);
@@ -197,11 +196,6 @@ __device__ __forceinline__ void stencil_block(const LevelOp<T>& op, const Stenci
     const bool out_k = owner && k >= z0;
     const bool inner = out_k && inner_xy && k > 0 && k < n;
     const int vo = vcol + k * plane;
-    double eb[3] = {0.0, 0.0, 0.0};  // STOKES_B: A u, read early so that its latency overlaps the compute
-    if (MODE == ST_STOKES_B && inner) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) eb[c] = __ldg(a.b + (c * V + vo));
-    }
     int32_t f[6];
     if constexpr (COARSE) {
       if (cube_xy && k >= 0 && k < n) {
@@ -275,8 +269,6 @@ __device__ __forceinline__ void stencil_block(const LevelOp<T>& op, const Stenci
         cube_dca<T, NC>(Xl, Xh, cf, Y);
       } else if constexpr (MODE == ST_STOKES) {
         cube_stokes<T>(Xl, Xh, cf, op.hq, Y);
-      } else if constexpr (MODE == ST_STOKES_B) {
-        cube_stokes_b<T>(Xl, Xh, op.hq, Y);
       } else {
         cube_dca<T, NC>(Xl, Xh, cf, Y);
       }
@@ -327,7 +319,7 @@ __device__ __forceinline__ void stencil_block(const LevelOp<T>& op, const Stenci
         for (int c = 0; c < 3; ++c) {
           const int i = c * V + vo;
           const double y = (double)yk[c];
-          a.out[i] = inner ? (MODE == ST_STOKES_B ? eb[c] + y : y) : 0.0;
+          a.out[i] = inner ? y : 0.0;
         }
         if (NC == 4) a.out2[vo] = (double)yk[NC - 1];  // (B_f u) on every fine vertex
       }
@@ -348,7 +340,13 @@ __device__ __forceinline__ void stencil_block(const LevelOp<T>& op, const Stenci
 }
 
 constexpr int BY = 8;          // block rows of the wide tiles
-constexpr int kMinBlocks = 2;  // resident blocks per SM
+// resident blocks per SM: FP32 arithmetic fits three, but not with a batch's
+// task fields in registers
+template <typename T>
+__host__ __device__ constexpr int min_blocks() {
+  return sizeof(T) == 4 ? 3 : 2;
+}
+constexpr int kBatchBlocks = 2;
 
 // Two tile classes: wide tiles (32 x BY threads, 31 x (BY-1) owned vertices)
 // cover the first gxw * 31 vertex columns, narrow tiles (8 x 4BY threads,
@@ -373,7 +371,7 @@ __device__ __forceinline__ void stencil_tile(const LevelOp<T>& op, const Stencil
 }
 
 template <typename T, int MODE, bool COARSE>
-__global__ void __launch_bounds__(32 * BY, kMinBlocks)
+__global__ void __launch_bounds__(32 * BY, min_blocks<T>())
     stencil_kernel(const LevelOp<T> op, const StencilArgs<double> a, const int zch, const int gxw, const int gyw,
                    const int gxn, const int x0n) {
   grid_dep_entry();
@@ -385,7 +383,7 @@ __global__ void __launch_bounds__(32 * BY, kMinBlocks)
 // independent problems; every CTA walks the flattened (problem, tile) work
 // list, skipping problems whose MINRES has converged.
 template <typename T, int MODE>
-__global__ void __launch_bounds__(32 * BY, kMinBlocks)
+__global__ void __launch_bounds__(32 * BY, kBatchBlocks)
     stencil_batch_kernel(const StencilTask<double, T>* __restrict__ tasks, const int ntasks, const int64_t ntiles) {
   grid_dep_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -473,14 +471,18 @@ cudaError_t launch_stencil_batch(int mode, bool coarse, const StencilTask<TS, T>
   if constexpr (std::is_same<T, double>::value) {
     if (edge_form_step<TS, T>(mode, coarse)) return launch_stencil_edge_batch<T>(mode, tasks, ntasks, ntiles, s);
   }
-  if (mode != ST_STOKES || coarse) return cudaErrorInvalidValue;
-  static bool set[64] = {};
-  KL(allow_smem(stencil_batch_kernel<T, ST_STOKES>, tile_smem<T, ST_STOKES>(), set));
-  int dev = 0, sms = 152;
-  KL(cudaGetDevice(&dev));
-  KL(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  return launch_k(stencil_batch_kernel<T, ST_STOKES>, dim3((unsigned)std::min<int64_t>(ntiles, (int64_t)sms * kMinBlocks)),
-                  dim3(32 * BY), tile_smem<T, ST_STOKES>(), s, tasks, ntasks, ntiles);
+  if constexpr (std::is_same<T, float>::value) {
+    if (mode != ST_STOKES || coarse) return cudaErrorInvalidValue;
+    static bool set[64] = {};
+    KL(allow_smem(stencil_batch_kernel<T, ST_STOKES>, tile_smem<T, ST_STOKES>(), set));
+    int dev = 0, sms = 152;
+    KL(cudaGetDevice(&dev));
+    KL(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const dim3 grid((unsigned)std::min<int64_t>(ntiles, (int64_t)sms * kBatchBlocks));
+    return launch_k(stencil_batch_kernel<T, ST_STOKES>, grid, dim3(32 * BY), tile_smem<T, ST_STOKES>(), s, tasks, ntasks,
+                    ntiles);
+  }
+  return cudaErrorInvalidValue;
 }
 template cudaError_t launch_stencil_batch<double, double>(int, bool, const StencilTask<double, double>*, int, int64_t,
                                                           cudaStream_t);
@@ -495,19 +497,20 @@ cudaError_t launch_stencil(int mode, const LevelOp<T>& op, const StencilArgs<TS>
                            const TileCfg* cfg) {
   const int zch = cfg ? cfg->zch : 0;
   if constexpr (std::is_same<TS, T>::value) {
-    if (op.n <= kPointMaxN && mode != ST_STOKES && mode != ST_STOKES_B)
+    if (op.n <= kPointMaxN && mode != ST_STOKES)
       return launch_stencil_point<T>(mode, op, a, s);
   }
   if constexpr (std::is_same<TS, float>::value) {
     return launch_stencil_f32(mode, op, a, s, zch);
   } else {
     if constexpr (std::is_same<T, double>::value) {
-      if (op.hedge && mode != ST_STOKES && mode != ST_STOKES_B) return launch_stencil_edge<T>(mode, op, a, s, zch);
+      if (op.hedge && mode != ST_STOKES) return launch_stencil_edge<T>(mode, op, a, s, zch);
       if (mode == ST_APPLY)
         return op.fidx ? launch_tiles<T, ST_APPLY, true>(op, a, s, zch) : launch_tiles<T, ST_APPLY, false>(op, a, s, zch);
-      if (mode == ST_STOKES_B) return launch_tiles<T, ST_STOKES_B, false>(op, a, s, zch);
     }
-    if (mode == ST_STOKES) return launch_tiles<T, ST_STOKES, false>(op, a, s, zch);
+    if constexpr (std::is_same<T, float>::value) {
+      if (mode == ST_STOKES) return launch_tiles<T, ST_STOKES, false>(op, a, s, zch);
+    }
     return cudaErrorInvalidValue;
   }
 }

@@ -241,8 +241,8 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
     if (inner) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        if (MODE != ST_APPLY) eb[c] = __ldg(a.b + c * V + vo);
-        if (MODE == ST_CHEB_FIRST || MODE == ST_CHEB_STEP || MODE == ST_CHEB_PRE) ed[c] = __ldg(a.invD + c * V + vo);
+        if (MODE != ST_APPLY && MODE != ST_POWER) eb[c] = __ldg(a.b + c * V + vo);
+        if (MODE == ST_CHEB_FIRST || MODE == ST_CHEB_STEP || PRE || MODE == ST_POWER) ed[c] = __ldg(a.invD + c * V + vo);
         if (MODE == ST_CHEB_STEP) ep[c] = a.xprev[c * V + vo];
         if (MODE == ST_CHEB_FIRST || MODE == ST_CHEB_STEP || PRE) xo[c] = __ldg(a.x + c * V + vo);
       }
@@ -308,8 +308,9 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
         const T sum = ((fl[c] - Fx[c]) + (fd - Fy[c])) + (fzp[c] - Fz[c]);
         T o = T(0);
         if (inner) {
-          if (MODE == ST_APPLY) {
+          if (MODE == ST_APPLY || MODE == ST_POWER) {
             o = op.sten ? fma(op.h6, sum, gs[c]) : op.h6 * sum;
+            if (MODE == ST_POWER) o = ed[c] * o;
           } else {
             const T r = op.sten ? eb[c] - fma(op.h6, sum, gs[c]) : fma(-op.h6, sum, eb[c]);  // b - A x
             if (MODE == ST_RESID) o = r;
@@ -370,8 +371,9 @@ __global__ void __launch_bounds__(ENT, edge_min_blocks<T, MODE>())
 
 // the coefficient record of every vertex, rec[q][v], q < EREC (edge_record)
 template <typename T>
-__global__ void edge_record_kernel(const int n, const T* __restrict__ eta, T* __restrict__ rec) {
-  grid_dep_entry();  // the coefficients may come from the kernel before (masked_coef_kernel)
+__global__ void edge_record_kernel(const int n, const T* __restrict__ eta, const int32_t* __restrict__ fidx,
+                                   T* __restrict__ rec) {
+  grid_dep_entry();  // the coefficients may come from the kernel before
   const int nv = n + 1;
   const int64_t V = (int64_t)nv * nv * nv;
   const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -380,7 +382,8 @@ __global__ void edge_record_kernel(const int n, const T* __restrict__ eta, T* __
   auto c = [&](int di, int dj, int dk, int t) -> T {
     const int ci = i + di, cj = j + dj, ck = k + dk;
     if (ci < 0 || cj < 0 || ck < 0 || ci >= n || cj >= n || ck >= n) return T(0);
-    return __ldg(eta + 6 * (ci + (int64_t)n * (cj + (int64_t)n * ck)) + t);
+    const int64_t e = 6 * (ci + (int64_t)n * (cj + (int64_t)n * ck)) + t;
+    return fidx && __ldg(fidx + e) >= 0 ? T(0) : __ldg(eta + e);
   };
   T r[EREC];
   edge_record<T>(c(0, 0, 0, 0), c(0, 0, 0, 1), c(0, 0, 0, 2), c(0, 0, 0, 3), c(0, 0, 0, 4), c(0, 0, 0, 5),
@@ -427,11 +430,11 @@ TileGrid edge_tiles(int n, int zch_req, int slots) {
 }
 
 template <typename T>
-cudaError_t launch_edge_records(int n, const T* eta, T* rec, cudaStream_t s) {
+cudaError_t launch_edge_records(int n, const T* eta, const int32_t* fidx, T* rec, cudaStream_t s) {
   const int64_t V = nverts(n);
-  return launch_k(edge_record_kernel<T>, dim3((unsigned)((V + 255) / 256)), dim3(256), 0, s, n, eta, rec);
+  return launch_k(edge_record_kernel<T>, dim3((unsigned)((V + 255) / 256)), dim3(256), 0, s, n, eta, fidx, rec);
 }
-template cudaError_t launch_edge_records<double>(int, const double*, double*, cudaStream_t);
+template cudaError_t launch_edge_records<double>(int, const double*, const int32_t*, double*, cudaStream_t);
 
 template <typename T>
 cudaError_t launch_stencil_edge(int mode, const LevelOp<T>& op, const StencilArgs<T>& a, cudaStream_t s, int zch_req) {
@@ -457,6 +460,7 @@ cudaError_t launch_stencil_edge(int mode, const LevelOp<T>& op, const StencilArg
     case ST_RESID: AGCA_ELAUNCH(ST_RESID); break;
     case ST_CHEB_FIRST: AGCA_ELAUNCH(ST_CHEB_FIRST); break;
     case ST_CHEB_STEP: AGCA_ELAUNCH(ST_CHEB_STEP); break;
+    case ST_POWER: AGCA_ELAUNCH(ST_POWER); break;
     case ST_CHEB_PRE: AGCA_ELAUNCH(ST_CHEB_PRE); break;
     default: return cudaErrorInvalidValue;
   }
@@ -485,6 +489,7 @@ cudaError_t launch_stencil_edge_batch(int mode, const StencilTask<T, T>* tasks, 
                 ntasks, ntiles));                                                                             \
   } while (0)
   switch (mode) {
+    case ST_APPLY: AGCA_EBLAUNCH(ST_APPLY); break;
     case ST_RESID: AGCA_EBLAUNCH(ST_RESID); break;
     case ST_CHEB_FIRST: AGCA_EBLAUNCH(ST_CHEB_FIRST); break;
     case ST_CHEB_STEP: AGCA_EBLAUNCH(ST_CHEB_STEP); break;

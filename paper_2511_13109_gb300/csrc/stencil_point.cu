@@ -94,8 +94,8 @@ __device__ __forceinline__ void stencil_point(const LevelOp<T>& op, const Stenci
   const int vo = (e < 3 ? e : 0) * V + v;
   T eb = T(0), ed = T(0), ep = T(0), xo = T(0);
   if (out_lane && inner) {
-    if (MODE != ST_APPLY) eb = __ldg(a.b + vo);
-    if (MODE == ST_CHEB_FIRST || MODE == ST_CHEB_STEP || PRE) ed = __ldg(a.invD + vo);
+    if (MODE != ST_APPLY && MODE != ST_POWER) eb = __ldg(a.b + vo);
+    if (MODE == ST_CHEB_FIRST || MODE == ST_CHEB_STEP || PRE || MODE == ST_POWER) ed = __ldg(a.invD + vo);
     if (MODE == ST_CHEB_STEP) ep = a.xprev[vo];
     if (MODE == ST_CHEB_FIRST || MODE == ST_CHEB_STEP) xo = __ldg(a.x + vo);
   }
@@ -187,8 +187,9 @@ __device__ __forceinline__ void stencil_point(const LevelOp<T>& op, const Stenci
   const T gs = e == 0 ? g[0] : (e == 1 ? g[1] : g[2]);
   T o = T(0);
   if (inner) {
-    if (MODE == ST_APPLY) {
+    if (MODE == ST_APPLY || MODE == ST_POWER) {
       o = op.sten ? fma(op.h6, sum, gs) : op.h6 * sum;
+      if (MODE == ST_POWER) o = ed * o;
     } else {
       const T r = op.sten ? eb - fma(op.h6, sum, gs) : fma(-op.h6, sum, eb);  // b - A x
       if (MODE == ST_RESID) o = r;
@@ -283,6 +284,12 @@ cudaError_t launch_stencil_point(int mode, const LevelOp<T>& op, const StencilAr
     case ST_CHEB_FIRST: AGCA_PLAUNCH(ST_CHEB_FIRST); break;
     case ST_CHEB_STEP: AGCA_PLAUNCH(ST_CHEB_STEP); break;
     case ST_CHEB_PRE: AGCA_PLAUNCH(ST_CHEB_PRE); break;
+    case ST_POWER:
+      if constexpr (sizeof(T) == 8) {
+        AGCA_PLAUNCH(ST_POWER);
+        break;
+      }
+      [[fallthrough]];
     default: return cudaErrorInvalidValue;
   }
 #undef AGCA_PLAUNCH
@@ -296,6 +303,7 @@ cudaError_t launch_stencil_point_batch(int mode, const StencilTask<T, T>* tasks,
   constexpr int COEF = sizeof(T) == 8 ? PC_RECORD : PC_PLAIN;  // batched FP64 steps belong to FP64 contexts
   const dim3 grid(point_blocks(max_n), (unsigned)ntasks), block(PT);
   switch (mode) {
+    case ST_APPLY: KL(launch_k(stencil_point_batch_kernel<T, ST_APPLY, COEF>, grid, block, 0, s, tasks)); break;
     case ST_RESID: KL(launch_k(stencil_point_batch_kernel<T, ST_RESID, COEF>, grid, block, 0, s, tasks)); break;
     case ST_CHEB_FIRST:
       KL(launch_k(stencil_point_batch_kernel<T, ST_CHEB_FIRST, COEF>, grid, block, 0, s, tasks));

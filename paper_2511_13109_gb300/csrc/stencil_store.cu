@@ -143,7 +143,6 @@ cudaError_t launch_masked_coef(int64_t E, const double* mean, const int32_t* fid
   return cudaGetLastError();
 }
 
-template cudaError_t launch_masked_coef<double>(int64_t, const double*, const int32_t*, double*, cudaStream_t);
 template cudaError_t launch_masked_coef<float>(int64_t, const double*, const int32_t*, float*, cudaStream_t);
 
 }  // namespace agca
