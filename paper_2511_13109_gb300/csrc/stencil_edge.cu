@@ -34,19 +34,22 @@
 // launch_gather (at 128^3 cubes with 8 spheres one thread walking a vertex's 135
 // values held its block up: FP64 cycle at 64^3 pressure cubes 3.18 -> 2.62 ms).
 //
-// Tiling: a CTA of 32 x 8 threads, thread (tx, ty) <-> vertex column
-// (x0 - 1 + tx, y0 - 1 + ty), marches a chunk of z-planes.  Per plane k it
-// stages the x plane k + 2 (cp.async, one plane ahead), forms the edge
-// differences of plane k + 1 for its
-// (34 x 10)-vertex tile, computes the three fluxes of its vertex's forward
-// edges from the differences of planes k - 1..k + 1 and its vertex's
-// coefficient record, exchanges the x and y fluxes (warp shuffle, shared
-// memory; the z flux stays in registers for the next plane), and the threads
-// with tx, ty >= 1 finish their vertex (owner-computes: no atomics; every
-// vertex sums its fluxes in one fixed order, whatever the tile shape or
-// z-chunk).  Staging copies whole tile rows per warp: a row's geometry is
-// warp-uniform and each lane's column bounds are fixed for the block, so a
-// copy costs an address add and a predicate.
+// Tiling: a CTA owns 32 x 8 vertex columns starting at vertex (1, 1), one per
+// thread, and marches a chunk of z-planes; n a multiple of 32 then wastes no
+// lane.  Per plane k it stages the x plane k + 2 (cp.async, one plane ahead),
+// forms the edge differences of plane k + 1 for its (34 x 10)-vertex tile,
+// computes the three fluxes of its vertex's forward edges from the differences
+// of planes k - 1..k + 1 and its vertex's coefficient record, and exchanges the
+// x and y fluxes (warp shuffle, shared memory; the z flux stays in registers
+// for the next plane).  The fluxes that enter the tile are computed beside: the
+// y edges below it by warp 0, the x edges left of it by 8 lanes of warp 7.
+// Owner-computes: no atomics; every vertex sums its fluxes in one fixed order,
+// whatever the tile shape or z-chunk.  Tiles of 31 x 7 owned vertices, whose
+// halo threads supplied those fluxes, computed 72 FP64 instructions a vertex
+// and 1.09 vertices for each one of 257^3; these compute 69 and 1.  Staging
+// copies whole tile rows per warp: a row's geometry is warp-uniform and each
+// lane's column bounds are fixed for the block, so a copy costs an address add
+// and a predicate.
 #include <algorithm>
 
 #include "agca_internal.cuh"
@@ -57,7 +60,7 @@ namespace agca {
 namespace {
 
 constexpr int EBX = 32, EBY = 8, ENT = EBX * EBY, NWARP = ENT / 32;
-constexpr int XW = EBX + 3, XH = EBY + 3, XT = XW * XH;  // x tile: vertices (x0-2 .., y0-2 ..)
+constexpr int XW = EBX + 3, XH = EBY + 3, XT = XW * XH;  // x tile: vertices (x0-1 .., y0-1 ..)
 constexpr int DW = EBX + 2, DH = EBY + 2, DT = DW * DH;  // edge-difference tile
 constexpr int DRING = 84;                                // halo entries of the difference tile
 static_assert(EBX == 32, "a tile row is one warp");
@@ -71,9 +74,9 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;
 
 template <typename T, int MODE>
 __host__ __device__ constexpr size_t edge_smem_elems() {
-  // x ring [3][3][XT], difference ring [3][6][DT], y-flux exchange [3][ENT]:
-  // 82 KB in FP64
-  return (size_t)3 * 3 * XT + (size_t)3 * 6 * DT + (size_t)3 * ENT;
+  // x ring [3][3][XT], difference ring [3][6][DT], y fluxes entering each row
+  // [3][EBY + 1][32], x fluxes entering column 0 [3][EBY]: 84 KB in FP64
+  return (size_t)3 * 3 * XT + (size_t)3 * 6 * DT + (size_t)3 * (ENT + 32) + (size_t)3 * EBY;
 }
 // resident CTAs per SM (shared memory and the 128-register budget)
 template <typename T, int MODE>
@@ -115,6 +118,14 @@ __device__ __forceinline__ void edge_record(T v0, T v1, T v2, T v3, T v4, T v5, 
   r[23] = v5 + mx1, r[24] = my3 + mxy0, r[25] = v4, r[26] = mxy2;
 }
 
+// 2 h through the exponent, off the FP64 pipe, for the edge sums h >= 0 (zero
+// and values beyond 2^1022 take the product)
+__device__ __forceinline__ double twice(double h) {
+  const int hi = __double2hiint(h);
+  if ((unsigned)hi - 0x00100000u < 0x7fc00000u) return __hiloint2double(hi + 0x00100000, __double2loint(h));
+  return 2.0 * h;
+}
+
 // difference-tile coordinates of halo entry r (0..83): rows 0 and DH-1, then
 // columns 0 and DW-1 of the rows between
 __device__ __forceinline__ void ring_entry(int r, int& i, int& j) {
@@ -134,23 +145,29 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
                                                    T* __restrict__ sm) {
   const int n = op.n, nv = n + 1, V = nv * nv * nv;
   const int tx = tid & (EBX - 1), ty = tid >> 5;  // lane, warp
-  const int gx = x0 - 1 + tx, gy = y0 - 1 + ty;
-  const int za = bz * zch, zb = min(za + zch, nv);
-  const bool owner = tx >= 1 && ty >= 1 && gx <= n && gy <= n;
-  const bool inner_xy = gx > 0 && gx < n && gy > 0 && gy < n;
+  const int gx = x0 + tx, gy = y0 + ty;
+  const int za = 1 + bz * zch, zb = min(za + zch, nv);
+  const bool owner = gx <= n && gy <= n;
+  const bool inner_xy = gx < n && gy < n;  // gx, gy >= 1
+  // Dirichlet entries of column 0 and row 0: one per thread of warps 2, 3 and 4
+  int ze = -1;
+  if (x0 == 1 && ty == 2 && tx < EBY && y0 + tx <= n) ze = nv * (y0 + tx);
+  if (y0 == 1 && ty == 3 && gx <= n) ze = gx;
+  if (x0 == 1 && y0 == 1 && ty == 4 && tx == 0) ze = 0;
   constexpr bool PRE = MODE == ST_CHEB_PRE;
 
   T* xs = sm;                                    // [3][3][XT]
   T* ds = xs + 3 * 3 * XT;                       // [3][6][DT]
-  T* fy = ds + 3 * 6 * DT;                       // [3][ENT]
+  T* fy = ds + 3 * 6 * DT;                       // [3][EBY + 1][32]
+  T* fxl = fy + 3 * (ENT + 32);                  // [3][EBY]
 
   const int zs = za - 2;  // planes zs + i use ring slot i mod 3
   auto slot = [&](int p) { return (p - zs) % 3; };
 
-  // this lane's columns of the x tile (x0 - 2 + tx, and x0 + 30 + tx for the
+  // this lane's columns of the x tile (x0 - 1 + tx, and x0 + 31 + tx for the
   // last XW - 32 lanes): interior in x?  Dirichlet and outside vertices read 0
-  const bool inx0 = x0 - 2 + tx > 0 && x0 - 2 + tx < n;
-  const bool inx1 = tx < XW - 32 && x0 + 30 + tx > 0 && x0 + 30 + tx < n;
+  const bool inx0 = x0 - 1 + tx > 0 && x0 - 1 + tx < n;
+  const bool inx1 = tx < XW - 32 && x0 + 31 + tx < n;
   // stage x plane p: warp ty copies the rows r = ty, ty + 8, ..
   // of the [3][XH] rows of the tile
   auto issue_x = [&](int p) {
@@ -158,9 +175,9 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
     const bool zin = p > 0 && p < n;
     for (int r = ty; r < 3 * XH; r += NWARP) {
       const int c = r / XH, j = r - c * XH;
-      const int vy = y0 - 2 + j;
+      const int vy = y0 - 1 + j;
       const bool rin = zin && vy > 0 && vy < n;
-      const int g = c * V + (x0 - 2) + nv * (vy + nv * p);  // valid when rin (then vy >= 1, so g >= 0)
+      const int g = c * V + (x0 - 1) + nv * (vy + nv * p);
       const int e = c * XT + j * XW + tx;
       const bool ok0 = rin && inx0, ok1 = rin && inx1;
       const int g0 = ok0 ? g + tx : 0, g1 = ok1 ? g + 32 + tx : 0;
@@ -190,10 +207,14 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
     dp[ZX * DT + e] = d[2][0];
     dp[ZY * DT + e] = d[2][1];
   };
-  auto compute_d = [&](int p, T (&own)[3][3]) {
+  // (halo: the on-axis difference of the entering flux that warp 0 or 7 computes
+  // for plane p: the y edge below the thread's column, the x edge left of row tx)
+  auto compute_d = [&](int p, T (&own)[3][3], T& halo) {
     const T* xl = xs + slot(p) * 3 * XT;
     const T* xh = xs + slot(p + 1) * 3 * XT;
     T* dp = ds + slot(p) * 6 * DT;
+    if (ty == 0) halo = xl[XT + XW + tx + 1] - xl[XT + tx + 1];
+    if (ty == EBY - 1 && tx < EBY) halo = xl[(tx + 1) * XW + 1] - xl[(tx + 1) * XW];
     diffs_at(xl, xh, tx + 1, ty + 1, own);
     store_d(dp, tx + 1, ty + 1, own);
     if (tid < DRING) {
@@ -212,9 +233,9 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
   cp_commit();
   cp_wait_all();
   __syncthreads();
-  T dcur[3][3], dnext[3][3];
-  compute_d(zs, dnext);
-  compute_d(zs + 1, dcur);
+  T dcur[3][3], dnext[3][3], hcur = T(0), hnext = T(0);
+  compute_d(zs, dnext, hnext);
+  compute_d(zs + 1, dcur, hcur);
   __syncthreads();
   issue_x(za + 1);
   cp_commit();
@@ -225,18 +246,19 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
   for (int k = za - 1; k < zb; ++k) {
     cp_wait_all();
     __syncthreads();  // x plane k+2 staged; ring slots of k-2 free
-    compute_d(k + 1, dnext);
+    compute_d(k + 1, dnext, hnext);
     __syncthreads();  // differences of plane k+1 visible; x slot of plane k free
     if (k + 1 < zb) issue_x(k + 3);
     cp_commit();
 
     // own coefficient record and epilogue inputs of plane k, read early
-    const bool kin = k >= 0 && k <= n && gx >= 0 && gx <= n && gy >= 0 && gy <= n;
+    const bool kin = k <= n && gx <= n && gy <= n;
     const int vo = kin ? gx + nv * (gy + nv * k) : 0;
     const T* rec = op.hedge + vo;
     auto R = [&](int q) { return kin ? __ldg(rec + (int64_t)q * V) : T(0); };
-    const bool out_k = owner && k >= za;
-    const bool inner = out_k && inner_xy && k > 0 && k < n;
+    const bool full = k >= za;  // the halo plane za - 1 supplies only the z fluxes of plane za
+    const bool out_k = owner && full;
+    const bool inner = out_k && inner_xy && k < n;
     T eb[3] = {T(0), T(0), T(0)}, ed[3] = {T(0), T(0), T(0)}, ep[3] = {T(0), T(0), T(0)}, xo[3] = {T(0), T(0), T(0)};
     if (inner) {
 #pragma unroll
@@ -253,42 +275,60 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
     const T* dp = ds + slot(k + 1) * 6 * DT;  // plane k+1
     auto D = [&](const T* p, int comp, int di, int dj) { return p[comp * DT + (J + dj) * DW + I + di]; };
 
-    // the halo row (warp 0) supplies only the y fluxes of row 1, and the
-    // halo plane za-1 only the z fluxes of plane za (warp-uniform branches)
-    const bool need_x = ty != 0 && k >= za, need_y = k >= za, need_z = ty != 0;
     T Fx[3] = {T(0), T(0), T(0)}, Fy[3] = {T(0), T(0), T(0)}, Fz[3] = {T(0), T(0), T(0)};
     // flux component c != m of edge m: the H_m term and the four distinct
     // c-edge differences around the edge, weighted by the record (EREC order)
-    auto flux = [&](int q0, T hd, T da, T db, T dc, T dd) {
+    auto flux = [&](auto R, int q0, T hd, T da, T db, T dc, T dd) {
       T f = fma(da, R(q0), hd);
       f = fma(db, R(q0 + 1), f);
       f = fma(dc, R(q0 + 2), f);
       return fma(dd, R(q0 + 3), f);
     };
-    if (need_x) {  // x edge (v, v + ex)
-      const T h = R(0);
-      Fx[0] = T(2) * (h * dcur[0][0]);
-      Fx[1] = flux(3, h * dcur[0][1], D(d0, YX, 1, 0), D(d0, YX, 0, -1), D(dp, YX, 1, 0), D(dm, YX, 0, -1));
-      Fx[2] = flux(7, h * dcur[0][2], D(d0, ZX, 1, 0), D(dm, ZX, 0, 0), D(d0, ZX, 1, 1), D(dm, ZX, 0, -1));
+    if (full) {
+      // x edge (v, v + ex)
+      T h = R(0);
+      Fx[0] = twice(h) * dcur[0][0];
+      Fx[1] = flux(R, 3, h * dcur[0][1], D(d0, YX, 1, 0), D(d0, YX, 0, -1), D(dp, YX, 1, 0), D(dm, YX, 0, -1));
+      Fx[2] = flux(R, 7, h * dcur[0][2], D(d0, ZX, 1, 0), D(dm, ZX, 0, 0), D(d0, ZX, 1, 1), D(dm, ZX, 0, -1));
+      // y edge (v, v + ey)
+      h = R(1);
+      Fy[1] = twice(h) * dcur[1][1];
+      Fy[0] = flux(R, 11, h * dcur[1][0], D(d0, XY, 0, 1), D(d0, XY, -1, 0), D(dp, XY, 0, 1), D(dm, XY, -1, 0));
+      Fy[2] = flux(R, 15, h * dcur[1][2], D(d0, ZY, 0, 1), D(dm, ZY, 0, 0), D(d0, ZY, 1, 1), D(dm, ZY, -1, 0));
     }
-    if (need_y) {  // y edge (v, v + ey)
-      const T h = R(1);
-      Fy[1] = T(2) * (h * dcur[1][1]);
-      Fy[0] = flux(11, h * dcur[1][0], D(d0, XY, 0, 1), D(d0, XY, -1, 0), D(dp, XY, 0, 1), D(dm, XY, -1, 0));
-      Fy[2] = flux(15, h * dcur[1][2], D(d0, ZY, 0, 1), D(dm, ZY, 0, 0), D(d0, ZY, 1, 1), D(dm, ZY, -1, 0));
-    }
-    if (need_z) {  // z edge (v, v + ez)
+    {  // z edge (v, v + ez)
       const T h = R(2);
-      Fz[2] = T(2) * (h * dcur[2][2]);
-      Fz[0] = flux(19, h * dcur[2][0], D(dp, XZ, 0, 0), D(d0, XZ, -1, 0), D(dp, XZ, 0, 1), D(d0, XZ, -1, -1));
-      Fz[1] = flux(23, h * dcur[2][1], D(dp, YZ, 0, 0), D(d0, YZ, 0, -1), D(dp, YZ, 1, 0), D(d0, YZ, -1, -1));
+      Fz[2] = twice(h) * dcur[2][2];
+      Fz[0] = flux(R, 19, h * dcur[2][0], D(dp, XZ, 0, 0), D(d0, XZ, -1, 0), D(dp, XZ, 0, 1), D(d0, XZ, -1, -1));
+      Fz[1] = flux(R, 23, h * dcur[2][1], D(dp, YZ, 0, 0), D(d0, YZ, 0, -1), D(dp, YZ, 1, 0), D(d0, YZ, -1, -1));
+    }
+    if (full && ty == 0) {  // y edges from row -1 into row 0
+      const T* rb = op.hedge + (kin ? vo - nv : 0);
+      auto Rb = [&](int q) { return kin ? __ldg(rb + (int64_t)q * V) : T(0); };
+      auto B = [&](const T* p, int comp, int di, int dj) { return p[comp * DT + (J - 1 + dj) * DW + I + di]; };
+      const T h = Rb(1);
+      fy[32 + ENT + tx] = twice(h) * hcur;
+      fy[tx] = flux(Rb, 11, h * B(d0, YX, 0, 0), B(d0, XY, 0, 1), B(d0, XY, -1, 0), B(dp, XY, 0, 1), B(dm, XY, -1, 0));
+      fy[2 * (32 + ENT) + tx] =
+          flux(Rb, 15, h * B(d0, YZ, 0, 0), B(d0, ZY, 0, 1), B(dm, ZY, 0, 0), B(d0, ZY, 1, 1), B(dm, ZY, -1, 0));
+    }
+    if (full && ty == EBY - 1 && tx < EBY) {  // x edges from column -1 into column 0: lane <-> row
+      const bool in = k <= n && y0 + tx <= n;
+      const T* rb = op.hedge + (in ? x0 - 1 + nv * (y0 + tx + nv * k) : 0);
+      auto Rb = [&](int q) { return in ? __ldg(rb + (int64_t)q * V) : T(0); };
+      auto B = [&](const T* p, int comp, int di, int dj) { return p[comp * DT + (tx + 1 + dj) * DW + di]; };
+      const T h = Rb(0);
+      fxl[tx] = twice(h) * hcur;
+      fxl[EBY + tx] = flux(Rb, 3, h * B(d0, XY, 0, 0), B(d0, YX, 1, 0), B(d0, YX, 0, -1), B(dp, YX, 1, 0), B(dm, YX, 0, -1));
+      fxl[2 * EBY + tx] =
+          flux(Rb, 7, h * B(d0, XZ, 0, 0), B(d0, ZX, 1, 0), B(dm, ZX, 0, 0), B(d0, ZX, 1, 1), B(dm, ZX, 0, -1));
     }
     // the x edge ending at v belongs to lane tx - 1 of the same row (a warp)
     T fl[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       fl[c] = __shfl_up_sync(0xffffffffu, Fx[c], 1);
-      fy[c * ENT + tid] = Fy[c];
+      fy[c * (32 + ENT) + 32 + tid] = Fy[c];
     }
     __syncthreads();  // y fluxes of the tile visible
     T gs[3] = {T(0), T(0), T(0)};  // stored-Galerkin part (coarse levels, launch_gather)
@@ -302,7 +342,8 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
     if (out_k) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const T fd = fy[c * ENT + tid - EBX];  // flux of the y edge ending at v
+        const T fd = fy[c * (32 + ENT) + tid];  // flux of the y edge ending at v
+        if (tx == 0) fl[c] = fxl[c * EBY + ty];
         // the DCA fluxes carry the unscaled coefficient (y = (h/6) sum), the
         // stencils the scaled operator
         const T sum = ((fl[c] - Fx[c]) + (fd - Fy[c])) + (fzp[c] - Fz[c]);
@@ -325,9 +366,21 @@ __device__ __forceinline__ void stencil_edge_block(const LevelOp<T>& op, const S
           a.out[c * V + vo] = o;
       }
     }
+    // Dirichlet entries: plane 0, column 0 and row 0
+    auto zero = [&](int v) {
+      for (int c = 0; c < 3; ++c) {
+        if (a.out64)
+          a.out64[c * V + v] = 0.0;
+        else
+          a.out[c * V + v] = T(0);
+      }
+    };
+    if (k == 0 && owner) zero(vo);
+    if (ze >= 0 && (full || k == 0)) zero(ze + k * nv * nv);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       fzp[c] = Fz[c];
+      hcur = hnext;
 #pragma unroll
       for (int q = 0; q < 3; ++q) dcur[c][q] = dnext[c][q];
     }
@@ -341,7 +394,7 @@ __global__ void __launch_bounds__(ENT, edge_min_blocks<T, MODE>())
   grid_dep_entry();
   extern __shared__ __align__(16) unsigned char sm_edge_raw[];
   const int t = blockIdx.x;
-  stencil_edge_block<T, MODE>(op, a, zch, (t % gxw) * (EBX - 1), (t / gxw) * (EBY - 1), blockIdx.y, threadIdx.x,
+  stencil_edge_block<T, MODE>(op, a, zch, 1 + (t % gxw) * EBX, 1 + (t / gxw) * EBY, blockIdx.y, threadIdx.x,
                               reinterpret_cast<T*>(sm_edge_raw));
 }
 
@@ -363,7 +416,7 @@ __global__ void __launch_bounds__(ENT, edge_min_blocks<T, MODE>())
     if (tk.sc && tk.sc[MS_DONE] != 0.0) continue;  // converged problem
     const int local = (int)(it - tk.tile0), per = tk.tg.per_z();
     const int bz = local / per, t = local % per;
-    stencil_edge_block<T, MODE>(tk.op, tk.a, tk.tg.zch, (t % tk.tg.gxw) * (EBX - 1), (t / tk.tg.gxw) * (EBY - 1),
+    stencil_edge_block<T, MODE>(tk.op, tk.a, tk.tg.zch, 1 + (t % tk.tg.gxw) * EBX, 1 + (t / tk.tg.gxw) * EBY,
                                 bz, threadIdx.x, reinterpret_cast<T*>(sm_edge_raw));
     __syncthreads();  // the shared-memory rings are reused by the next tile
   }
@@ -396,13 +449,12 @@ __global__ void edge_record_kernel(const int n, const T* __restrict__ eta, const
 
 }  // namespace
 
+// tiles over the vertices 1 .. n of each axis (coordinate 0 is written by the first tile)
 TileGrid edge_tiles(int n, int zch_req, int slots) {
-  const int nv = n + 1;
   TileGrid g;
-  g.gxw = (nv + EBX - 2) / (EBX - 1);
-  g.gyw = (nv + EBY - 2) / (EBY - 1);
-  g.gxn = g.gyn = 0;
-  g.x0n = 31 * g.gxw;
+  g.gxw = (n + EBX - 1) / EBX;
+  g.gyw = (n + EBY - 1) / EBY;
+  g.x0n = n + 1;
   const int per = g.per_z();
   int zch = zch_req;
   if (zch <= 0) {
@@ -411,9 +463,9 @@ TileGrid edge_tiles(int n, int zch_req, int slots) {
     // plus about one plane's worth of prologue); longer chunks win ties
     const int sl = slots > 0 ? slots : 2 * 152;
     double best = 1e300;
-    for (int gz = 1; gz <= nv; ++gz) {
-      const int z = (nv + gz - 1) / gz;
-      if ((nv + z - 1) / z != gz) continue;  // the same chunk as a smaller gz
+    for (int gz = 1; gz <= n; ++gz) {
+      const int z = (n + gz - 1) / gz;
+      if ((n + z - 1) / z != gz) continue;  // the same chunk as a smaller gz
       const double waves = (double)(((int64_t)per * gz + sl - 1) / sl);
       const double cost = waves * (z + 1.0);
       if (cost < best - 1e-9) {
@@ -422,9 +474,8 @@ TileGrid edge_tiles(int n, int zch_req, int slots) {
       }
     }
   }
-  zch = std::max(zch, 1);
-  zch = std::min(zch, nv);
-  g.gz = (nv + zch - 1) / zch;
+  zch = std::min(std::max(zch, 1), n);
+  g.gz = (n + zch - 1) / zch;
   g.zch = zch;
   return g;
 }
