@@ -324,8 +324,8 @@ cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s, 
 cudaError_t launch_f2d(const float* in, double* out, int64_t n, cudaStream_t s);
 cudaError_t launch_coarse_assemble(const LevelOp<double>& op, double* dense, cudaStream_t s);
 cudaError_t launch_cholesky(double* a, int m, int* status, cudaStream_t s);
-cudaError_t launch_trinv(const double* l, int m, double* linv_cm, double* linv_rm, cudaStream_t s);
-cudaError_t launch_coarse_inverse(const double* linv_rm, int m, double* ainv, cudaStream_t s);
+cudaError_t launch_trinv(const double* l, int m, double* linv, cudaStream_t s);
+cudaError_t launch_coarse_inverse(const double* linv, int m, double* ainv, cudaStream_t s);
 template <typename T>
 cudaError_t launch_coarse_solve(int n, const double* ainv, const T* r, T* z, cudaStream_t s);
 // work: 6 np^3 doubles of scratch

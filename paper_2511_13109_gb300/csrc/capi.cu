@@ -1806,7 +1806,7 @@ agca_status agca_setup(agca_ctx* ctx) {
   LK(1, launch_coarse_assemble(op64(ctx, 1), ctx->cdense, s));
   CK(cudaMemcpyAsync(ctx->cfac, ctx->cdense, (size_t)ctx->mc * ctx->mc * sizeof(double), cudaMemcpyDeviceToDevice, s));
   LK(1, launch_cholesky(ctx->cfac, ctx->mc, ctx->status, s));
-  LK(1, launch_trinv(ctx->cfac, ctx->mc, ctx->ainv, ctx->linv, s));
+  LK(1, launch_trinv(ctx->cfac, ctx->mc, ctx->linv, s));
   LK(1, launch_coarse_inverse(ctx->linv, ctx->mc, ctx->ainv, s));
   CKS(check_status(ctx, "agca_setup"));
   for (int l = 2; l <= L; ++l) CKS(power_lambda(ctx, l));

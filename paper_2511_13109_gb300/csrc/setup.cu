@@ -215,7 +215,7 @@ __global__ void compact_scatter_kernel(const uint8_t* flags, int64_t n, const in
 // lookup and one FP64 multiply-add; a stored child one multiply-add per pair of
 // non-zero weights.  Converting those integers to FP64 in the loop (conversions
 // issue at the FP64 rate) took 2.78 + 2.08 ms for the 15,635 + 11,291 parents of
-// the two finest coarse levels of 8 spheres at 64^3.
+// the two finest coarse levels of 8 spheres at 64^3; now 0.11 ms a level on average.
 __global__ void galerkin_kernel(const RefineTables rt, int nc, int64_t n_flag, const int32_t* __restrict__ list, int nf,
                                 int child_finest, const double* __restrict__ coef_f,
                                 const int32_t* __restrict__ fidx_f, const double* __restrict__ gca_f,
@@ -339,12 +339,6 @@ __global__ void x1_kernel(const double* __restrict__ b, const FirstIterate<doubl
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     fi.x1[i] = fi.s2 * __ldg(fi.invD + i) * b[i];
 }
-__global__ void f2d_kernel(const float* in, double* out, int64_t n) {
-  grid_dep_entry();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = (double)in[i];
-}
-
 // dense level-1 operator on interior DoFs: row (c, iv), col (d, jv)
 __global__ void coarse_assemble_kernel(const LevelOp<double> op, double* dense) {
   grid_dep_entry();
@@ -383,11 +377,19 @@ __global__ void coarse_assemble_kernel(const LevelOp<double> op, double* dense) 
   dense[id] = acc;
 }
 
-// in-place lower Cholesky of a row-major m x m SPD matrix, one block
-__global__ void cholesky_kernel(double* a, int m, int* status) {
+// in-place lower Cholesky of a row-major m x m SPD matrix, one block; kept in
+// shared memory while it fits (SM; the usual 81 unknowns take 52 KB)
+template <bool SM>
+__global__ void cholesky_kernel(double* g, int m, int* status) {
   grid_dep_entry();
+  extern __shared__ double sm_chol[];
   __shared__ double piv;
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  double* a = SM ? sm_chol : g;
+  if (SM) {
+    for (int i = tid; i < m * m; i += nt) a[i] = g[i];
+    __syncthreads();
+  }
   for (int k = 0; k < m; ++k) {
     if (tid == 0) {
       double dk = a[(int64_t)k * m + k];
@@ -407,24 +409,28 @@ __global__ void cholesky_kernel(double* a, int m, int* status) {
     }
     __syncthreads();
   }
+  if (SM)
+    for (int i = tid; i < m * m; i += nt) g[i] = a[i];
 }
 
-// X = L^-1 (lower), one thread per column; writes column- and row-major copies
-// (the column-major one is scratch: the inverse takes its place)
-__global__ void trinv_kernel(const double* l, int m, double* xcm, double* xrm) {
+// X = L^-1 (lower, row-major), one warp per column: each row's sum over the
+// entries above is spread over the lanes, the column kept in shared memory
+__global__ void __launch_bounds__(32) trinv_kernel(const double* __restrict__ l, int m, double* __restrict__ x) {
   grid_dep_entry();
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= m) return;
-  for (int i = 0; i < j; ++i) {
-    xcm[(int64_t)j * m + i] = 0.0;
-    xrm[(int64_t)i * m + j] = 0.0;
-  }
+  extern __shared__ double sm_col[];
+  const int j = blockIdx.x, lane = threadIdx.x;
+  for (int i = lane; i < j; i += 32) x[(int64_t)i * m + j] = 0.0;
   for (int i = j; i < m; ++i) {
-    double s = (i == j) ? 1.0 : 0.0;
-    for (int k = j; k < i; ++k) s -= l[(int64_t)i * m + k] * xcm[(int64_t)j * m + k];
-    const double x = s / l[(int64_t)i * m + i];
-    xcm[(int64_t)j * m + i] = x;
-    xrm[(int64_t)i * m + j] = x;
+    double s = 0.0;
+    for (int k = j + lane; k < i; k += 32) s = fma(l[(int64_t)i * m + k], sm_col[k], s);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    const double v = ((i == j ? 1.0 : 0.0) - s) / l[(int64_t)i * m + i];
+    if (lane == 0) {
+      sm_col[i] = v;
+      x[(int64_t)i * m + j] = v;
+    }
+    __syncwarp();
   }
 }
 
@@ -571,11 +577,6 @@ cudaError_t launch_x1(const double* b, const FirstIterate<double>& fi, int64_t n
   KL(launch_k(x1_kernel, dim3(1216), dim3(256), 0, s, b, fi, n));
   return cudaGetLastError();
 }
-cudaError_t launch_f2d(const float* in, double* out, int64_t n, cudaStream_t s) {
-  KL(launch_k(f2d_kernel, dim3(1216), dim3(256), 0, s, in, out, n));
-  return cudaGetLastError();
-}
-
 cudaError_t launch_coarse_assemble(const LevelOp<double>& op, double* dense, cudaStream_t s) {
   const int64_t ni = op.n - 1, m = 3 * ni * ni * ni;
   KL(launch_k(coarse_assemble_kernel, dim3(blocks_for(m * m, 128)), dim3(128), 0, s, op, dense));
@@ -583,17 +584,20 @@ cudaError_t launch_coarse_assemble(const LevelOp<double>& op, double* dense, cud
 }
 
 cudaError_t launch_cholesky(double* a, int m, int* status, cudaStream_t s) {
-  KL(launch_k(cholesky_kernel, dim3(1), dim3(1024), 0, s, a, m, status));
-  return cudaGetLastError();
+  const size_t bytes = (size_t)m * m * sizeof(double);
+  if (bytes <= 200 * 1024) {
+    KL(cudaFuncSetAttribute(cholesky_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    return launch_k(cholesky_kernel<true>, dim3(1), dim3(1024), bytes, s, a, m, status);
+  }
+  return launch_k(cholesky_kernel<false>, dim3(1), dim3(1024), 0, s, a, m, status);
 }
 
-cudaError_t launch_trinv(const double* l, int m, double* linv_cm, double* linv_rm, cudaStream_t s) {
-  KL(launch_k(trinv_kernel, dim3(blocks_for(m, 64)), dim3(64), 0, s, l, m, linv_cm, linv_rm));
-  return cudaGetLastError();
+cudaError_t launch_trinv(const double* l, int m, double* linv, cudaStream_t s) {
+  return launch_k(trinv_kernel, dim3((unsigned)m), dim3(32), (size_t)m * sizeof(double), s, l, m, linv);
 }
 
-cudaError_t launch_coarse_inverse(const double* linv_rm, int m, double* ainv, cudaStream_t s) {
-  KL(launch_k(coarse_inverse_kernel, dim3(blocks_for(m, 128), (unsigned)m), dim3(128), 0, s, linv_rm, m, ainv));
+cudaError_t launch_coarse_inverse(const double* linv, int m, double* ainv, cudaStream_t s) {
+  KL(launch_k(coarse_inverse_kernel, dim3(blocks_for(m, 128), (unsigned)m), dim3(128), 0, s, linv, m, ainv));
   return cudaGetLastError();
 }
 

@@ -90,17 +90,27 @@ __global__ void stencil_assemble_kernel(const int n, const int64_t n_sv, const i
     for (int d = 0; d < 3; ++d) out[o * 9 + c * 3 + d] = acc[o][d];
 }
 
+// one warp per stencil (a thread walking its 135 values took 128 us a level whatever its size)
 __global__ void stencil_to_f32_kernel(const int64_t n_sv, const double* __restrict__ s64, float* __restrict__ s32,
                                       float* __restrict__ scale) {
   grid_dep_entry();
-  const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (s >= n_sv) return;
   const double* in = s64 + s * 135;
-  double mx = 0.0;
-  for (int q = 0; q < 135; ++q) mx = fmax(mx, fabs(in[q]));
+  double v[5], mx = 0.0;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    v[i] = lane + 32 * i < 135 ? in[lane + 32 * i] : 0.0;
+    mx = fmax(mx, fabs(v[i]));
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
   const double sc = mx > 0.0 ? mx : 1.0;
-  for (int q = 0; q < 135; ++q) s32[s * 135 + q] = (float)(in[q] / sc);
-  scale[s] = (float)sc;
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+    if (lane + 32 * i < 135) s32[s * 135 + lane + 32 * i] = (float)(v[i] / sc);
+  if (lane == 0) scale[s] = (float)sc;
 }
 
 // DCA coefficient with the flagged elements zeroed (their part is in the stencils)
@@ -133,7 +143,7 @@ cudaError_t launch_stencil_assemble(int n, int64_t n_sv, const int32_t* slist, c
 
 cudaError_t launch_stencil_to_f32(int64_t n_sv, const double* s64, float* s32, float* scale, cudaStream_t s) {
   if (n_sv == 0) return cudaSuccess;
-  KL(launch_k(stencil_to_f32_kernel, dim3(nblocks(n_sv, 128)), dim3(128), 0, s, n_sv, s64, s32, scale));
+  KL(launch_k(stencil_to_f32_kernel, dim3(nblocks(32 * n_sv, 128)), dim3(128), 0, s, n_sv, s64, s32, scale));
   return cudaGetLastError();
 }
 
