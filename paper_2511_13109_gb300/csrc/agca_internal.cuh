@@ -177,8 +177,9 @@ struct StencilArgs {
   T s0, s1, s2;    // mode scalars
 };
 
-// Tile shape of a stencil launch: block rows BY (8, 12 or 16 for FP32; 8
-// otherwise) and the z-chunk (0 = automatic).  Chosen by the autotuner.
+// Tile shape of a stencil launch: block rows (8; 12 and 16 are accepted in FP32
+// contexts, and the tiles ignore them) and the z-chunk (0 = automatic).  Chosen
+// by the autotuner.
 struct TileCfg {
   int by = 8;
   int zch = 0;
@@ -255,9 +256,12 @@ cudaError_t launch_stencil_point_batch(int mode, const StencilTask<T, T>* tasks,
 // stored-Galerkin parts of a batch of tile steps (max_sv: the largest n_sv)
 template <typename T>
 cudaError_t launch_gather_batch(const StencilTask<T, T>* tasks, int ntasks, int64_t max_sv, cudaStream_t s);
-// FP32 tiles of a batch (from f32_tiles); sten: every task has stored-Galerkin stencils, or none has
-cudaError_t launch_stencil_f32_batch(int mode, bool sten, const StencilTask<float, float>* tasks, int ntasks,
-                                     int64_t ntiles, cudaStream_t s);
+// FP32 tiles of a batch (tasks: HOST array, tiles from f32_tiles; a launch takes
+// kF32BatchTasks of them); sten: every task has stored-Galerkin stencils, or none
+// has; wide: every task writes out64 (the later step on finest levels), or none does
+constexpr int kF32BatchTasks = 120;
+cudaError_t launch_stencil_f32_batch(int mode, bool sten, bool wide, const StencilTask<float, float>* tasks, int ntasks,
+                                     cudaStream_t s);
 // whether a step of this kind runs the edge form: every level of an FP64
 // context (its coefficient records exist on every level); the FP32 cycle and
 // the Stokes operator run the per-cube kernel
@@ -282,9 +286,9 @@ struct XferTask {
   double s2;
   const double* sc;     // skip when sc[MS_DONE] != 0, or nullptr
 };
-enum XferKind { XK_RESTRICT = 0, XK_PROLONG_ADD, XK_D2F, XK_F2D, XK_COARSE, XK_PROLONG, XK_COPY64, XK_X1, XK_GRADIENT, XK_DIVERGENCE };
+enum XferKind { XK_RESTRICT = 0, XK_PROLONG_ADD, XK_D2F, XK_COARSE, XK_PROLONG, XK_X1, XK_GRADIENT, XK_DIVERGENCE };
 template <typename T>
-cudaError_t launch_xfer_batch(int kind, const XferTask* tasks, int ntasks, int64_t max_count, int max_m,
+cudaError_t launch_xfer_batch(int kind, int ncomp, const XferTask* tasks, int ntasks, int64_t max_count, int max_m,
                               cudaStream_t s);
 
 // grid transfers (transfer.cu)
@@ -300,6 +304,9 @@ cudaError_t launch_restrict(int nf, int ncomp, bool mask, T scale, const T* rf, 
                             const FirstIterate<T>& fi = {});
 // x1 from a right-hand side in place; n = 3 V entries (D^-1 is 0 on Dirichlet entries, where b is ignored)
 cudaError_t launch_x1(const double* b, const FirstIterate<double>& fi, int64_t n, cudaStream_t s);
+// batched (XK_RESTRICT, XK_PROLONG_ADD, XK_PROLONG); max_n: cubes per axis of the largest grid written
+template <typename T>
+cudaError_t launch_transfer_batch(int kind, int ncomp, const XferTask* tasks, int ntasks, int max_n, cudaStream_t s);
 template <typename T>
 cudaError_t launch_prolong(int nf, int ncomp, bool mask, bool add, const T* ec, T* xf, cudaStream_t s);
 
@@ -321,7 +328,6 @@ cudaError_t launch_galerkin(int nc, int64_t n_flag, const int32_t* list, int nf,
                             cudaStream_t s);
 cudaError_t launch_diag(const LevelOp<double>& op, double* diag, double* invD64, float* invD32, cudaStream_t s);
 cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s, const FirstIterate<float>& fi = {});
-cudaError_t launch_f2d(const float* in, double* out, int64_t n, cudaStream_t s);
 cudaError_t launch_coarse_assemble(const LevelOp<double>& op, double* dense, cudaStream_t s);
 cudaError_t launch_cholesky(double* a, int m, int* status, cudaStream_t s);
 cudaError_t launch_trinv(const double* l, int m, double* linv, cudaStream_t s);

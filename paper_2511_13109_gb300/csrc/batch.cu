@@ -2,7 +2,7 @@
 // Grid (chunks, problems): block row y serves problem y, blocks past the end
 // of a smaller problem exit at once.  A problem whose MINRES has converged
 // (sc[MS_DONE] != 0) is skipped.  Used by the batched solve of
-// agca_batch_solve (persistent stencil launches live in stencil.cu).
+// agca_batch_solve (the stencil launches live in the stencil files).
 #include <math.h>
 
 #include <algorithm>
@@ -18,58 +18,6 @@ constexpr int kBT = 256;
 constexpr int kDotBlocks = 64;  // per problem: fixed, so the reductions are deterministic
 
 __device__ __forceinline__ bool skip(const double* sc) { return sc && sc[MS_DONE] != 0.0; }
-
-template <typename T>
-__global__ void restrict_batch_kernel(const XferTask* __restrict__ tasks) {
-  grid_dep_entry();
-  const XferTask tk = tasks[blockIdx.y];
-  if (skip(tk.sc)) return;
-  const int nf = tk.nf, nvf = nf + 1, nvc = nf / 2 + 1;
-  const int Vc = nvc * nvc * nvc, Vf = nvf * nvf * nvf;
-  const int id = blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= Vc) return;
-  const T* rf = static_cast<const T*>(tk.src);
-  T* rc = static_cast<T*>(tk.dst);
-  const int t = id / nvc, I = id - t * nvc, K = t / nvc, J = t - K * nvc;
-  T* x1 = static_cast<T*>(tk.x1);
-  for (int c = 0; c < tk.ncomp; ++c) {
-    const T v = restrict_point<T>(nf, tk.mask, (T)tk.scale, rf + c * Vf, I, J, K);
-    rc[c * Vc + id] = v;
-    if (x1) x1[c * Vc + id] = (T)tk.s2 * __ldg(static_cast<const T*>(tk.invD) + c * Vc + id) * v;
-  }
-}
-
-template <typename T, bool ADD>
-__global__ void prolong_batch_kernel(const XferTask* __restrict__ tasks) {
-  grid_dep_entry();
-  const XferTask tk = tasks[blockIdx.y];
-  if (skip(tk.sc)) return;
-  const int nf = tk.nf, nvf = nf + 1, nvc = nf / 2 + 1;
-  const int Vc = nvc * nvc * nvc, Vf = nvf * nvf * nvf;
-  const int id = blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= Vf) return;
-  const T* ec = static_cast<const T*>(tk.src);
-  T* xf = static_cast<T*>(tk.dst);
-  const int t = id / nvf, i = id - t * nvf, k = t / nvf, j = t - k * nvf;
-  for (int c = 0; c < tk.ncomp; ++c) {
-    const T v = prolong_point<T>(nf, tk.mask, ec + c * Vc, i, j, k);
-    if (ADD)
-      xf[c * Vf + id] = add_rn(xf[c * Vf + id], v);
-    else
-      xf[c * Vf + id] = v;
-  }
-}
-
-template <typename TI, typename TO>
-__global__ void convert_batch_kernel(const XferTask* __restrict__ tasks) {
-  grid_dep_entry();
-  const XferTask tk = tasks[blockIdx.y];
-  if (skip(tk.sc)) return;
-  const TI* in = static_cast<const TI*>(tk.src);
-  TO* out = static_cast<TO*>(tk.dst);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tk.count; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = (TO)in[i];
-}
 
 // FP32 right-hand sides (XK_D2F) or the FP64 ones in place (XK_X1, WRITE false), with the first Chebyshev iterate
 template <typename TO, bool WRITE>
@@ -221,18 +169,15 @@ inline unsigned chunks(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs)
 }  // namespace
 
 template <typename T>
-cudaError_t launch_xfer_batch(int kind, const XferTask* tasks, int ntasks, int64_t max_count, int max_m,
+cudaError_t launch_xfer_batch(int kind, int ncomp, const XferTask* tasks, int ntasks, int64_t max_count, int max_m,
                               cudaStream_t s) {
   if (ntasks <= 0) return cudaSuccess;
   const dim3 g(chunks(max_count, kBT), (unsigned)ntasks);
   const dim3 gc(std::min<unsigned>(g.x, 1216u), (unsigned)ntasks);
   switch (kind) {
-    case XK_RESTRICT: KL(launch_k(restrict_batch_kernel<T>, g, dim3(kBT), 0, s, tasks)); break;
-    case XK_PROLONG_ADD: KL(launch_k(prolong_batch_kernel<T, true>, g, dim3(kBT), 0, s, tasks)); break;
-    case XK_PROLONG: KL(launch_k(prolong_batch_kernel<T, false>, g, dim3(kBT), 0, s, tasks)); break;
-    case XK_COPY64:
-      KL(launch_k(convert_batch_kernel<double, double>, gc, dim3(kBT), 0, s, tasks));
-      break;
+    case XK_RESTRICT:
+    case XK_PROLONG_ADD:
+    case XK_PROLONG: return launch_transfer_batch<T>(kind, ncomp, tasks, ntasks, max_m, s);
     case XK_D2F:
       KL(launch_k(rhs_batch_kernel<float, true>, gc, dim3(kBT), 0, s, tasks));
       break;
@@ -240,9 +185,6 @@ cudaError_t launch_xfer_batch(int kind, const XferTask* tasks, int ntasks, int64
     case XK_DIVERGENCE: return launch_divergence_batch(tasks, ntasks, max_count, s);
     case XK_X1:
       KL(launch_k(rhs_batch_kernel<double, false>, gc, dim3(kBT), 0, s, tasks));
-      break;
-    case XK_F2D:
-      KL(launch_k(convert_batch_kernel<float, double>, gc, dim3(kBT), 0, s, tasks));
       break;
     case XK_COARSE:
       KL(launch_k(coarse_solve_batch_kernel<T>, dim3(chunks(max_m, kCoarseWarps), (unsigned)ntasks),
@@ -252,8 +194,8 @@ cudaError_t launch_xfer_batch(int kind, const XferTask* tasks, int ntasks, int64
   }
   return cudaGetLastError();
 }
-template cudaError_t launch_xfer_batch<float>(int, const XferTask*, int, int64_t, int, cudaStream_t);
-template cudaError_t launch_xfer_batch<double>(int, const XferTask*, int, int64_t, int, cudaStream_t);
+template cudaError_t launch_xfer_batch<float>(int, int, const XferTask*, int, int64_t, int, cudaStream_t);
+template cudaError_t launch_xfer_batch<double>(int, int, const XferTask*, int, int64_t, int, cudaStream_t);
 
 cudaError_t launch_krylov_batch(int op, const KTask* tasks, int ntasks, int64_t max_n, double* partials,
                                 cudaStream_t s) {

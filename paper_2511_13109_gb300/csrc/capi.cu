@@ -1099,8 +1099,8 @@ agca_status tune_level(agca_ctx* ctx, int l, int reps, std::map<std::string, Til
 // Many independent problems solved together: every problem has its own
 // context (hierarchy, workspace slice, MINRES state); the MINRES iteration of
 // all problems runs in lockstep as one CUDA graph whose launches each cover
-// every problem (persistent stencil launches over the (problem, tile) work
-// list, 2-D element-wise grids over (chunk, problem)), skipping converged
+// every problem (stencil launches over the (problem, tile) work list,
+// 2-D element-wise grids over (chunk, problem)), skipping converged
 // problems on the device.
 struct BatchStep {
   // 0 stencil, 1 xfer, 2 krylov, 3 stencil on small levels (work = cubes per
@@ -1113,7 +1113,9 @@ struct BatchStep {
   size_t off;      // byte offset of the task array in the task table
   int ntasks;
   int64_t work;    // tiles (stencil), max count (xfer), max n (krylov)
-  int max_m;       // coarsest solve size
+  int max_m;       // coarsest solve size; transfers: cubes per axis of the largest
+                   // grid written; FP32 tiles: results widened to FP64
+  int ncomp = 0;   // components (transfers)
 };
 
 }  // namespace
@@ -1241,7 +1243,7 @@ void push_stencil(agca_batch* b, std::vector<BatchStep>& steps, int mode, bool c
       }
       const size_t off = push_tasks(b, u);
       push_gather(steps, u, off, prec);
-      steps.push_back(BatchStep{4, mode, prec, sten, off, (int)u.size(), tiles, 0});
+      steps.push_back(BatchStep{4, mode, prec, sten, off, (int)u.size(), tiles, u[0].a.out64 ? 1 : 0});
     }
     return;
   }
@@ -1274,8 +1276,10 @@ void push_xfer(agca_batch* b, std::vector<BatchStep>& steps, int kind, const std
   for (auto& tk : t) {
     mx = std::max(mx, tk.count);
     if (kind == XK_COARSE) mm = std::max(mm, 3 * (tk.nf - 1) * (tk.nf - 1) * (tk.nf - 1));
+    if (kind == XK_RESTRICT) mm = std::max(mm, tk.nf / 2);
+    if (kind == XK_PROLONG || kind == XK_PROLONG_ADD) mm = std::max(mm, tk.nf);
   }
-  BatchStep st{1, kind, prec, false, push_tasks(b, t), (int)t.size(), mx, mm};
+  BatchStep st{1, kind, prec, false, push_tasks(b, t), (int)t.size(), mx, mm, t[0].ncomp};
   steps.push_back(st);
 }
 
@@ -1287,7 +1291,7 @@ void push_krylov(agca_batch* b, std::vector<BatchStep>& steps, int op, const std
   steps.push_back(st);
 }
 
-// Batched V(2,2) cycle z_p = V_p(r_p) (degree-2 Chebyshev), result copied to z_p.
+// Batched V(2,2) cycle z_p = V_p(r_p) (degree-2 Chebyshev).
 template <typename T>
 void build_cycle(agca_batch* b, std::vector<BatchStep>& steps, const std::vector<const double*>& r,
                  const std::vector<double*>& z, bool skip_done) {
@@ -1392,23 +1396,16 @@ void build_cycle(agca_batch* b, std::vector<BatchStep>& steps, const std::vector
       const double rho = 1.0 / ch.sigma, rn = 1.0 / (2.0 * ch.sigma - rho);
       first.push_back(make_task<T, T>(c, l, ST_CHEB_FIRST, X, bl, nullptr, Tb, 1.0 / ch.theta, 0, 0, sc_of(p)));
       step.push_back(make_task<T, T>(c, l, ST_CHEB_STEP, Tb, bl, X, X, rn * rho, 2.0 * rn / ch.delta, 0, sc_of(p)));
+      if (d == 0) {  // the cycle's result: widened, or written in place of the copy
+        if constexpr (std::is_same<T, float>::value)
+          step.back().a.out64 = z[p];
+        else
+          step.back().a.out = z[p];
+      }
     }
     push_xfer(b, steps, XK_PROLONG_ADD, pro, pr);
     push_stencil<T, T>(b, steps, ST_CHEB_FIRST, d > 0, first, pr);
     push_stencil<T, T>(b, steps, ST_CHEB_STEP, d > 0, step, pr);
-  }
-  {
-    std::vector<XferTask> t;
-    for (int p : b->members) {
-      agca_ctx* c = b->ctx[p];
-      XferTask x{};
-      x.count = 3 * c->lev[c->L].V;
-      x.src = c->lev[c->L].vx;
-      x.dst = z[p];
-      x.sc = sc_of(p);
-      t.push_back(x);
-    }
-    push_xfer(b, steps, mixed ? XK_F2D : XK_COPY64, t, pr);
   }
 }
 
@@ -1544,13 +1541,15 @@ agca_status run_steps(agca_batch* b, const std::vector<BatchStep>& steps, int64_
         BCK(launch_gather_batch<float>((const StencilTask<float, float>*)t, st.ntasks, st.work, s));
       *launches += 1;
     } else if (st.kind == 4) {
-      BCK(launch_stencil_f32_batch(st.mode, st.coarse, (const StencilTask<float, float>*)t, st.ntasks, st.work, s));
-      *launches += 1;
+      BCK(launch_stencil_f32_batch(st.mode, st.coarse, st.max_m != 0,
+                                   reinterpret_cast<const StencilTask<float, float>*>(b->host_tab.data() + st.off),
+                                   st.ntasks, s));
+      *launches += st.ntasks <= 24 ? 1 : (st.ntasks + kF32BatchTasks - 1) / kF32BatchTasks;
     } else if (st.kind == 1) {
       if (st.prec == 1)
-        BCK(launch_xfer_batch<float>(st.mode, (const XferTask*)t, st.ntasks, st.work, st.max_m, s));
+        BCK(launch_xfer_batch<float>(st.mode, st.ncomp, (const XferTask*)t, st.ntasks, st.work, st.max_m, s));
       else
-        BCK(launch_xfer_batch<double>(st.mode, (const XferTask*)t, st.ntasks, st.work, st.max_m, s));
+        BCK(launch_xfer_batch<double>(st.mode, st.ncomp, (const XferTask*)t, st.ntasks, st.work, st.max_m, s));
       *launches += 1;
     } else {
       BCK(launch_krylov_batch(st.mode, (const KTask*)t, st.ntasks, st.work, b->partials, s));

@@ -118,38 +118,93 @@ __device__ __forceinline__ void cube_stokes(const T (&Xl)[4][4], const T (&Xh)[4
 //   (P^T r)(i) = r(2i) + 1/2 sum_d [ r(2i + d) + r(2i - d) ].
 // The weights are known a priori and never stored.
 
-// scale * (P^T r)(I, J, K) for one component r of the fine grid (nf cubes);
-// 0 on the coarse boundary when mask is set
-template <typename T>
-__device__ __forceinline__ T restrict_point(const int nf, const bool mask, const T scale, const T* r, const int I,
-                                            const int J, const int K) {
-  const int nc = nf / 2, nvf = nf + 1;
-  if (mask && (I == 0 || J == 0 || K == 0 || I == nc || J == nc || K == nc)) return T(0);
-  const int fi = 2 * I, fj = 2 * J, fk = 2 * K;
-  T acc = T(0);
-#pragma unroll
-  for (int d = 1; d < 8; ++d) {
-    const int dx = d & 1, dy = (d >> 1) & 1, dz = (d >> 2) & 1;
-    if (fi + dx <= nf && fj + dy <= nf && fk + dz <= nf)
-      acc += __ldg(r + (fi + dx) + nvf * ((fj + dy) + nvf * (fk + dz)));
-    if (fi - dx >= 0 && fj - dy >= 0 && fk - dz >= 0)
-      acc += __ldg(r + (fi - dx) + nvf * ((fj - dy) + nvf * (fk - dz)));
-  }
-  return scale * (__ldg(r + fi + nvf * (fj + nvf * fk)) + T(0.5) * acc);
+// One warp's piece w of the vertices of a grid with nv vertices per axis: 32
+// consecutive ones of a row (whose position is warp-uniform: the per-vertex
+// divisions of a flat index would cost more than the arithmetic)
+struct RowPiece {
+  int i, j, k;  // this lane's vertex; i < nv must hold for it to exist
+};
+__device__ __forceinline__ int row_pieces(const int nv) { return nv * nv * ((nv + 31) / 32); }
+__device__ __forceinline__ RowPiece row_piece(const int nv, const int w, const int lane) {
+  const int per = (nv + 31) / 32, row = w / per, k = row / nv;
+  return RowPiece{32 * (w - row * per) + lane, row - k * nv, k};
 }
 
-// (P e)(i, j, k) for one component e of the coarse grid of a fine grid with
-// nf cubes; 0 on the fine boundary when mask is set
-template <typename T>
-__device__ __forceinline__ T prolong_point(const int nf, const bool mask, const T* e, const int i, const int j,
-                                           const int k) {
-  if (mask && (i == 0 || j == 0 || k == 0 || i == nf || j == nf || k == nf)) return T(0);
-  const int nvc = nf / 2 + 1;
-  const int I = i >> 1, J = j >> 1, K = k >> 1, dx = i & 1, dy = j & 1, dz = k & 1;
-  const T e0 = __ldg(e + I + nvc * (J + nvc * K));
-  if (!(dx | dy | dz)) return e0;
-  // explicit roundings: x + (P e) then rounds the same in every kernel that adds it
-  return mul_rn(T(0.5), add_rn(e0, __ldg(e + (I + dx) + nvc * ((J + dy) + nvc * (K + dz)))));
+// scale * P^T r at coarse vertex (I, J, K) for NC components of a fine grid with
+// nf cubes per axis; 0 on the coarse boundary when mask is set; with fi.x1, the
+// first Chebyshev iterate beside it.  The sum runs over d = 1 .. 7, +d before -d,
+// and a neighbour outside the grid contributes nothing.
+template <typename T, int NC>
+__device__ __forceinline__ void restrict_point(const int nf, const bool mask, const T scale, const T* __restrict__ rf,
+                                               T* __restrict__ rc, const FirstIterate<T>& fi, const RowPiece& p) {
+  const int nc = nf / 2, nvc = nc + 1, nvf = nf + 1, Vc = nvc * nvc * nvc, Vf = nvf * nvf * nvf;
+  const int I = p.i, J = p.j, K = p.k;
+  if (I >= nvc) return;
+  const bool edge = I == 0 || J == 0 || K == 0 || I == nc || J == nc || K == nc;
+  const int f = 2 * I + nvf * (2 * J + nvf * 2 * K), c0 = I + nvc * (J + nvc * K);
+  T v[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) v[c] = T(0);
+  if (!edge) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const T* r = rf + c * Vf + f;
+      T acc = T(0);
+#pragma unroll
+      for (int d = 1; d < 8; ++d) {
+        const int o = (d & 1) + nvf * (((d >> 1) & 1) + nvf * ((d >> 2) & 1));
+        acc += __ldg(r + o);
+        acc += __ldg(r - o);
+      }
+      v[c] = scale * (__ldg(r) + T(0.5) * acc);
+    }
+  } else if (!mask) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const T* r = rf + c * Vf + f;
+      T acc = T(0);
+#pragma unroll
+      for (int d = 1; d < 8; ++d) {
+        const int dx = d & 1, dy = (d >> 1) & 1, dz = (d >> 2) & 1, o = dx + nvf * (dy + nvf * dz);
+        if (2 * I + dx <= nf && 2 * J + dy <= nf && 2 * K + dz <= nf) acc += __ldg(r + o);
+        if (2 * I >= dx && 2 * J >= dy && 2 * K >= dz) acc += __ldg(r - o);
+      }
+      v[c] = scale * (__ldg(r) + T(0.5) * acc);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    rc[c * Vc + c0] = v[c];
+    if (fi.x1) fi.x1[c * Vc + c0] = fi.s2 * __ldg(fi.invD + c * Vc + c0) * v[c];
+  }
+}
+
+// P e at fine vertex (i, j, k) (added to xf when ADD) for NC components; 0 on the
+// fine boundary when mask is set.  Explicit roundings: x + (P e) rounds the same
+// in every kernel that adds it.
+template <typename T, int NC, bool ADD>
+__device__ __forceinline__ void prolong_point(const int nf, const bool mask, const T* __restrict__ ec,
+                                              T* __restrict__ xf, const RowPiece& p) {
+  const int nvf = nf + 1, nvc = nf / 2 + 1, Vc = nvc * nvc * nvc, Vf = nvf * nvf * nvf;
+  const int i = p.i, j = p.j, k = p.k;
+  if (i >= nvf) return;
+  const bool zero = mask && (i == 0 || j == 0 || k == 0 || i == nf || j == nf || k == nf);
+  if (ADD && zero) return;
+  const int dx = i & 1, dy = j & 1, dz = k & 1;
+  const int e0 = (i >> 1) + nvc * ((j >> 1) + nvc * (k >> 1)), e1 = e0 + dx + nvc * (dy + nvc * dz);
+  T* x = xf + i + nvf * (j + nvf * k);
+  T a[NC], b[NC], o[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    a[c] = zero ? T(0) : __ldg(ec + c * Vc + e0);
+    b[c] = zero ? T(0) : __ldg(ec + c * Vc + e1);
+    if (ADD) o[c] = x[c * Vf];
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const T v = (dx | dy | dz) ? mul_rn(T(0.5), add_rn(a[c], b[c])) : a[c];
+    x[c * Vf] = ADD ? add_rn(o[c], v) : v;
+  }
 }
 
 // ------------------------------------------------------------- coarsest solve

@@ -436,38 +436,28 @@ __global__ void __launch_bounds__(FNT, 2)
   f32_block<MODE, STEN, WIDE>(op, a, zch, blockIdx.x % gx, blockIdx.x / gx, blockIdx.y, sm_f32);
 }
 
-// Persistent batched form: every CTA walks the flattened (problem, tile) list.
-template <int MODE, bool STEN>
-__global__ void __launch_bounds__(FNT, 2)
-    stencil_f32_batch_kernel(const StencilTask<float, float>* __restrict__ tasks, const int ntasks,
-                             const int64_t ntiles) {
+// Batched form: a CTA per tile of up to N tasks, which come as kernel parameters:
+// their fields are then read from the constant bank where they are used, as the
+// single launch's.  Read from a device table or a copy in shared memory they
+// stayed in registers across the march and spilled: the later step of twelve
+// problems of 80^3 to 128^3 cubes took 597 us, 2.0 times the single launch's time
+// per vertex.
+template <int N>
+struct F32Tasks {
+  StencilTask<float, float> t[N];
+  int n;
+};
+template <int MODE, bool STEN, bool WIDE, int N>
+__global__ void __launch_bounds__(FNT, 2) stencil_f32_batch_kernel(const __grid_constant__ F32Tasks<N> p) {
   grid_dep_entry();
   extern __shared__ __align__(16) float sm_f32[];
-  for (int64_t it = blockIdx.x; it < ntiles; it += gridDim.x) {
-    int lo = 0, hi = ntasks - 1;  // last task with tile0 <= it
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (tasks[mid].tile0 <= it)
-        lo = mid;
-      else
-        hi = mid - 1;
-    }
-    // the task's fields are read from shared memory as they are needed: held
-    // in registers across the march they spill
-    __shared__ StencilTask<float, float> tk;
-    static_assert(sizeof(tk) % 4 == 0, "copied by words");
-    for (int i = threadIdx.x; i < (int)(sizeof(tk) / 4); i += FNT)
-      reinterpret_cast<int*>(&tk)[i] = reinterpret_cast<const int*>(tasks + lo)[i];
-    __syncthreads();
-    if (tk.sc && tk.sc[MS_DONE] != 0.0) {  // converged problem
-      __syncthreads();
-      continue;
-    }
-    const int local = (int)(it - tk.tile0), per = tk.tg.per_z();
-    const int bz = local / per, u = local % per;
-    f32_block<MODE, STEN, false>(tk.op, tk.a, tk.tg.zch, u % tk.tg.gxw, u / tk.tg.gxw, bz, sm_f32);
-    __syncthreads();  // the shared-memory rings are reused by the next tile
-  }
+  int q = 0;
+  while (q + 1 < p.n && p.t[q + 1].tile0 <= (int64_t)blockIdx.x) ++q;
+  const StencilTask<float, float>& tk = p.t[q];
+  if (tk.sc && tk.sc[MS_DONE] != 0.0) return;  // converged problem
+  const int local = (int)((int64_t)blockIdx.x - tk.tile0), per = tk.tg.gxw * tk.tg.gyw;
+  const int bz = local / per, u = local % per;
+  f32_block<MODE, STEN, WIDE>(tk.op, tk.a, tk.tg.zch, u % tk.tg.gxw, u / tk.tg.gxw, bz, sm_f32);
 }
 
 template <typename K>
@@ -489,12 +479,27 @@ cudaError_t launch_one(const LevelOp<float>& op, const StencilArgs<float>& a, co
   return launch_k(stencil_f32_kernel<MODE, STEN, WIDE>, dim3((unsigned)tg.per_z(), (unsigned)tg.gz), dim3(FNT), f32_smem<MODE>(),
                   s, op, a, tg.zch, tg.gxw);
 }
-template <int MODE, bool STEN>
-cudaError_t launch_many(const StencilTask<float, float>* tasks, int ntasks, int64_t ntiles, int blocks, cudaStream_t s) {
+template <int MODE, bool STEN, bool WIDE, int N>
+cudaError_t launch_some(const StencilTask<float, float>* tasks, int n, cudaStream_t s) {
   static bool done[64] = {};
-  KL(set_smem(stencil_f32_batch_kernel<MODE, STEN>, f32_smem<MODE>(), done));
-  return launch_k(stencil_f32_batch_kernel<MODE, STEN>, dim3((unsigned)std::min<int64_t>(ntiles, blocks)), dim3(FNT),
-                  f32_smem<MODE>(), s, tasks, ntasks, ntiles);
+  KL(set_smem(stencil_f32_batch_kernel<MODE, STEN, WIDE, N>, f32_smem<MODE>(), done));
+  F32Tasks<N> p{};
+  p.n = n;
+  int64_t tiles = 0;
+  for (int i = 0; i < n; ++i) {
+    p.t[i] = tasks[i];
+    p.t[i].tile0 = tiles;
+    tiles += (int64_t)tasks[i].tg.per_z() * tasks[i].tg.gz;
+  }
+  return launch_k(stencil_f32_batch_kernel<MODE, STEN, WIDE, N>, dim3((unsigned)tiles), dim3(FNT), f32_smem<MODE>(), s, p);
+}
+template <int MODE, bool STEN, bool WIDE = false>
+cudaError_t launch_many(const StencilTask<float, float>* tasks, int ntasks, cudaStream_t s) {
+  constexpr int N = kF32BatchTasks, S = 24;
+  static_assert(sizeof(F32Tasks<N>) <= 32764, "kernel parameter limit");
+  if (ntasks <= S) return launch_some<MODE, STEN, WIDE, S>(tasks, ntasks, s);
+  for (int i = 0; i < ntasks; i += N) KL(launch_some<MODE, STEN, WIDE, N>(tasks + i, std::min(N, ntasks - i), s));
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -551,26 +556,22 @@ cudaError_t launch_stencil_f32(int mode, const LevelOp<float>& op, const Stencil
   }
 }
 
-cudaError_t launch_stencil_f32_batch(int mode, bool sten, const StencilTask<float, float>* tasks, int ntasks,
-                                     int64_t ntiles, cudaStream_t s) {
-  if (ntasks <= 0 || ntiles <= 0) return cudaSuccess;
-  int dev = 0, sms = 152;
-  KL(cudaGetDevice(&dev));
-  KL(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int nb = 2 * sms;
+cudaError_t launch_stencil_f32_batch(int mode, bool sten, bool wide, const StencilTask<float, float>* tasks, int ntasks,
+                                     cudaStream_t s) {
+  if (ntasks <= 0) return cudaSuccess;
+  if (wide && mode != ST_CHEB_STEP) return cudaErrorInvalidValue;
   switch (mode) {
     case ST_RESID:
-      return sten ? launch_many<ST_RESID, true>(tasks, ntasks, ntiles, nb, s)
-                  : launch_many<ST_RESID, false>(tasks, ntasks, ntiles, nb, s);
+      return sten ? launch_many<ST_RESID, true>(tasks, ntasks, s) : launch_many<ST_RESID, false>(tasks, ntasks, s);
     case ST_CHEB_FIRST:
-      return sten ? launch_many<ST_CHEB_FIRST, true>(tasks, ntasks, ntiles, nb, s)
-                  : launch_many<ST_CHEB_FIRST, false>(tasks, ntasks, ntiles, nb, s);
+      return sten ? launch_many<ST_CHEB_FIRST, true>(tasks, ntasks, s)
+                  : launch_many<ST_CHEB_FIRST, false>(tasks, ntasks, s);
     case ST_CHEB_STEP:
-      return sten ? launch_many<ST_CHEB_STEP, true>(tasks, ntasks, ntiles, nb, s)
-                  : launch_many<ST_CHEB_STEP, false>(tasks, ntasks, ntiles, nb, s);
+      if (wide) return sten ? cudaErrorInvalidValue : launch_many<ST_CHEB_STEP, false, true>(tasks, ntasks, s);
+      return sten ? launch_many<ST_CHEB_STEP, true>(tasks, ntasks, s)
+                  : launch_many<ST_CHEB_STEP, false>(tasks, ntasks, s);
     case ST_CHEB_PRE:
-      return sten ? launch_many<ST_CHEB_PRE, true>(tasks, ntasks, ntiles, nb, s)
-                  : launch_many<ST_CHEB_PRE, false>(tasks, ntasks, ntiles, nb, s);
+      return sten ? launch_many<ST_CHEB_PRE, true>(tasks, ntasks, s) : launch_many<ST_CHEB_PRE, false>(tasks, ntasks, s);
     default: return cudaErrorInvalidValue;
   }
 }

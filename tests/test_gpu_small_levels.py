@@ -10,6 +10,7 @@ import pytest
 import torch
 
 from oracle import agca as oagca
+from oracle import stokes as ostokes
 from synth import random_vector
 
 pytestmark = pytest.mark.gpu
@@ -68,3 +69,37 @@ def test_point_kernel_meets_tile_kernel(N):
     r = torch.from_numpy(random_vector(3 * c64.V[c64.L], 7)).to(DEV)
     ref = c64.vcycle(r)
     assert float((c32.vcycle(r) - ref).abs().max()) <= 1e-4 * float(ref.abs().max())
+
+
+# pressure grids of 2 to 9 cubes: no, one and several pressure vertices whose whole divergence stencil is interior
+@pytest.mark.parametrize("N", [2, 3, 5, 9])
+def test_stokes_coupling_matches_oracle(N):
+    eta = _eta(N, 60 + N)
+    S = ostokes.Stokes(oagca.Hierarchy(N, 2, eta, 10.0))
+    x = random_vector(3 * (2 * N + 1) ** 3 + (N + 1) ** 3, N)
+    xm = x.copy()
+    xm[:S.nu_] *= S.mask  # boundary velocities are ignored
+    ref = S.K(xm)
+    for prec in (pkg.FP64, pkg.MIXED):
+        c = pkg.Context(N, 2, prec, device=DEV)
+        c.prepare(torch.from_numpy(eta).to(DEV), 10.0)
+        y = c.stokes_apply(torch.from_numpy(x).to(DEV)).cpu().numpy()
+        for part in (slice(None, S.nu_), slice(S.nu_, None)):
+            assert np.abs(y[part] - ref[part]).max() <= 1e-12 * np.abs(ref[part]).max()
+
+
+# tasks of the batched FP32 tiles travel as kernel parameters, 24 or 120 to a launch
+@pytest.mark.parametrize("count", [25, 121])
+def test_large_batch_equals_single(count):
+    N = 18  # 36 cubes per axis: tiles on the finest level
+    etas = [torch.from_numpy(_eta(N, s)).to(DEV) for s in (1, 2)]
+    b = pkg.Batch([N] * count, pkg.MIXED, device=DEV)
+    b.prepare([etas[i % 2] for i in range(count)], 10.0)
+    r = [torch.from_numpy(random_vector(3 * (2 * N + 1) ** 3, 9 + i)).to(DEV) for i in range(2)]
+    z = b.vcycle([r[i % 2] for i in range(count)])
+    for i in range(2):
+        c = pkg.Context(N, None, pkg.MIXED, device=DEV)
+        c.prepare(etas[i], 10.0)
+        ref = c.vcycle(r[i])
+        for j in (i, count - 2 - (count - i) % 2, count - 1 - (count - 1 - i) % 2):
+            assert torch.equal(z[j], ref), j
