@@ -347,11 +347,12 @@ template <typename T>
 cudaError_t launch_masked_coef(int64_t E, const double* mean, const int32_t* fidx, T* coefm, cudaStream_t s);
 cudaError_t launch_start_vector(int n, double* v, cudaStream_t s);
 
-// pressure coupling of the FP64 Stokes operator (stokes.cu): y += -B_f^T q on
-// the interior vertices of the velocity grid (n cubes per axis), y = B u on the
-// pressure grid (np cubes per axis; boundary entries of u are ignored).  Batched:
+// pressure coupling of the FP64 Stokes operator (stokes.cu): y = scale * (a - B_f^T q)
+// on the velocity grid (n cubes per axis; a nullptr: 0, may be y; scale nullptr: 1;
+// 0 on the boundary), y = B u on the pressure grid (np cubes per axis; boundary
+// entries of u are ignored).  Batched: y += -B_f^T q on the interior vertices;
 // tasks with nf = velocity cubes per axis, src, dst
-cudaError_t launch_gradient(int n, const double* q, double* y, cudaStream_t s);
+cudaError_t launch_gradient(int n, const double* q, const double* a, const double* scale, double* y, cudaStream_t s);
 cudaError_t launch_divergence(int np, const double* u, double* y, cudaStream_t s);
 cudaError_t launch_gradient_batch(const XferTask* tasks, int ntasks, int64_t max_count, cudaStream_t s);
 cudaError_t launch_divergence_batch(const XferTask* tasks, int ntasks, int64_t max_count, cudaStream_t s);
@@ -363,18 +364,27 @@ enum MinresSlot {
   MS_INV_GAMMA_PREV, MS_UPD_SKIP, MS_DONE, MS_ITERS, MS_TOL_ABS, MS_DOT_KZZ, MS_DOT_ZV, MS_TMP0, MS_TMP1, MS_TMP2,
   MS_COUNT
 };
-enum VecOp { VOP_SUB = 0, VOP_ADD, VOP_COPY, VOP_ZERO, VOP_PDIV, VOP_SUBS, VOP_MUL, VOP_SCALE_RSQRT, VOP_RECIP };
+enum VecOp { VOP_SUB = 0, VOP_ADD, VOP_COPY, VOP_ZERO, VOP_SUBS, VOP_MUL, VOP_SCALE_RSQRT, VOP_NEG };
 int dot_blocks();
-// out[j] = scale * sum_i xs[j][i] * ys[j][i] for npairs <= 3, deterministic
-cudaError_t launch_dots(int npairs, const double* const* xs, const double* const* ys, int64_t n, double* partials,
-                        double* out, double scale, cudaStream_t s);
-cudaError_t launch_sum(const double* x, int64_t n, double* partials, double* out, double scale, cudaStream_t s);
-cudaError_t launch_vec_op(int op, int64_t n, double* y, const double* a, const double* b, const double* c,
-                          const double* scal, cudaStream_t s);
+// *out = scale * sum x y, scale * sum x; deterministic, one launch (partials:
+// dot_blocks() doubles; counter: 0, and 0 again afterwards)
+cudaError_t launch_dot(const double* x, const double* y, int64_t n, double* partials, int* counter, double* out,
+                       double scale, cudaStream_t s);
+cudaError_t launch_sum(const double* x, int64_t n, double* partials, int* counter, double* out, double scale,
+                       cudaStream_t s);
+cudaError_t launch_vec_op(int op, int64_t n, double* y, const double* a, const double* b, const double* scal,
+                          cudaStream_t s);
 cudaError_t launch_minres_init(double* sc, double tol_rel, cudaStream_t s);
-cudaError_t launch_lanczos(int64_t n, const double* kz, const double* v, double* vold_to_vnew, const double* sc,
-                           cudaStream_t s);
-cudaError_t launch_minres_scalars(double* sc, cudaStream_t s);
+// one MINRES iteration's vector work; the Lanczos step also writes the mean of
+// v_new's pressure part (entries n3 and on) to sc[MS_TMP0]
+cudaError_t launch_lanczos(int64_t n, const double* kz, const double* v, double* vold_to_vnew, double* sc, int64_t n3,
+                           double* partials, int* counter, cudaStream_t s);
+// z = (r - sc[MS_TMP0]) minv, sc[MS_TMP1] = mean of z
+cudaError_t launch_pdiv(int64_t n, const double* r, const double* minv, double* z, double* sc, double* partials,
+                        int* counter, cudaStream_t s);
+// z -= sc[MS_TMP1] in the entries n3 and on, sc[MS_DOT_ZV] = z . v and the scalars of the recurrence
+cudaError_t launch_minres_finish(int64_t n, int64_t n3, double* z, const double* v, double* sc, double* partials,
+                                 int* counter, cudaStream_t s);
 cudaError_t launch_minres_update(int64_t n, const double* z, const double* w, double* wold_to_wnew, double* x,
                                  const double* sc, cudaStream_t s);
 cudaError_t launch_load_vector(int n, const double* fbar, double* b, cudaStream_t s);
@@ -409,7 +419,7 @@ cudaError_t launch_scatter_zrow(int np, int colour, const double* y, double* zs,
 // mean-free on entry, overwritten; x not projected); partials: partials_cap
 // doubles of scratch
 cudaError_t launch_zcg(int np, const double* zs, const double* dinv, double* x, double* r, double* p, double* q,
-                       double* partials, int64_t partials_cap, int iters, cudaStream_t s);
+                       double* z, double* partials, int64_t partials_cap, int iters, cudaStream_t s);
 cudaError_t launch_zdiag_inv(int np, const double* zs, double* dinv, cudaStream_t s);
 cudaError_t launch_sensitivity(int n, const double* eta, const double* lam, const double* u, double* g,
                                cudaStream_t s);

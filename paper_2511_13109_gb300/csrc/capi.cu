@@ -90,6 +90,7 @@ struct agca_ctx {
   double* sc = nullptr;
   double* partials = nullptr;
   int* status = nullptr;
+  int* counter = nullptr;  // of the one-launch reductions: 0 between launches
   int64_t* totals = nullptr;
   int32_t* block_counts = nullptr;
   double nu = 10.0;
@@ -113,6 +114,7 @@ struct agca_ctx {
   cudaGraphExec_t minres_graph[2] = {nullptr, nullptr};
   const double* minres_key[2] = {nullptr, nullptr};  // the correction vector d the graph updates
   int64_t minres_launches[2] = {0, 0};
+  cudaStream_t cap = nullptr;  // for capturing when the context is on the legacy default stream, which cannot
   bool use_graphs = true;
   bool prof = false;
   std::vector<cudaEvent_t> ev;
@@ -124,6 +126,7 @@ struct agca_ctx {
   ~agca_ctx() {
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
     clear_graphs();
+    if (cap) cudaStreamDestroy(cap);
   }
   void clear_graphs() {
     for (auto& g : graphs) cudaGraphExecDestroy(g.exec);
@@ -212,6 +215,7 @@ void carve_workspace(agca_ctx* ctx, char* base) {
   ctx->block_counts = cv.take<int32_t>(compact_scratch_blocks(max_coarse_e) + 1);
   ctx->totals = cv.take<int64_t>(2 * (ctx->L + 1));  // flagged elements, then touched vertices, per level
   ctx->status = cv.take<int>(4);
+  ctx->counter = ctx->status ? ctx->status + 1 : nullptr;
   ctx->sc = cv.take<double>(64);
   ctx->partials = cv.take<double>(3 * (int64_t)dot_blocks());
   const int64_t m2 = (int64_t)ctx->mc * ctx->mc;
@@ -346,7 +350,7 @@ double stencil_bytes(int mode, size_t s) {
 // per-tetrahedron form of the same operator takes 129).  The scaling by h/6
 // folds into the epilogue (3 products, or a fused b - (h/6) y).  The
 // Chebyshev epilogues add per component: residual 2, first step 5, later
-// step 8, step from zero 7 plus 2 for its staged first iterate.
+// step 8, step from zero 7 (its first iterate is an input on tiled levels).
 double stencil_flops(int mode) {
   const double op = 9.0 + 3.0 * (2.0 + 2.0 * 9.0) + 15.0;
   switch (mode) {
@@ -354,7 +358,7 @@ double stencil_flops(int mode) {
     case ST_RESID: return op + 3.0 * 2.0;
     case ST_CHEB_FIRST: return op + 3.0 * 5.0;
     case ST_CHEB_STEP: return op + 3.0 * 8.0;
-    case ST_CHEB_PRE: return op + 3.0 * (7.0 + 2.0);
+    case ST_CHEB_PRE: return op + 3.0 * 7.0;
     default: return 0.0;
   }
 }
@@ -547,7 +551,7 @@ agca_status stokes_impl(agca_ctx* ctx, const double* x, double* y) {
   if (std::is_same<TC, double>::value) {
     // FP64: the viscous block, then the pressure coupling (y_u += B^T p, y_p = B u)
     LK(1, launch_stencil<double, double>(ST_APPLY, op64(ctx, L), a, ctx->stream));
-    LK(1, launch_gradient(lf.n, ctx->qfine, y, ctx->stream));
+    LK(1, launch_gradient(lf.n, ctx->qfine, y, nullptr, y, ctx->stream));
     LK(1, launch_divergence(ctx->N, x, y + n3, ctx->stream));
   } else {
     a.q = ctx->qfine;
@@ -566,20 +570,15 @@ agca_status stokes_dispatch(agca_ctx* ctx, const double* x, double* y, bool low)
 agca_status precond_impl(agca_ctx* ctx, const double* r, double* z) {
   const int64_t n3 = 3 * ctx->lev[ctx->L].V;
   CKS(vcycle_impl(ctx, r, z));
-  const double* rp = r + n3;
-  double* zp = z + n3;
-  const double inv = 1.0 / (double)ctx->Vp;
-  LK(2, launch_sum(rp, ctx->Vp, ctx->partials, ctx->sc + MS_TMP0, inv, ctx->stream));
-  LK(1, launch_vec_op(VOP_PDIV, ctx->Vp, zp, rp, ctx->pmass_inv, nullptr, ctx->sc + MS_TMP0, ctx->stream));
-  LK(2, launch_sum(zp, ctx->Vp, ctx->partials, ctx->sc + MS_TMP1, inv, ctx->stream));
-  LK(1, launch_vec_op(VOP_SUBS, ctx->Vp, zp, zp, nullptr, nullptr, ctx->sc + MS_TMP1, ctx->stream));
+  const int64_t np = ctx->Vp;
+  LK(1, launch_sum(r + n3, np, ctx->partials, ctx->counter, ctx->sc + MS_TMP0, 1.0 / (double)np, ctx->stream));
+  LK(1, launch_pdiv(np, r + n3, ctx->pmass_inv, z + n3, ctx->sc, ctx->partials, ctx->counter, ctx->stream));
+  LK(1, launch_vec_op(VOP_SUBS, np, z + n3, z + n3, nullptr, ctx->sc + MS_TMP1, ctx->stream));
   return AGCA_OK;
 }
 
 agca_status dot1(agca_ctx* ctx, const double* x, const double* y, int64_t n, double* out_dev) {
-  const double* xs[1] = {x};
-  const double* ys[1] = {y};
-  LK(2, launch_dots(1, xs, ys, n, ctx->partials, out_dev, 1.0, ctx->stream));
+  LK(1, launch_dot(x, y, n, ctx->partials, ctx->counter, out_dev, 1.0, ctx->stream));
   return AGCA_OK;
 }
 
@@ -603,11 +602,11 @@ agca_status minres_impl(agca_ctx* ctx, const double* b, double* d, double tol_re
   double* wold = ctx->kv[KV_WOLD];
   double* w = ctx->kv[KV_W];
   double* kz = ctx->kv[KV_KZ];
-  LK(1, launch_vec_op(VOP_ZERO, nt, d, nullptr, nullptr, nullptr, nullptr, s));
-  LK(1, launch_vec_op(VOP_ZERO, nt, vold, nullptr, nullptr, nullptr, nullptr, s));
-  LK(1, launch_vec_op(VOP_ZERO, nt, wold, nullptr, nullptr, nullptr, nullptr, s));
-  LK(1, launch_vec_op(VOP_ZERO, nt, w, nullptr, nullptr, nullptr, nullptr, s));
-  LK(1, launch_vec_op(VOP_COPY, nt, v, b, nullptr, nullptr, nullptr, s));
+  LK(1, launch_vec_op(VOP_ZERO, nt, d, nullptr, nullptr, nullptr, s));
+  LK(1, launch_vec_op(VOP_ZERO, nt, vold, nullptr, nullptr, nullptr, s));
+  LK(1, launch_vec_op(VOP_ZERO, nt, wold, nullptr, nullptr, nullptr, s));
+  LK(1, launch_vec_op(VOP_ZERO, nt, w, nullptr, nullptr, nullptr, s));
+  LK(1, launch_vec_op(VOP_COPY, nt, v, b, nullptr, nullptr, s));
   CKS(precond_impl(ctx, v, z));
   CKS(dot1(ctx, z, v, nt, ctx->sc + MS_DOT_ZV));
   LK(1, launch_minres_init(ctx->sc, tol_rel, s));
@@ -615,10 +614,11 @@ agca_status minres_impl(agca_ctx* ctx, const double* b, double* d, double tol_re
   auto iteration = [&]() -> agca_status {
     CKS(stokes_dispatch(ctx, z, kz, low));
     CKS(dot1(ctx, kz, z, nt, ctx->sc + MS_DOT_KZZ));
-    LK(1, launch_lanczos(nt, kz, v, vold, ctx->sc, s));  // vold <- v_new
-    CKS(precond_impl(ctx, vold, zn));
-    CKS(dot1(ctx, zn, vold, nt, ctx->sc + MS_DOT_ZV));
-    LK(1, launch_minres_scalars(ctx->sc, s));
+    const int64_t n3 = nt - ctx->Vp;
+    LK(1, launch_lanczos(nt, kz, v, vold, ctx->sc, n3, ctx->partials, ctx->counter, s));  // vold <- v_new
+    CKS(vcycle_direct(ctx, vold, zn));
+    LK(1, launch_pdiv(ctx->Vp, vold + n3, ctx->pmass_inv, zn + n3, ctx->sc, ctx->partials, ctx->counter, s));
+    LK(1, launch_minres_finish(nt, n3, zn, vold, ctx->sc, ctx->partials, ctx->counter, s));
     LK(1, launch_minres_update(nt, z, w, wold, d, ctx->sc, s));  // wold <- w_new
     std::swap(vold, v);
     std::swap(z, zn);
@@ -628,21 +628,37 @@ agca_status minres_impl(agca_ctx* ctx, const double* b, double* d, double tol_re
   // iterations past convergence change nothing (the device scalars freeze the
   // update), so the loop may run a few beyond it between host checks
   const int gi = low ? 1 : 0;
-  bool graph = ctx->use_graphs && !ctx->prof && s != nullptr;
-  if (graph) {
+  // The legacy default stream cannot be captured, but a graph captured on
+  // another stream runs on it: some 25 launches an iteration at small sizes
+  // otherwise cost more on the host than on the GPU.
+  const bool legacy = s == nullptr || s == cudaStreamLegacy;
+  bool graph = ctx->use_graphs && !ctx->prof;
+  if (graph && !legacy) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CK(cudaStreamIsCapturing(s, &cs));
     graph = (cs == cudaStreamCaptureStatusNone);
+  }
+  if (graph && legacy && !ctx->cap && cudaStreamCreateWithFlags(&ctx->cap, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->cap = nullptr;
+    graph = false;
   }
   if (graph && (ctx->minres_graph[gi] == nullptr || ctx->minres_key[gi] != d)) {
     if (ctx->minres_graph[gi]) cudaGraphExecDestroy(ctx->minres_graph[gi]);
     ctx->minres_graph[gi] = nullptr;
     const int64_t l0 = ctx->launches;
     cudaGraph_t g = nullptr;
-    CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    agca_status st = iteration();
-    if (st == AGCA_OK) st = iteration();
-    const cudaError_t ee = cudaStreamEndCapture(s, &g);
+    const cudaStream_t own = ctx->stream;
+    if (legacy) s = ctx->stream = ctx->cap;
+    const cudaError_t be = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+    agca_status st = AGCA_OK;
+    cudaError_t ee = be;
+    if (be == cudaSuccess) {
+      st = iteration();
+      if (st == AGCA_OK) st = iteration();
+      ee = cudaStreamEndCapture(s, &g);
+    }
+    s = ctx->stream = own;
     ctx->minres_launches[gi] = ctx->launches - l0;
     ctx->launches = l0;
     if (st != AGCA_OK) {
@@ -680,9 +696,20 @@ agca_status minres_impl(agca_ctx* ctx, const double* b, double* d, double tol_re
 
 agca_status project_pressure(agca_ctx* ctx, double* x) {
   const int64_t n3 = 3 * ctx->lev[ctx->L].V;
-  LK(2, launch_sum(x + n3, ctx->Vp, ctx->partials, ctx->sc + MS_TMP2, 1.0 / (double)ctx->Vp, ctx->stream));
-  LK(1, launch_vec_op(VOP_SUBS, ctx->Vp, x + n3, x + n3, nullptr, nullptr, ctx->sc + MS_TMP2, ctx->stream));
+  LK(1, launch_sum(x + n3, ctx->Vp, ctx->partials, ctx->counter, ctx->sc + MS_TMP2, 1.0 / (double)ctx->Vp,
+                   ctx->stream));
+  LK(1, launch_vec_op(VOP_SUBS, ctx->Vp, x + n3, x + n3, nullptr, ctx->sc + MS_TMP2, ctx->stream));
   return AGCA_OK;
+}
+
+// Tolerance of an inner MINRES that would have to reduce the residual by `want`
+// to end a tenth below the outer one's.  Mixed refinement stops at the floor,
+// where FP32 arithmetic still converges well, and goes on from the true residual
+// -- unless a little more ends the solve: stopping just short of it, the result
+// lay barely below or barely above the tolerance, by chance.
+double inner_tolerance(double want, bool mixed, double floor) {
+  if (mixed && want < floor && !(30.0 * want >= floor)) want = floor;
+  return std::max(want, 1e-14);
 }
 
 agca_status solve_impl(agca_ctx* ctx, const double* b_in, double* x, double rtol, int maxit, int* iters,
@@ -694,10 +721,10 @@ agca_status solve_impl(agca_ctx* ctx, const double* b_in, double* x, double rtol
   double* kx = ctx->kv[KV_KZ];
   // Dirichlet rows carry no equation: work on a copy of b with them zeroed
   double* bm = ctx->kv[KV_B];
-  LK(1, launch_vec_op(VOP_COPY, nt, bm, b_in, nullptr, nullptr, nullptr, s));
+  LK(1, launch_vec_op(VOP_COPY, nt, bm, b_in, nullptr, nullptr, s));
   LK(1, launch_mask_boundary(ctx->lev[ctx->L].n, bm, s));
   const double* b = bm;
-  LK(1, launch_vec_op(VOP_ZERO, nt, x, nullptr, nullptr, nullptr, nullptr, s));
+  LK(1, launch_vec_op(VOP_ZERO, nt, x, nullptr, nullptr, nullptr, s));
   double nb2 = 0.0;
   CKS(dot1(ctx, b, b, nt, ctx->sc + MS_TMP0));
   CKS(read_scalar(ctx, ctx->sc + MS_TMP0, &nb2));
@@ -707,19 +734,17 @@ agca_status solve_impl(agca_ctx* ctx, const double* b_in, double* x, double rtol
   const bool mixed = ctx->prec == AGCA_MIXED;
   for (int outer = 0; outer < 60 && nb > 0.0; ++outer) {
     CKS(stokes_dispatch(ctx, x, kx, false));
-    LK(1, launch_vec_op(VOP_SUB, nt, r, b, kx, nullptr, nullptr, s));
+    LK(1, launch_vec_op(VOP_SUB, nt, r, b, kx, nullptr, s));
     double nr2 = 0.0;
     CKS(dot1(ctx, r, r, nt, ctx->sc + MS_TMP0));
     CKS(read_scalar(ctx, ctx->sc + MS_TMP0, &nr2));
     rel = sqrt(nr2) / nb;
     if (!(rel > rtol) || total >= maxit) break;
-    double inner = 0.1 * rtol / rel;
-    if (mixed) inner = std::max(inner, ctx->mixed_inner);
-    inner = std::max(inner, 1e-14);
+    const double inner = inner_tolerance(0.1 * rtol / rel, mixed, ctx->mixed_inner);
     int its = 0;
     CKS(minres_impl(ctx, r, d, inner, maxit - total, mixed, &its));
     total += its;
-    LK(1, launch_vec_op(VOP_ADD, nt, x, x, d, nullptr, nullptr, s));
+    LK(1, launch_vec_op(VOP_ADD, nt, x, x, d, nullptr, s));
     CKS(project_pressure(ctx, x));
     if (its == 0) break;
   }
@@ -745,14 +770,16 @@ agca_status solve_impl(agca_ctx* ctx, const double* b_in, double* x, double rtol
 // apart, so 125 applies of the matrix-free Z to colour indicators (vertices
 // equal mod 5 per axis) give every row as a 5x5x5 stencil; Z^-1 by
 // Jacobi-preconditioned conjugate gradients on the mean-free pressures.  In
-// mixed contexts the preconditioner's Stokes applies use FP32 arithmetic;
+// mixed contexts the preconditioner's Stokes apply uses FP32 arithmetic;
 // the outer K z stays FP64.  Arnoldi by classical
 // Gram-Schmidt with one reorthogonalisation (two block dot products and two
 // block updates per iteration); the small Hessenberg least-squares problem
 // by Givens rotations on the host.
 struct FgmresWork {
-  double *V, *Z, *w, *t1, *t2, *partials, *hbuf, *ycoef, *zdinv, *cx, *cr, *cz, *cp, *cq, *m, *sc, *zsten;
+  double *V, *Z, *w, *t1, *t2, *partials, *hbuf, *ycoef, *zdinv, *cx, *cr, *cz, *cp, *cq, *m, *sc, *zsten, *rec;
   int64_t npartials;
+  bool has_rec;
+  size_t need_bare;  // bytes without rec
   size_t need;
 };
 
@@ -778,28 +805,30 @@ FgmresWork fgmres_layout(const agca_ctx* ctx, int restart, char* base) {
   w.m = cv.take<double>(np);
   w.sc = cv.take<double>(8);
   w.zsten = cv.take<double>(np * ZSTENCIL);
+  // a mixed context keeps no coefficient records of its finest level; K z in FP64
+  // every iteration pays for them (204 -> 60 us an apply at 64^3 cubes); a smaller
+  // workspace does without
+  w.need_bare = (cv.off + kAlign - 1) / kAlign * kAlign;
+  const Level& lf = ctx->lev[ctx->L];
+  w.rec = lf.hedge == nullptr && lf.n > kPointMaxN ? cv.take<double>(EREC * lf.V) : nullptr;
+  w.has_rec = lf.hedge == nullptr && lf.n > kPointMaxN;
   w.need = (cv.off + kAlign - 1) / kAlign * kAlign;
   return w;
 }
 
-// t2 = K [W^-1 B^T p; 0]: pressure part Z p, velocity part A W^-1 B^T p (t1 scratch)
-agca_status z_apply(agca_ctx* ctx, const FgmresWork& W, const double* p) {
-  const int64_t n3 = 3 * ctx->lev[ctx->L].V, np = ctx->Vp;
-  cudaStream_t s = ctx->stream;
-  LK(1, launch_vec_op(VOP_ZERO, n3, W.t1, nullptr, nullptr, nullptr, nullptr, s));
-  LK(1, launch_vec_op(VOP_COPY, np, W.t1 + n3, p, nullptr, nullptr, nullptr, s));
-  CKS(stokes_dispatch(ctx, W.t1, W.t2, true));  // t2_u = B^T p
-  LK(1, launch_vec_op(VOP_MUL, n3, W.t1, W.t2, ctx->lev[ctx->L].invD64, nullptr, nullptr, s));
-  LK(1, launch_vec_op(VOP_ZERO, np, W.t1 + n3, nullptr, nullptr, nullptr, nullptr, s));
-  CKS(stokes_dispatch(ctx, W.t1, W.t2, true));  // [A W^-1 B^T p; Z p]
+// t1 = scale * (a + B^T p) on the velocity grid (a, scale as launch_gradient)
+agca_status bt_apply(agca_ctx* ctx, const double* p, const double* a, const double* scale, double* t1) {
+  const int n = ctx->lev[ctx->L].n;
+  LK(1, launch_prolong<double>(n, 1, false, false, p, ctx->qfine, ctx->stream));
+  LK(1, launch_gradient(n, ctx->qfine, a, scale, t1, ctx->stream));
   return AGCA_OK;
 }
 
 // y = y - mean(y) over the pressure DoFs
 agca_status mean_free(agca_ctx* ctx, double* y) {
   const int64_t np = ctx->Vp;
-  LK(2, launch_sum(y, np, ctx->partials, ctx->sc + MS_TMP2, 1.0 / (double)np, ctx->stream));
-  LK(1, launch_vec_op(VOP_SUBS, np, y, y, nullptr, nullptr, ctx->sc + MS_TMP2, ctx->stream));
+  LK(1, launch_sum(y, np, ctx->partials, ctx->counter, ctx->sc + MS_TMP2, 1.0 / (double)np, ctx->stream));
+  LK(1, launch_vec_op(VOP_SUBS, np, y, y, nullptr, ctx->sc + MS_TMP2, ctx->stream));
   return AGCA_OK;
 }
 
@@ -807,21 +836,21 @@ agca_status mean_free(agca_ctx* ctx, double* y) {
 agca_status z_solve(agca_ctx* ctx, const FgmresWork& W, const double* rhs, double* x, int iters) {
   const int64_t np = ctx->Vp;
   cudaStream_t s = ctx->stream;
-  LK(1, launch_vec_op(VOP_COPY, np, W.cr, rhs, nullptr, nullptr, nullptr, s));
+  LK(1, launch_vec_op(VOP_COPY, np, W.cr, rhs, nullptr, nullptr, s));
   CKS(mean_free(ctx, W.cr));
-  LK(1, launch_zcg(ctx->N, W.zsten, W.zdinv, x, W.cr, W.cp, W.cq, W.partials, W.npartials, iters, s));
+  LK(1, launch_zcg(ctx->N, W.zsten, W.zdinv, x, W.cr, W.cp, W.cq, W.cz, W.partials, W.npartials, iters, s));
   CKS(mean_free(ctx, x));
   return AGCA_OK;
 }
 
 // Z assembled by probing with the 125 colours (i, j, k) mod 5, and its inverse diagonal
 agca_status z_assemble(agca_ctx* ctx, const FgmresWork& W) {
-  const int64_t n3 = 3 * ctx->lev[ctx->L].V;
   cudaStream_t s = ctx->stream;
   for (int c = 0; c < 125; ++c) {
     LK(1, launch_colour5(ctx->N, c, W.cp, s));
-    CKS(z_apply(ctx, W, W.cp));
-    LK(1, launch_scatter_zrow(ctx->N, c, W.t2 + n3, W.zsten, s));
+    CKS(bt_apply(ctx, W.cp, nullptr, ctx->lev[ctx->L].invD64, W.t1));  // W^-1 B^T e
+    LK(1, launch_divergence(ctx->N, W.t1, W.cq, s));                   // Z e
+    LK(1, launch_scatter_zrow(ctx->N, c, W.cq, W.zsten, s));
   }
   LK(1, launch_zdiag_inv(ctx->N, W.zsten, W.zdinv, s));
   return AGCA_OK;
@@ -834,27 +863,22 @@ agca_status blocktri_precond(agca_ctx* ctx, const FgmresWork& W, const double* r
   const double* rp = r + n3;
   double* zp = z + n3;
   if (schur == 0) {
-    const double inv = 1.0 / (double)np;
-    LK(2, launch_sum(rp, np, ctx->partials, ctx->sc + MS_TMP0, inv, s));
-    LK(1, launch_vec_op(VOP_PDIV, np, zp, rp, ctx->pmass_inv, nullptr, ctx->sc + MS_TMP0, s));
-    CKS(mean_free(ctx, zp));
+    LK(1, launch_sum(rp, np, ctx->partials, ctx->counter, ctx->sc + MS_TMP0, 1.0 / (double)np, s));
+    LK(1, launch_pdiv(np, rp, ctx->pmass_inv, zp, ctx->sc, ctx->partials, ctx->counter, s));
+    LK(1, launch_vec_op(VOP_SUBS, np, zp, zp, nullptr, ctx->sc + MS_TMP1, s));
   } else {
-    CKS(z_solve(ctx, W, rp, W.m, z_iters));                 // t = Z^-1 r_p
-    CKS(z_apply(ctx, W, W.m));                              // t2_u = A W^-1 B^T t
-    LK(1, launch_vec_op(VOP_MUL, n3, W.t1, W.t2, ctx->lev[ctx->L].invD64, nullptr, nullptr, s));
-    LK(1, launch_vec_op(VOP_ZERO, np, W.t1 + n3, nullptr, nullptr, nullptr, nullptr, s));
-    CKS(stokes_dispatch(ctx, W.t1, W.t2, true));          // t2_p = B W^-1 A W^-1 B^T t
-    LK(1, launch_vec_op(VOP_COPY, np, W.m, W.t2 + n3, nullptr, nullptr, nullptr, s));
-    CKS(z_solve(ctx, W, W.m, zp, z_iters));                 // S~^-1 r_p
+    const double* invD = ctx->lev[ctx->L].invD64;
+    CKS(z_solve(ctx, W, rp, W.m, z_iters));               // t = Z^-1 r_p
+    CKS(bt_apply(ctx, W.m, nullptr, invD, W.t1));         // t1 = W^-1 B^T t
+    LK(1, launch_vec_op(VOP_ZERO, np, W.t1 + n3, nullptr, nullptr, nullptr, s));
+    CKS(stokes_dispatch(ctx, W.t1, W.t2, true));          // t2_u = A W^-1 B^T t
+    LK(1, launch_vec_op(VOP_MUL, n3, W.t1, W.t2, invD, nullptr, s));
+    LK(1, launch_divergence(ctx->N, W.t1, W.m, s));       // B W^-1 A W^-1 B^T t
+    CKS(z_solve(ctx, W, W.m, zp, z_iters));               // S~^-1 r_p
   }
-  // z_p = -S~^-1 r_p
-  LK(1, launch_vec_op(VOP_ZERO, np, W.cq, nullptr, nullptr, nullptr, nullptr, s));
-  LK(1, launch_vec_op(VOP_SUB, np, zp, W.cq, zp, nullptr, nullptr, s));
-  // z_u = A~^-1 (r_u - B^T z_p)
-  LK(1, launch_vec_op(VOP_ZERO, n3, W.t1, nullptr, nullptr, nullptr, nullptr, s));
-  LK(1, launch_vec_op(VOP_COPY, np, W.t1 + n3, zp, nullptr, nullptr, nullptr, s));
-  CKS(stokes_dispatch(ctx, W.t1, W.t2, true));  // t2_u = B^T z_p
-  LK(1, launch_vec_op(VOP_SUB, n3, W.t1, r, W.t2, nullptr, nullptr, s));
+  // z_u = A~^-1 (r_u - B^T z_p) with z_p = -S~^-1 r_p
+  CKS(bt_apply(ctx, zp, r, nullptr, W.t1));
+  LK(1, launch_vec_op(VOP_NEG, np, zp, zp, nullptr, nullptr, s));
   CKS(vcycle_impl(ctx, W.t1, z));
   return AGCA_OK;
 }
@@ -866,9 +890,9 @@ agca_status fgmres_impl(agca_ctx* ctx, const FgmresWork& W, int restart, const d
   double* r = ctx->kv[KV_R];
   double* kx = ctx->kv[KV_KZ];
   double* bm = ctx->kv[KV_B];
-  LK(1, launch_vec_op(VOP_COPY, nt, bm, b_in, nullptr, nullptr, nullptr, s));
+  LK(1, launch_vec_op(VOP_COPY, nt, bm, b_in, nullptr, nullptr, s));
   LK(1, launch_mask_boundary(ctx->lev[ctx->L].n, bm, s));
-  LK(1, launch_vec_op(VOP_ZERO, nt, x, nullptr, nullptr, nullptr, nullptr, s));
+  LK(1, launch_vec_op(VOP_ZERO, nt, x, nullptr, nullptr, nullptr, s));
   if (schur == 1) CKS(z_assemble(ctx, W));
   double nb2 = 0.0;
   CKS(dot1(ctx, bm, bm, nt, ctx->sc + MS_TMP0));
@@ -884,14 +908,14 @@ agca_status fgmres_impl(agca_ctx* ctx, const FgmresWork& W, int restart, const d
   double* const wn2 = W.hbuf + 2 * (restart + 1);
   while (nb > 0.0) {
     CKS(stokes_dispatch(ctx, x, kx, false));
-    LK(1, launch_vec_op(VOP_SUB, nt, r, bm, kx, nullptr, nullptr, s));
+    LK(1, launch_vec_op(VOP_SUB, nt, r, bm, kx, nullptr, s));
     double beta2 = 0.0;
     CKS(dot1(ctx, r, r, nt, ctx->sc + MS_TMP0));
     CKS(read_scalar(ctx, ctx->sc + MS_TMP0, &beta2));
     const double beta = sqrt(beta2);
     rel = beta / nb;
     if (!(rel > rtol) || its >= maxit) break;
-    LK(1, launch_vec_op(VOP_SCALE_RSQRT, nt, W.V, r, nullptr, nullptr, ctx->sc + MS_TMP0, s));  // v0 = r / beta
+    LK(1, launch_vec_op(VOP_SCALE_RSQRT, nt, W.V, r, nullptr, ctx->sc + MS_TMP0, s));  // v0 = r / beta
     std::fill(g.begin(), g.end(), 0.0);
     g[0] = beta;
     int m = 0;
@@ -906,7 +930,7 @@ agca_status fgmres_impl(agca_ctx* ctx, const FgmresWork& W, int restart, const d
       LK(2, launch_block_dot(j + 1, W.V, nt, W.w, nt, W.partials, h2dev, s));
       LK(1, launch_block_axpy(j + 1, W.V, nt, h2dev, -1.0, W.w, nt, s));
       CKS(dot1(ctx, W.w, W.w, nt, wn2));
-      LK(1, launch_vec_op(VOP_SCALE_RSQRT, nt, W.V + (int64_t)(j + 1) * nt, W.w, nullptr, nullptr, wn2, s));
+      LK(1, launch_vec_op(VOP_SCALE_RSQRT, nt, W.V + (int64_t)(j + 1) * nt, W.w, nullptr, wn2, s));
       CK(cudaMemcpyAsync(hv.data(), W.hbuf, (2 * (restart + 1) + 1) * sizeof(double), cudaMemcpyDeviceToHost, s));
       CK(cudaStreamSynchronize(s));
       for (int i = 0; i <= j; ++i) Hh(i, j) = hv[i] + hv[restart + 1 + i];
@@ -983,12 +1007,12 @@ agca_status power_lambda(agca_ctx* ctx, int l) {
       std::swap(v, w);
       if (it % 16 == 15) {
         CKS(dot1(ctx, v, v, n3, ctx->sc + MS_TMP0));
-        LK(1, launch_vec_op(VOP_SCALE_RSQRT, n3, v, v, nullptr, nullptr, ctx->sc + MS_TMP0, s));
+        LK(1, launch_vec_op(VOP_SCALE_RSQRT, n3, v, v, nullptr, ctx->sc + MS_TMP0, s));
       }
     }
     CKS(stencil<double>(ctx, ST_APPLY, l, v, nullptr, nullptr, w, 0, 0, 0));
     CKS(dot1(ctx, v, w, n3, ctx->sc + kRaySlot + 2 * l));
-    LK(1, launch_vec_op(VOP_MUL, n3, w, v, lv.diag, nullptr, nullptr, s));
+    LK(1, launch_vec_op(VOP_MUL, n3, w, v, lv.diag, nullptr, s));
     return dot1(ctx, v, w, n3, ctx->sc + kRaySlot + 2 * l + 1);
   };
   const agca_status st = run();
@@ -1663,6 +1687,7 @@ agca_status agca_bind_workspace(agca_ctx* ctx, void* dev_ptr, size_t bytes) {
   ctx->ws = static_cast<char*>(dev_ptr);
   ctx->ws_bytes = bytes;
   carve_workspace(ctx, ctx->ws);
+  CK(cudaMemsetAsync(ctx->counter, 0, sizeof(int), ctx->stream));
   ctx->have_eta = ctx->flagged = ctx->setup_done = false;
   ctx->gs = nullptr;
   return AGCA_OK;
@@ -1909,9 +1934,17 @@ agca_status agca_solve_fgmres(agca_ctx* ctx, const double* b_dev, double* x_dev,
     return ctx->fail(AGCA_EINVAL, "bad FGMRES parameters");
   if (!ctx->setup_done) return ctx->fail(AGCA_ESTATE, "setup first");
   if (((uintptr_t)work_dev % kAlign) != 0) return ctx->fail(AGCA_EINVAL, "workspace must be 256-byte aligned");
-  const FgmresWork W = fgmres_layout(ctx, restart, static_cast<char*>(work_dev));
-  if (work_bytes < W.need) return ctx->fail(AGCA_ENOMEM, "FGMRES workspace too small");
-  return fgmres_impl(ctx, W, restart, b_dev, x_dev, rtol, maxit, schur, z_iters, iters, relres);
+  FgmresWork W = fgmres_layout(ctx, restart, static_cast<char*>(work_dev));
+  if (work_bytes < W.need) W.has_rec = false;
+  if (work_bytes < W.need_bare) return ctx->fail(AGCA_ENOMEM, "FGMRES workspace too small");
+  Level& lf = ctx->lev[ctx->L];
+  if (W.has_rec) {
+    LK(1, launch_edge_records(lf.n, lf.mean, nullptr, W.rec, ctx->stream));
+    lf.hedge = W.rec;
+  }
+  const agca_status st = fgmres_impl(ctx, W, restart, b_dev, x_dev, rtol, maxit, schur, z_iters, iters, relres);
+  if (W.has_rec) lf.hedge = nullptr;
+  return st;
 }
 
 agca_status agca_element_sensitivity(agca_ctx* ctx, const double* lam_u_dev, const double* u_dev, double* g_dev) {
@@ -2312,9 +2345,9 @@ agca_status agca_batch_solve(agca_batch* b, const double* const* b_devs, double*
     agca_ctx* ctx = b->ctx[p];
     const int64_t nt = ctx->nt;
     double* bm = ctx->kv[KV_B];
-    LK(1, launch_vec_op(VOP_COPY, nt, bm, b_devs[p], nullptr, nullptr, nullptr, b->stream));
+    LK(1, launch_vec_op(VOP_COPY, nt, bm, b_devs[p], nullptr, nullptr, b->stream));
     LK(1, launch_mask_boundary(ctx->lev[ctx->L].n, bm, b->stream));
-    LK(1, launch_vec_op(VOP_ZERO, nt, x_devs[p], nullptr, nullptr, nullptr, nullptr, b->stream));
+    LK(1, launch_vec_op(VOP_ZERO, nt, x_devs[p], nullptr, nullptr, nullptr, b->stream));
     double nb2 = 0.0;
     CKS(dot1(ctx, bm, bm, nt, ctx->sc + MS_TMP0));
     CKS(read_scalar(ctx, ctx->sc + MS_TMP0, &nb2));
@@ -2331,7 +2364,7 @@ agca_status agca_batch_solve(agca_batch* b, const double* const* b_devs, double*
       active[p] = 0;
       if (!(nb[p] > 0.0)) continue;
       CKS(stokes_dispatch(ctx, x_devs[p], ctx->kv[KV_KZ], false));
-      LK(1, launch_vec_op(VOP_SUB, nt, ctx->kv[KV_R], ctx->kv[KV_B], ctx->kv[KV_KZ], nullptr, nullptr, b->stream));
+      LK(1, launch_vec_op(VOP_SUB, nt, ctx->kv[KV_R], ctx->kv[KV_B], ctx->kv[KV_KZ], nullptr, b->stream));
       double nr2 = 0.0;
       CKS(dot1(ctx, ctx->kv[KV_R], ctx->kv[KV_R], nt, ctx->sc + MS_TMP0));
       CKS(read_scalar(ctx, ctx->sc + MS_TMP0, &nr2));
@@ -2359,14 +2392,12 @@ agca_status agca_batch_solve(agca_batch* b, const double* const* b_devs, double*
         continue;
       }
       budget = std::max(budget, maxit - total[p]);
-      double inner = 0.1 * rtol / rel[p];
-      if (mixed) inner = std::max(inner, ctx->mixed_inner);
-      inner = std::max(inner, 1e-14);
-      LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_D], nullptr, nullptr, nullptr, nullptr, s));
-      LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_VOLD], nullptr, nullptr, nullptr, nullptr, s));
-      LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_WOLD], nullptr, nullptr, nullptr, nullptr, s));
-      LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_W], nullptr, nullptr, nullptr, nullptr, s));
-      LK(1, launch_vec_op(VOP_COPY, nt, ctx->kv[KV_V], ctx->kv[KV_R], nullptr, nullptr, nullptr, s));
+      const double inner = inner_tolerance(0.1 * rtol / rel[p], mixed, ctx->mixed_inner);
+      LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_D], nullptr, nullptr, nullptr, s));
+      LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_VOLD], nullptr, nullptr, nullptr, s));
+      LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_WOLD], nullptr, nullptr, nullptr, s));
+      LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_W], nullptr, nullptr, nullptr, s));
+      LK(1, launch_vec_op(VOP_COPY, nt, ctx->kv[KV_V], ctx->kv[KV_R], nullptr, nullptr, s));
       CKS(precond_impl(ctx, ctx->kv[KV_V], ctx->kv[KV_Z]));
       CKS(dot1(ctx, ctx->kv[KV_Z], ctx->kv[KV_V], nt, ctx->sc + MS_DOT_ZV));
       LK(1, launch_minres_init(ctx->sc, inner, s));
@@ -2402,7 +2433,7 @@ agca_status agca_batch_solve(agca_batch* b, const double* const* b_devs, double*
       double its = 0.0;
       CKS(read_scalar(ctx, ctx->sc + MS_ITERS, &its));
       total[p] += (int)its;
-      LK(1, launch_vec_op(VOP_ADD, ctx->nt, x_devs[p], x_devs[p], ctx->kv[KV_D], nullptr, nullptr, b->stream));
+      LK(1, launch_vec_op(VOP_ADD, ctx->nt, x_devs[p], x_devs[p], ctx->kv[KV_D], nullptr, b->stream));
       CKS(project_pressure(ctx, x_devs[p]));
     }
     b->ctx[0]->launches += launches;

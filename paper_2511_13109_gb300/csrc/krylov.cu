@@ -18,36 +18,85 @@ namespace {
 constexpr int kRedBlocks = 1216;  // 8 per SM; fixed so reductions are deterministic
 constexpr int kRedThreads = 256;
 
-struct DotPairs {
-  const double* x[3];
-  const double* y[3];
-};
+// Blocks of a pass over n entries: a function of n alone, so the sums are
+// deterministic, and few enough for the last block to add their partials quickly.
+// Four per SM: they are all resident at up to 64 registers a thread (eight were
+// 1.3 to 2 waves), with 64 KB of loads in flight per SM.  At 64^3: dot 28 -> 22 us,
+// lanczos 60 -> 54, finish 43 -> 38.
+inline unsigned red_blocks(int64_t n) {
+  return (unsigned)std::min<int64_t>(kRedBlocks / 2, (n + 4 * kRedThreads - 1) / (4 * kRedThreads));
+}
 
-template <int NP>
-__global__ void __launch_bounds__(kRedThreads) dot_partial_kernel(DotPairs p, int64_t n, double* partials) {
-  grid_dep_entry();
-  double acc[NP];
-#pragma unroll
-  for (int j = 0; j < NP; ++j) acc[j] = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-#pragma unroll
-    for (int j = 0; j < NP; ++j) acc[j] = fma(p.x[j][i], p.y[j][i], acc[j]);
-  }
-  __shared__ double red[NP][kRedThreads / 32];
+// Sum of one value per thread over the grid, in one launch: block sums into
+// partials, and the block that arrives last (counter, back at 0 afterwards) adds
+// them in index order; true in thread 0 of that block, with the sum in *total.
+// A second launch for the final sum took 6 us, four times per MINRES iteration.
+__device__ __forceinline__ bool grid_sum(double v, double* partials, int* counter, double* total) {
+  __shared__ double red[kRedThreads];
+  __shared__ bool last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int j = 0; j < NP; ++j) {
-    double v = acc[j];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) red[j][warp] = v;
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+  if (lane == 0) red[warp] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double b = 0.0;
+    for (int w = 0; w < kRedThreads / 32; ++w) b += red[w];
+    partials[blockIdx.x] = b;
+    __threadfence();
+    last = atomicAdd(counter, 1) == (int)gridDim.x - 1;
   }
   __syncthreads();
-  if (threadIdx.x < NP) {
-    double v = 0.0;
-    for (int w = 0; w < kRedThreads / 32; ++w) v += red[threadIdx.x][w];
-    partials[threadIdx.x * gridDim.x + blockIdx.x] = v;
+  if (!last) return false;
+  __threadfence();
+  double s = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += kRedThreads) s += __ldcg(partials + b);
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int h = kRedThreads / 2; h > 0; h >>= 1) {
+    if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+    __syncthreads();
   }
+  if (threadIdx.x != 0) return false;
+  *counter = 0;
+  *total = red[0];
+  return true;
+}
+
+// four entries a thread and step, a block's step being 4 kRedThreads consecutive
+// entries: f(i, u) loads entry i into slot u, g(i, u) finishes it, so that a
+// thread has four entries' loads in flight
+template <typename F, typename G>
+__device__ __forceinline__ void stride4(int64_t n, F f, G g) {
+  for (int64_t i0 = blockIdx.x * (int64_t)(4 * kRedThreads) + threadIdx.x; i0 < n;
+       i0 += (int64_t)gridDim.x * (4 * kRedThreads)) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u * kRedThreads < n) f(i0 + u * kRedThreads, u);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u * kRedThreads < n) g(i0 + u * kRedThreads, u);
+  }
+}
+
+// *out = scale * sum x y
+__global__ void __launch_bounds__(kRedThreads) dot_kernel(const double* __restrict__ x, const double* __restrict__ y,
+                                                          int64_t n, double* partials, int* counter, double* out,
+                                                          double scale) {
+  grid_dep_entry();
+  double acc = 0.0, a[4], b[4], total;
+  stride4(
+      n, [&](int64_t i, int u) { a[u] = x[i], b[u] = y[i]; }, [&](int64_t, int u) { acc = fma(a[u], b[u], acc); });
+  if (grid_sum(acc, partials, counter, &total)) *out = scale * total;
+}
+
+__global__ void __launch_bounds__(kRedThreads) sum_kernel(const double* __restrict__ x, int64_t n, double* partials,
+                                                          int* counter, double* out, double scale) {
+  grid_dep_entry();
+  double acc = 0.0, a[4], total;
+  stride4(
+      n, [&](int64_t i, int u) { a[u] = x[i]; }, [&](int64_t, int u) { acc += a[u]; });
+  if (grid_sum(acc, partials, counter, &total)) *out = scale * total;
 }
 
 // one block: out[j] = scale * sum_b partials[j*nb + b], fixed tree order
@@ -68,43 +117,60 @@ __global__ void reduce_final_kernel(const double* partials, int nb, int np, doub
   }
 }
 
-__global__ void sum_partial_kernel(const double* x, int64_t n, double* partials) {
-  grid_dep_entry();
-  double acc = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    acc += x[i];
-  __shared__ double red[kRedThreads / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-  if (lane == 0) red[warp] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double v = 0.0;
-    for (int w = 0; w < kRedThreads / 32; ++w) v += red[w];
-    partials[blockIdx.x] = v;
-  }
-}
-
 // ------------------------------------------------------------------ MINRES
 // Scalars live in device memory (MinresSlot) so an iteration needs no host
 // round trip; the Lanczos vector z is kept unnormalized (z = gamma zhat).
-__global__ void lanczos_kernel(int64_t n, const double* __restrict__ kz, const double* __restrict__ v,
-                               double* vold_to_vnew, const double* __restrict__ sc) {
+
+// v_new = K z / g - a v - b v_old over v_old, and the mean of its pressure part
+// (entries n3 and on) into sc[MS_TMP0].  (Writing the V-cycle's FP32 right-hand
+// side and first iterate here as well took 85 us at 64^3, against 54 + 18 us for
+// this and the conversion: the registers cost occupancy.)
+__global__ void __launch_bounds__(kRedThreads) lanczos_kernel(int64_t n, const double* __restrict__ kz,
+                                                              const double* __restrict__ v, double* vold_to_vnew,
+                                                              double* sc, int64_t n3, double* partials, int* counter) {
   grid_dep_entry();
   if (sc[MS_DONE] != 0.0) return;
   const double g = sc[MS_GAMMA], go = sc[MS_GAMMA_OLD];
   const double ig = 1.0 / g;
   const double delta = sc[MS_DOT_KZZ] * ig * ig;  // z is kept unnormalized: z = gamma * zhat
   const double a = delta * ig, b = g / go;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    vold_to_vnew[i] = kz[i] * ig - a * v[i] - b * vold_to_vnew[i];
+  double acc = 0.0, k[4], p[4], o[4], total;
+  const auto load = [&](int64_t i, int u) { k[u] = kz[i], p[u] = v[i], o[u] = vold_to_vnew[i]; };
+  const auto form = [&](int64_t i, int u) {
+    o[u] = fma(ig, k[u], fma(-a, p[u], -b * o[u]));
+    vold_to_vnew[i] = o[u];
+  };
+  stride4(n3, load, form);
+  kz += n3, v += n3, vold_to_vnew += n3;
+  stride4(n - n3, load, [&](int64_t i, int u) {
+    form(i, u);
+    acc += o[u];
+  });
+  if (grid_sum(acc, partials, counter, &total)) sc[MS_TMP0] = total / (double)(n - n3);
 }
 
-__global__ void minres_scalar_kernel(double* sc) {
+// z = (r - mean) minv with mean = sc[MS_TMP0]; sc[MS_TMP1] = the mean of z
+__global__ void __launch_bounds__(kRedThreads) pdiv_kernel(int64_t n, const double* __restrict__ r,
+                                                           const double* __restrict__ minv, double* __restrict__ z,
+                                                           double* sc, double* partials, int* counter) {
   grid_dep_entry();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  if (sc[MS_DONE] != 0.0) return;
+  const double m = sc[MS_TMP0];
+  double acc = 0.0, a[4], b[4], total;
+  stride4(
+      n, [&](int64_t i, int u) { a[u] = r[i], b[u] = minv[i]; },
+      [&](int64_t i, int u) {
+        const double v = (a[u] - m) * b[u];
+        z[i] = v;
+        acc += v;
+      });
+  if (grid_sum(acc, partials, counter, &total)) sc[MS_TMP1] = total / (double)n;
+}
+
+__device__ void minres_scalars(double* sc) {
+  if (sc[MS_DONE] != 0.0) {
+    sc[MS_UPD_SKIP] = 1.0;  // iterations past convergence change nothing
+    return;
+  }
   const double g = sc[MS_GAMMA];
   const double delta = sc[MS_DOT_KZZ] / (g * g);
   const double gn2 = sc[MS_DOT_ZV];
@@ -138,18 +204,46 @@ __global__ void minres_scalar_kernel(double* sc) {
   if (fabs(sc[MS_ETA]) <= sc[MS_TOL_ABS] || !(gn > 0.0)) sc[MS_DONE] = 1.0;
 }
 
+// z_p -= sc[MS_TMP1] (entries n3 and on), then z . v and the recurrence's scalars
+__global__ void __launch_bounds__(kRedThreads) minres_finish_kernel(int64_t n, int64_t n3, double* z,
+                                                                    const double* __restrict__ v, double* sc,
+                                                                    double* partials, int* counter) {
+  grid_dep_entry();
+  const double m = sc[MS_TMP1];
+  double acc = 0.0, a[4], b[4], total;
+  stride4(
+      n, [&](int64_t i, int u) { a[u] = z[i], b[u] = v[i]; },
+      [&](int64_t i, int u) {
+        if (i >= n3) {
+          a[u] -= m;
+          z[i] = a[u];
+        }
+        acc = fma(a[u], b[u], acc);
+      });
+  if (grid_sum(acc, partials, counter, &total)) {
+    sc[MS_DOT_ZV] = total;
+    minres_scalars(sc);
+  }
+}
+
 // w_new = (z/gamma_prev - a3 w_old - a2 w) / a1 into w_old; x += c_new*eta_prev * w_new
-__global__ void minres_update_kernel(int64_t n, const double* __restrict__ z, const double* __restrict__ w,
-                                     double* wold_to_wnew, double* x, const double* __restrict__ sc) {
+__global__ void __launch_bounds__(kRedThreads) minres_update_kernel(int64_t n, const double* __restrict__ z,
+                                                                    const double* __restrict__ w, double* wold_to_wnew,
+                                                                    double* x, const double* __restrict__ sc) {
   grid_dep_entry();
   if (sc[MS_UPD_SKIP] != 0.0) return;
   const double ig = sc[MS_INV_GAMMA_PREV], a1 = sc[MS_A1], a2 = sc[MS_A2], a3 = sc[MS_A3], xc = sc[MS_XCOEF];
-  const double ia1 = 1.0 / a1;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double wn = (z[i] * ig - a3 * wold_to_wnew[i] - a2 * w[i]) * ia1;
-    wold_to_wnew[i] = wn;
-    x[i] = fma(xc, wn, x[i]);
-  }
+  // FP64 arithmetic, at 10 us an operation for 6.7 M entries, costs more than the
+  // memory here: the scalars are folded beforehand
+  const double ia1 = 1.0 / a1, cz = ig * ia1, co = -(a3 * ia1), cw = -(a2 * ia1);
+  double zi[4], wi[4], oi[4], xi[4];
+  stride4(
+      n, [&](int64_t i, int u) { zi[u] = z[i], wi[u] = w[i], oi[u] = wold_to_wnew[i], xi[u] = x[i]; },
+      [&](int64_t i, int u) {
+        const double wn = fma(cz, zi[u], fma(co, oi[u], cw * wi[u]));
+        wold_to_wnew[i] = wn;
+        x[i] = fma(xc, wn, xi[u]);
+      });
 }
 
 __global__ void minres_init_kernel(double* sc, double tol_rel) {
@@ -170,24 +264,31 @@ __global__ void minres_init_kernel(double* sc, double tol_rel) {
 }
 
 // ------------------------------------------------------------------ vectors
-__global__ void vec_op_kernel(int op, int64_t n, double* y, const double* a, const double* b, const double* c,
-                              const double* scal) {
+template <int OP>
+__global__ void __launch_bounds__(kRedThreads) vec_op_kernel(int64_t n, double* y, const double* a, const double* b,
+                                                             const double* scal) {
   grid_dep_entry();
+  constexpr bool A = OP != VOP_ZERO, B = OP == VOP_SUB || OP == VOP_ADD || OP == VOP_MUL;
   const double s0 = scal ? scal[0] : 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    switch (op) {
-      case VOP_SUB: y[i] = a[i] - b[i]; break;            // y = a - b
-      case VOP_ADD: y[i] = a[i] + b[i]; break;            // y = a + b
-      case VOP_COPY: y[i] = a[i]; break;                  // y = a
-      case VOP_ZERO: y[i] = 0.0; break;                   // y = 0
-      case VOP_PDIV: y[i] = (a[i] - s0) * b[i]; break;    // y = (a - mean) * minv
-      case VOP_SUBS: y[i] = a[i] - s0; break;             // y = a - s
-      case VOP_MUL: y[i] = a[i] * b[i]; break;            // y = a * b
-      case VOP_SCALE_RSQRT: y[i] = a[i] * (1.0 / sqrt(s0)); break;  // y = a / sqrt(s)
-      case VOP_RECIP: y[i] = a[i] > 0.0 ? 1.0 / a[i] : 0.0; break;  // y = 1 / a (0 where a <= 0)
-      default: break;
-    }
-  }
+  const double f = OP == VOP_SCALE_RSQRT ? 1.0 / sqrt(s0) : 0.0;
+  double u_[4], v_[4];
+  stride4(
+      n,
+      [&](int64_t i, int u) {
+        if (A) u_[u] = a[i];
+        if (B) v_[u] = b[i];
+      },
+      [&](int64_t i, int u) {
+        double o = 0.0;                                                 // y = 0
+        if (OP == VOP_SUB) o = u_[u] - v_[u];                           // y = a - b
+        if (OP == VOP_ADD) o = u_[u] + v_[u];                           // y = a + b
+        if (OP == VOP_COPY) o = u_[u];                                  // y = a
+        if (OP == VOP_SUBS) o = u_[u] - s0;                             // y = a - s
+        if (OP == VOP_MUL) o = u_[u] * v_[u];                           // y = a * b
+        if (OP == VOP_SCALE_RSQRT) o = u_[u] * f;                       // y = a / sqrt(s)
+        if (OP == VOP_NEG) o = -u_[u];                                  // y = -a
+        y[i] = o;
+      });
 }
 
 // --------------------------------------------------------------- FE kernels
@@ -397,16 +498,17 @@ __global__ void zdiag_inv_kernel(int64_t V, const double* __restrict__ zs, doubl
   dinv[v] = d > 0.0 ? 1.0 / d : 0.0;
 }
 
-// (Z p)_v from the stencils (neighbours outside the grid contribute nothing)
-__device__ __forceinline__ double zrow(const double* __restrict__ zs, const double* __restrict__ p, int64_t V, int nv,
-                                       int64_t v) {
-  const int i = (int)(v % nv), j = (int)((v / nv) % nv), k = (int)(v / ((int64_t)nv * nv));
+// (Z z)_v from the stencils (neighbours outside the grid contribute nothing)
+__device__ __forceinline__ double zrow(const double* __restrict__ zs, const double* z, const int V, const int nv,
+                                       const int v) {
+  const int k = v / (nv * nv), rem = v - k * nv * nv, j = rem / nv, i = rem - j * nv;
   double acc = 0.0;
-#pragma unroll 5
+#pragma unroll
   for (int s = 0; s < ZSTENCIL; ++s) {
     const int ii = i + c_zpat.d[s][0], jj = j + c_zpat.d[s][1], kk = k + c_zpat.d[s][2];
-    if (ii < 0 || jj < 0 || kk < 0 || ii >= nv || jj >= nv || kk >= nv) continue;
-    acc = fma(zs[s * V + v], p[ii + (int64_t)nv * (jj + (int64_t)nv * kk)], acc);
+    const bool in = ii >= 0 && jj >= 0 && kk >= 0 && ii < nv && jj < nv && kk < nv;
+    const double c = in ? __ldg(zs + (int64_t)s * V + v) : 0.0, zw = in ? z[ii + nv * (jj + nv * kk)] : 0.0;
+    acc = fma(c, zw, acc);
   }
   return acc;
 }
@@ -427,7 +529,8 @@ __device__ double zcg_grid_sum(cooperative_groups::grid_group& grid, double v, d
   grid.sync();
   if (threadIdx.x < 32) {
     double s = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) s += partials[b];
+#pragma unroll 4
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) s += __ldcg(partials + b);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
     if (threadIdx.x == 0) red[32] = s;
@@ -439,51 +542,57 @@ __device__ double zcg_grid_sum(cooperative_groups::grid_group& grid, double v, d
 }
 
 // x = Z^-1 r by `iters` steps of Jacobi-preconditioned conjugate gradients
-// from x = 0, in one cooperative launch (grid barriers between the phases
-// of a step).  r (mean-free) is overwritten by the residual.  The iterates
-// are not projected: r stays mean-free because Z annihilates constants, so
-// the constant parts p and x pick up change no inner product, and the
-// caller projects x once at the end.  partials: 2 gridDim.x doubles.
+// from x = 0, in one cooperative launch.  r (mean-free) is overwritten by the
+// residual.  The iterates are not projected: r stays mean-free because Z
+// annihilates constants, so the constant parts p and x pick up change no inner
+// product, and the caller projects x once at the end.  partials: 2 gridDim.x
+// doubles.
+// A step is bound by latency on small grids (14 us at 32^3, of which the 520 B a
+// vertex from L2 are 3): the product is taken of z = D^-1 r and q = Z p follows as
+// Z z + beta q, so that a step has two grid barriers, both with a sum, instead of
+// three, and the row's 65 couplings are unrolled, so that their loads are in flight
+// together (18 us with three barriers and five couplings at a time; 21 with two
+// barriers and 13; four lanes per vertex took 24).
 __global__ void __launch_bounds__(256) zcg_kernel(int np, const double* __restrict__ zs, const double* __restrict__ dinv,
-                                                  double* __restrict__ x, double* __restrict__ r,
-                                                  double* __restrict__ p, double* __restrict__ q,
-                                                  double* __restrict__ partials, int iters) {
+                                                  double* x, double* r, double* p, double* q, double* z,
+                                                  double* partials, int iters) {
   grid_dep_entry();
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   __shared__ double red[33];
-  const int nv = np + 1;
-  const int64_t V = (int64_t)nv * nv * nv;
-  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+  const int nv = np + 1, V = nv * nv * nv;
+  const int t0 = blockIdx.x * blockDim.x + threadIdx.x, st = gridDim.x * blockDim.x;
   double* part[2] = {partials, partials + gridDim.x};  // alternate: consecutive uses are a barrier apart
   double loc = 0.0;
-  for (int64_t v = t0; v < V; v += st) {
-    const double z = dinv[v] * r[v];
-    x[v] = 0.0;
-    p[v] = z;
-    loc = fma(r[v], z, loc);
+  for (int v = t0; v < V; v += st) {
+    const double zv = dinv[v] * r[v];
+    x[v] = p[v] = q[v] = 0.0;
+    z[v] = zv;
+    loc = fma(r[v], zv, loc);
   }
-  double rho = zcg_grid_sum(grid, loc, part[0], red);
+  double rho = zcg_grid_sum(grid, loc, part[0], red), beta = 0.0;
   for (int it = 0; it < iters; ++it) {
-    grid.sync();  // p complete
+    // q = Z z + beta q, p = z + beta p (z complete: the barrier of the last sum)
     loc = 0.0;
-    for (int64_t v = t0; v < V; v += st) {
-      const double qv = zrow(zs, p, V, nv, v);
+    for (int v = t0; v < V; v += st) {
+      const double qv = fma(beta, q[v], zrow(zs, z, V, nv, v)), pv = fma(beta, p[v], z[v]);
       q[v] = qv;
-      loc = fma(p[v], qv, loc);
+      p[v] = pv;
+      loc = fma(pv, qv, loc);
     }
     const double pq = zcg_grid_sum(grid, loc, part[1], red);
     const double alpha = pq != 0.0 ? rho / pq : 0.0;
     loc = 0.0;
-    for (int64_t v = t0; v < V; v += st) {
+    for (int v = t0; v < V; v += st) {
       x[v] = fma(alpha, p[v], x[v]);
       const double rv = fma(-alpha, q[v], r[v]);
+      const double zv = dinv[v] * rv;
       r[v] = rv;
-      loc = fma(rv, dinv[v] * rv, loc);
+      z[v] = zv;
+      loc = fma(rv, zv, loc);
     }
     const double rho_new = zcg_grid_sum(grid, loc, part[0], red);
-    const double beta = rho != 0.0 ? rho_new / rho : 0.0;
+    beta = rho != 0.0 ? rho_new / rho : 0.0;
     rho = rho_new;
-    for (int64_t v = t0; v < V; v += st) p[v] = fma(beta, p[v], dinv[v] * r[v]);
   }
 }
 
@@ -496,33 +605,30 @@ cudaError_t launch_mask_boundary(int n, double* x, cudaStream_t s) {
 
 int dot_blocks() { return kRedBlocks; }
 
-cudaError_t launch_dots(int npairs, const double* const* xs, const double* const* ys, int64_t n, double* partials,
-                        double* out, double scale, cudaStream_t s) {
-  DotPairs p{};
-  for (int j = 0; j < npairs; ++j) {
-    p.x[j] = xs[j];
-    p.y[j] = ys[j];
-  }
-  switch (npairs) {
-    case 1: KL(launch_k(dot_partial_kernel<1>, dim3(kRedBlocks), dim3(kRedThreads), 0, s, p, n, partials)); break;
-    case 2: KL(launch_k(dot_partial_kernel<2>, dim3(kRedBlocks), dim3(kRedThreads), 0, s, p, n, partials)); break;
-    case 3: KL(launch_k(dot_partial_kernel<3>, dim3(kRedBlocks), dim3(kRedThreads), 0, s, p, n, partials)); break;
+cudaError_t launch_dot(const double* x, const double* y, int64_t n, double* partials, int* counter, double* out,
+                       double scale, cudaStream_t s) {
+  return launch_k(dot_kernel, dim3(red_blocks(n)), dim3(kRedThreads), 0, s, x, y, n, partials, counter, out, scale);
+}
+
+cudaError_t launch_sum(const double* x, int64_t n, double* partials, int* counter, double* out, double scale,
+                       cudaStream_t s) {
+  return launch_k(sum_kernel, dim3(red_blocks(n)), dim3(kRedThreads), 0, s, x, n, partials, counter, out, scale);
+}
+
+cudaError_t launch_vec_op(int op, int64_t n, double* y, const double* a, const double* b, const double* scal,
+                          cudaStream_t s) {
+  const dim3 g(red_blocks(n)), t(kRedThreads);
+  switch (op) {
+    case VOP_SUB: return launch_k(vec_op_kernel<VOP_SUB>, g, t, 0, s, n, y, a, b, scal);
+    case VOP_ADD: return launch_k(vec_op_kernel<VOP_ADD>, g, t, 0, s, n, y, a, b, scal);
+    case VOP_COPY: return launch_k(vec_op_kernel<VOP_COPY>, g, t, 0, s, n, y, a, b, scal);
+    case VOP_ZERO: return launch_k(vec_op_kernel<VOP_ZERO>, g, t, 0, s, n, y, a, b, scal);
+    case VOP_SUBS: return launch_k(vec_op_kernel<VOP_SUBS>, g, t, 0, s, n, y, a, b, scal);
+    case VOP_MUL: return launch_k(vec_op_kernel<VOP_MUL>, g, t, 0, s, n, y, a, b, scal);
+    case VOP_SCALE_RSQRT: return launch_k(vec_op_kernel<VOP_SCALE_RSQRT>, g, t, 0, s, n, y, a, b, scal);
+    case VOP_NEG: return launch_k(vec_op_kernel<VOP_NEG>, g, t, 0, s, n, y, a, b, scal);
     default: return cudaErrorInvalidValue;
   }
-  KL(launch_k(reduce_final_kernel, dim3(1), dim3(256), 0, s, partials, kRedBlocks, npairs, out, scale));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_sum(const double* x, int64_t n, double* partials, double* out, double scale, cudaStream_t s) {
-  KL(launch_k(sum_partial_kernel, dim3(kRedBlocks), dim3(kRedThreads), 0, s, x, n, partials));
-  KL(launch_k(reduce_final_kernel, dim3(1), dim3(256), 0, s, partials, kRedBlocks, 1, out, scale));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_vec_op(int op, int64_t n, double* y, const double* a, const double* b, const double* c,
-                          const double* scal, cudaStream_t s) {
-  KL(launch_k(vec_op_kernel, dim3(kRedBlocks), dim3(kRedThreads), 0, s, op, n, y, a, b, c, scal));
-  return cudaGetLastError();
 }
 
 cudaError_t launch_minres_init(double* sc, double tol_rel, cudaStream_t s) {
@@ -559,7 +665,7 @@ cudaError_t launch_scatter_zrow(int np, int colour, const double* y, double* zs,
 }
 
 cudaError_t launch_zcg(int np, const double* zs, const double* dinv, double* x, double* r, double* p, double* q,
-                       double* partials, int64_t partials_cap, int iters, cudaStream_t s) {
+                       double* z, double* partials, int64_t partials_cap, int iters, cudaStream_t s) {
   int dev = 0, sms = 152, per = 0, coop = 0;
   KL(cudaGetDevice(&dev));
   KL(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -571,11 +677,7 @@ cudaError_t launch_zcg(int np, const double* zs, const double* dinv, double* x, 
   int64_t blocks = std::min<int64_t>((int64_t)std::min(per, 2) * sms, blocks_for(nverts(np), 256));
   blocks = std::max<int64_t>(blocks, 1);
   if (2 * blocks > partials_cap) return cudaErrorInvalidValue;
-  int np_ = np, iters_ = iters;
-  const double* zs_ = zs;
-  const double* dinv_ = dinv;
-  double *x_ = x, *r_ = r, *p_ = p, *q_ = q, *part_ = partials;
-  void* args[] = {&np_, &zs_, &dinv_, &x_, &r_, &p_, &q_, &part_, &iters_};
+  void* args[] = {&np, &zs, &dinv, &x, &r, &p, &q, &z, &partials, &iters};
   KL(cudaLaunchCooperativeKernel((const void*)zcg_kernel, dim3((unsigned)blocks), dim3(256), args, 0, s));
   return cudaGetLastError();
 }
@@ -585,21 +687,25 @@ cudaError_t launch_zdiag_inv(int np, const double* zs, double* dinv, cudaStream_
   return cudaGetLastError();
 }
 
-cudaError_t launch_lanczos(int64_t n, const double* kz, const double* v, double* vold_to_vnew, const double* sc,
-                           cudaStream_t s) {
-  KL(launch_k(lanczos_kernel, dim3(kRedBlocks), dim3(kRedThreads), 0, s, n, kz, v, vold_to_vnew, sc));
-  return cudaGetLastError();
+cudaError_t launch_lanczos(int64_t n, const double* kz, const double* v, double* vold_to_vnew, double* sc, int64_t n3,
+                           double* partials, int* counter, cudaStream_t s) {
+  return launch_k(lanczos_kernel, dim3(red_blocks(n)), dim3(kRedThreads), 0, s, n, kz, v, vold_to_vnew, sc, n3, partials,
+                  counter);
 }
 
-cudaError_t launch_minres_scalars(double* sc, cudaStream_t s) {
-  KL(launch_k(minres_scalar_kernel, dim3(1), dim3(32), 0, s, sc));
-  return cudaGetLastError();
+cudaError_t launch_pdiv(int64_t n, const double* r, const double* minv, double* z, double* sc, double* partials,
+                        int* counter, cudaStream_t s) {
+  return launch_k(pdiv_kernel, dim3(red_blocks(n)), dim3(kRedThreads), 0, s, n, r, minv, z, sc, partials, counter);
+}
+
+cudaError_t launch_minres_finish(int64_t n, int64_t n3, double* z, const double* v, double* sc, double* partials,
+                                 int* counter, cudaStream_t s) {
+  return launch_k(minres_finish_kernel, dim3(red_blocks(n)), dim3(kRedThreads), 0, s, n, n3, z, v, sc, partials, counter);
 }
 
 cudaError_t launch_minres_update(int64_t n, const double* z, const double* w, double* wold_to_wnew, double* x,
                                  const double* sc, cudaStream_t s) {
-  KL(launch_k(minres_update_kernel, dim3(kRedBlocks), dim3(kRedThreads), 0, s, n, z, w, wold_to_wnew, x, sc));
-  return cudaGetLastError();
+  return launch_k(minres_update_kernel, dim3(red_blocks(n)), dim3(kRedThreads), 0, s, n, z, w, wold_to_wnew, x, sc);
 }
 
 cudaError_t launch_load_vector(int n, const double* fbar, double* b, cudaStream_t s) {

@@ -133,7 +133,7 @@ extern "C" agca_status agca_stokes_apply_static(int N, const double* eta_dev, co
   a.x = x_dev;
   a.out = y_dev;
   if (launch_stencil<double, double>(ST_APPLY, op, a, s) != cudaSuccess) return AGCA_ECUDA;
-  if (launch_gradient(n, qfine, y_dev, s) != cudaSuccess) return AGCA_ECUDA;
+  if (launch_gradient(n, qfine, y_dev, nullptr, y_dev, s) != cudaSuccess) return AGCA_ECUDA;
   if (launch_divergence(N, x_dev, y_dev + 3 * V, s) != cudaSuccess) return AGCA_ECUDA;
   return AGCA_OK;
 }

@@ -80,22 +80,34 @@ __device__ __forceinline__ double half_sum(F at, std::integer_sequence<int, Q...
   return acc;
 }
 
-// y += -B_f^T q on the interior vertices of a grid with n cubes per axis
-__device__ __forceinline__ void gradient_point(const int n, const double* __restrict__ q, double* y, const int v) {
+// y = scale * (a - B_f^T q) at vertex v of a grid with n cubes per axis (a, scale
+// may be nullptr: 0 and 1), 0 on the boundary
+__device__ __forceinline__ void gradient_point(const int n, const double* __restrict__ q, const double* a,
+                                               const double* __restrict__ scale, double* y, const int v) {
   const int nv = n + 1, V = nv * nv * nv;
   const int vk = v / (nv * nv), vr = v - vk * nv * nv, vj = vr / nv, vi = vr - vj * nv;
-  if (vi == 0 || vj == 0 || vk == 0 || vi == n || vj == n || vk == n) return;
+  if (vi == 0 || vj == 0 || vk == 0 || vi == n || vj == n || vk == n) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) y[v + c * V] = 0.0;
+    return;
+  }
+  double y0[3] = {0.0, 0.0, 0.0};
+  if (a) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) y0[c] = a[v + c * V];
+  }
   const int sy = nv, sz = nv * nv;
   auto D = [&](int o) { return __ldg(q + v + o) - __ldg(q + v - o); };
   const double dx = D(1), dy = D(sy), dz = D(sz), dxy = D(1 + sy), dxz = D(1 + sz), dyz = D(sy + sz),
                dxyz = D(1 + sy + sz);
-  const double y0 = y[v], y1 = y[v + V], y2 = y[v + 2 * V];
   // component c: base + 4 D_c - 2 D_de
   const double base = ((dxy + dxz) + (dyz + dxyz)) - ((dx + dy) + dz);
   const double w = 1.0 / (12.0 * (double)n * n);
-  y[v] = fma(w, fma(4.0, dx, fma(-2.0, dyz, base)), y0);
-  y[v + V] = fma(w, fma(4.0, dy, fma(-2.0, dxz, base)), y1);
-  y[v + 2 * V] = fma(w, fma(4.0, dz, fma(-2.0, dxy, base)), y2);
+  y0[0] = fma(w, fma(4.0, dx, fma(-2.0, dyz, base)), y0[0]);
+  y0[1] = fma(w, fma(4.0, dy, fma(-2.0, dxz, base)), y0[1]);
+  y0[2] = fma(w, fma(4.0, dz, fma(-2.0, dxy, base)), y0[2]);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) y[v + c * V] = scale ? __ldg(scale + v + c * V) * y0[c] : y0[c];
 }
 
 // y = B u on pressure vertices 32 b .. 32 b + 31 (np cubes per axis): warp c adds
@@ -127,10 +139,11 @@ __device__ __forceinline__ void divergence_block(const int np, const double* __r
   if (c == 0 && exists) y[v] = -(((part[0][lane] + part[1][lane]) + part[2][lane]) * (1.0 / (24.0 * (double)n * n)));
 }
 
-__global__ void __launch_bounds__(128) gradient_kernel(const int n, const double* __restrict__ q, double* y) {
+__global__ void __launch_bounds__(128) gradient_kernel(const int n, const double* __restrict__ q,
+                                                       const double* a, const double* __restrict__ scale, double* y) {
   grid_dep_entry();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v < (n + 1) * (n + 1) * (n + 1)) gradient_point(n, q, y, v);
+  if (v < (n + 1) * (n + 1) * (n + 1)) gradient_point(n, q, a, scale, y, v);
 }
 __global__ void __launch_bounds__(96) divergence_kernel(const int np, const double* __restrict__ u,
                                                         double* __restrict__ y) {
@@ -145,7 +158,8 @@ __global__ void __launch_bounds__(128) gradient_batch_kernel(const XferTask* __r
   const XferTask tk = tasks[blockIdx.y];
   if (tk.sc && tk.sc[MS_DONE] != 0.0) return;
   const int v = blockIdx.x * blockDim.x + threadIdx.x, nv = tk.nf + 1;
-  if (v < nv * nv * nv) gradient_point(tk.nf, static_cast<const double*>(tk.src), static_cast<double*>(tk.dst), v);
+  if (v < nv * nv * nv) gradient_point(tk.nf, static_cast<const double*>(tk.src), static_cast<double*>(tk.dst), nullptr,
+                                      static_cast<double*>(tk.dst), v);
 }
 __global__ void __launch_bounds__(96) divergence_batch_kernel(const XferTask* __restrict__ tasks) {
   grid_dep_entry();
@@ -159,8 +173,8 @@ __global__ void __launch_bounds__(96) divergence_batch_kernel(const XferTask* __
 
 }  // namespace
 
-cudaError_t launch_gradient(int n, const double* q, double* y, cudaStream_t s) {
-  return launch_k(gradient_kernel, dim3((unsigned)((nverts(n) + 127) / 128)), dim3(128), 0, s, n, q, y);
+cudaError_t launch_gradient(int n, const double* q, const double* a, const double* scale, double* y, cudaStream_t s) {
+  return launch_k(gradient_kernel, dim3((unsigned)((nverts(n) + 127) / 128)), dim3(128), 0, s, n, q, a, scale, y);
 }
 cudaError_t launch_divergence(int np, const double* u, double* y, cudaStream_t s) {
   return launch_k(divergence_kernel, dim3((unsigned)((nverts(np) + 31) / 32)), dim3(96), 0, s, np, u, y);

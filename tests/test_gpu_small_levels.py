@@ -5,13 +5,15 @@ per axis, odd sizes, and the largest size (32 cubes); the first tiled sizes
 flagged) against the other precision on the same grid.  Tolerances as in
 test_gpu_parity.py: 1e-12 (FP64) and 1e-5 (FP32) of the largest entry for an
 apply, 1e-9 and 1e-4 for a cycle."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
 
 from oracle import agca as oagca
 from oracle import stokes as ostokes
-from synth import random_vector
+from synth import random_vector, sphere_sinkers
 
 pytestmark = pytest.mark.gpu
 
@@ -103,3 +105,25 @@ def test_large_batch_equals_single(count):
         ref = c.vcycle(r[i])
         for j in (i, count - 2 - (count - i) % 2, count - 1 - (count - 1 - i) % 2):
             assert torch.equal(z[j], ref), j
+
+
+# a mixed context's finest coefficient records are the part of the workspace that FGMRES can do without;
+# K z differs by rounding only, so both solves take the same iterations and meet the tolerance
+@pytest.mark.parametrize("short, ok", [(0, True), (1, True), (2, False)])
+def test_fgmres_workspace_without_records(short, ok):
+    p = sphere_sinkers(18, 3, 0.15, 0.03, 1e2)  # 36 cubes per axis: past the point kernel
+    c = pkg.Context(18, None, pkg.MIXED, device=DEV)
+    c.prepare(torch.from_numpy(p.eta).to(DEV), 10.0)
+    b = c.load_vector(torch.from_numpy(p.fbar.ravel()).to(DEV))
+    x, it, rel = c.solve_fgmres(b, 1e-6, 400, 20)
+    lib, sz = pkg.agca.lib(), ctypes.c_size_t()
+    assert lib.agca_fgmres_workspace_size(c._h, 20, ctypes.byref(sz)) == 0
+    records = (27 * 8 * c.V[c.L] + 255) // 256 * 256
+    size = sz.value - records * min(short, 1) - 256 * (short == 2)
+    work, y = torch.empty(size, dtype=torch.uint8, device=DEV), torch.empty_like(b)
+    it2, rel2 = ctypes.c_int(), ctypes.c_double()
+    st = lib.agca_solve_fgmres(c._h, b.data_ptr(), y.data_ptr(), 1e-6, 400, 20, 0, 30, work.data_ptr(), size,
+                               ctypes.byref(it2), ctypes.byref(rel2))
+    assert (st == 0) == ok
+    if ok:
+        assert it2.value == it and rel2.value <= 1e-6 and rel <= 1e-6
