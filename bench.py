@@ -52,7 +52,7 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # stencil launch, mean over the four launches of one V-cycle, from one ncu
 # capture of the current kernels at 64^3 pressure cubes scaled by the vertex
 # count (x 7.907) to 128^3 (None where no capture of the current kernel exists)
-FINE_STENCIL_DRAM_BYTES = {("logbump", 128, "f64"): 5.298e9, ("logbump", 128, "f32"): 1.059e9}
+FINE_STENCIL_DRAM_BYTES = {("logbump", 128, "f64"): 5.40e9, ("logbump", 128, "f32"): 1.128e9}
 
 
 def _dist():

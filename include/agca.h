@@ -219,7 +219,9 @@ agca_status agca_solve(agca_ctx* ctx, const double* b_dev, double* x_dev, double
  * cooperative launch per solve; the device must support cooperative
  * launches, else the call fails with AGCA_ECUDA).
  * work_dev: caller-owned device memory of agca_fgmres_workspace_size bytes
- * (256-byte aligned; holds the 2 restart + 1 Krylov vectors and Z).  x is
+ * (256-byte aligned; holds the 2 restart + 1 Krylov vectors and Z, and in
+ * mixed contexts the finest level's coefficient records, 27 doubles a vertex:
+ * a workspace smaller by these also serves, with slower FP64 products).  x is
  * overwritten (initial guess 0; pressure returned mean-free).  *iters,
  * *relres (host): iterations and the final true relative residual.
  * Synchronizes (once per iteration).  AGCA_ENOTCONV above the tolerance
@@ -244,10 +246,10 @@ agca_status agca_adjoint_gradient(agca_ctx* ctx, const double* x_dev, const doub
  * per axis, for callers that cannot allocate device memory themselves (code
  * whose device memory belongs to another allocator or pool it must not
  * bypass, or loops that cannot afford an allocation).  No context, workspace
- * or allocation: the operator's two fine-grid scratch fields live in a fixed
+ * or allocation: the operator's fine-grid scratch field lives in a fixed
  * device array inside the library, held by every GPU that loads it until the
  * process exits.  The paper has no counterpart of this entry point.
- *   N: 1..32 (AGCA_EINVAL beyond: the scratch holds 2 (2N+1)^3 doubles);
+ *   N: 1..32 (AGCA_EINVAL beyond: the scratch holds (2N+1)^3 doubles);
  *   eta: double[6 (2N)^3] element viscosities (as agca_set_viscosity);
  *   x, y: double[3 (2N+1)^3 + (N+1)^3] Stokes vectors as agca_stokes_apply;
  *   cuda_stream: cudaStream_t (NULL = legacy default stream).
@@ -266,8 +268,8 @@ agca_status agca_stokes_apply_static(int N, const double* eta_dev, const double*
 
 /* Autotuner: for every level >= 2 and V-cycle stencil mode (0 apply,
  * 1 residual, 2 first and 3 later Chebyshev steps, 4 pre-smoothing step from
- * zero), time the candidate tile shapes (block rows 8/12/16 in FP32, 8 in
- * FP64; z-chunks 1..64) with CUDA events on the context stream, reps
+ * zero), time the candidate tile shapes (8 block rows; z-chunks 1..64 and
+ * those that fill whole waves) with CUDA events on the context stream, reps
  * launches each, and keep the fastest for the context's later launches.
  * cache_path (nullable): text file of earlier results, read first and
  * rewritten.  Uses the cycle vectors as scratch.  Synchronizes. */
@@ -275,12 +277,13 @@ agca_status agca_autotune(agca_ctx* ctx, int reps, const char* cache_path);
 /* The tile shape in use for (level, mode): block rows and z-chunk (0 = automatic). */
 agca_status agca_tile_config(const agca_ctx* ctx, int level, int mode, int* by, int* zch);
 /* Set the tile shape of (level, mode) by hand (mode 5: the Stokes operator
- * on the finest level): by = 8, 12 or 16 block rows (12 and 16 in FP32 only),
+ * on the finest level): by = 8, 12 or 16 block rows (12 and 16 in FP32 only;
+ * the tiles of the V-cycle have one number of rows, whatever by says),
  * zch = z-chunk in vertex planes (0 = automatic, at most 4096).  Results do
  * not depend on the tile shape: every vertex sums its element contributions
  * in the same order.  Host only; AGCA_EINVAL for other values. */
 agca_status agca_set_tile_config(agca_ctx* ctx, int level, int mode, int by, int zch);
-/* The tile grid the stencil kernels use on a grid of n cubes per axis with
+/* The tile grid of the per-cube stencil kernel on a grid of n cubes per axis with
  * by block rows and z-chunk request zch (0 = automatic): out[0..6] = wide
  * strips in x, wide tile rows in y, narrow strips in x, narrow tile rows in
  * y, first vertex column of the narrow strips, z-chunks, vertex planes per
@@ -310,9 +313,9 @@ agca_status agca_profile_fine(agca_ctx* ctx, int enable, double* ms, double* byt
  * Batched solves of many independent problems (uneven sizes allowed).
  * Every problem keeps its own hierarchy; the MINRES iterations of all
  * problems run in lockstep, each launch covering every problem: the stencil
- * launches are persistent (every CTA walks the flattened (problem, tile)
- * work list) and one lockstep iteration pair is captured once as a CUDA graph
- * (when the stream is not the legacy default stream) and replayed.
+ * launches walk the flattened (problem, tile) work list, and one lockstep
+ * iteration pair is captured once as a CUDA graph (when the stream is not the
+ * legacy default stream) and replayed.
  * Converged problems are skipped on the device.  The batch owns its
  * sub-contexts; device memory is bound by the caller as for one context.
  * ---------------------------------------------------------------------- */
