@@ -90,7 +90,7 @@ struct agca_ctx {
   double* sc = nullptr;
   double* partials = nullptr;
   int* status = nullptr;
-  int* counter = nullptr;  // of the one-launch reductions: 0 between launches
+  int* counter = nullptr;  // of the one-launch reductions: zeroed by agca_setup, 0 between launches
   int64_t* totals = nullptr;
   int32_t* block_counts = nullptr;
   double nu = 10.0;
@@ -661,15 +661,18 @@ agca_status minres_impl(agca_ctx* ctx, const double* b, double* d, double tol_re
     s = ctx->stream = own;
     ctx->minres_launches[gi] = ctx->launches - l0;
     ctx->launches = l0;
-    if (st != AGCA_OK) {
-      if (g) cudaGraphDestroy(g);
-      return st;
+    cudaError_t ie = ee;
+    if (st == AGCA_OK && ee == cudaSuccess) ie = cudaGraphInstantiate(&ctx->minres_graph[gi], g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (st == AGCA_OK && ie == cudaSuccess) {
+      ctx->minres_key[gi] = d;
+    } else if (legacy) {  // launch directly
+      cudaGetLastError();
+      ctx->minres_graph[gi] = nullptr;
+      graph = false;
+    } else {
+      return st != AGCA_OK ? st : ctx->fail(AGCA_ECUDA, std::string("MINRES graph: ") + cudaGetErrorString(ie));
     }
-    if (ee != cudaSuccess) return ctx->fail(AGCA_ECUDA, std::string("MINRES capture: ") + cudaGetErrorString(ee));
-    const cudaError_t ie = cudaGraphInstantiate(&ctx->minres_graph[gi], g, 0);
-    cudaGraphDestroy(g);
-    if (ie != cudaSuccess) return ctx->fail(AGCA_ECUDA, std::string("MINRES graph: ") + cudaGetErrorString(ie));
-    ctx->minres_key[gi] = d;
   }
   const int check_every = ctx->check_every;
   int it = 0;
@@ -1687,7 +1690,6 @@ agca_status agca_bind_workspace(agca_ctx* ctx, void* dev_ptr, size_t bytes) {
   ctx->ws = static_cast<char*>(dev_ptr);
   ctx->ws_bytes = bytes;
   carve_workspace(ctx, ctx->ws);
-  CK(cudaMemsetAsync(ctx->counter, 0, sizeof(int), ctx->stream));
   ctx->have_eta = ctx->flagged = ctx->setup_done = false;
   ctx->gs = nullptr;
   return AGCA_OK;
@@ -1795,7 +1797,7 @@ agca_status agca_setup(agca_ctx* ctx) {
   cudaStream_t s = ctx->stream;
   const int L = ctx->L;
   const bool mixed = ctx->prec == AGCA_MIXED;
-  CK(cudaMemsetAsync(ctx->status, 0, sizeof(int), s));
+  CK(cudaMemsetAsync(ctx->status, 0, 2 * sizeof(int), s));  // and counter, the int behind it
   // Galerkin matrices, finest to coarsest (Eq. 2.7)
   for (int l = L - 1; l >= 1; --l) {
     Level& lc = ctx->lev[l];
