@@ -649,6 +649,7 @@ agca_status minres_impl(agca_ctx* ctx, const double* b, double* d, double tol_re
     const int64_t l0 = ctx->launches;
     cudaGraph_t g = nullptr;
     const cudaStream_t own = ctx->stream;
+    double* const roles[6] = {vold, v, z, zn, wold, w};
     if (legacy) s = ctx->stream = ctx->cap;
     const cudaError_t be = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     agca_status st = AGCA_OK;
@@ -666,9 +667,11 @@ agca_status minres_impl(agca_ctx* ctx, const double* b, double* d, double tol_re
     if (g) cudaGraphDestroy(g);
     if (st == AGCA_OK && ie == cudaSuccess) {
       ctx->minres_key[gi] = d;
-    } else if (legacy) {  // launch directly
+    } else if (legacy) {  // launch directly, from the roles that an iteration captured before the failure exchanged
       cudaGetLastError();
+      ctx->err.clear();
       ctx->minres_graph[gi] = nullptr;
+      vold = roles[0], v = roles[1], z = roles[2], zn = roles[3], wold = roles[4], w = roles[5];
       graph = false;
     } else {
       return st != AGCA_OK ? st : ctx->fail(AGCA_ECUDA, std::string("MINRES graph: ") + cudaGetErrorString(ie));

@@ -1,0 +1,205 @@
+// Host side of the library (capi.cu) against fakes of the CUDA runtime and of
+// the kernel launchers: "device" memory is host memory, launches do nothing but
+// set the scalars that the host reads, and a launch or a capture can be made to
+// fail.  One scenario per run (its name is the argument); "ok" on success.
+#include <stdio.h>
+#include <stdlib.h>
+#include <string.h>
+
+#include <new>
+#include <string>
+#include <vector>
+
+#include "../paper_2511_13109_gb300/csrc/agca_internal.cuh"
+
+// ------------------------------------------------------------- fake CUDA runtime
+static bool g_capturing = false;
+static int g_graph_launches = 0;
+static double* g_sc = nullptr;  // scalars of the last launch_minres_init
+static bool legacy(cudaStream_t s) { return s == nullptr || s == cudaStreamLegacy; }
+
+extern "C" {
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+  if (!g_capturing) memmove(d, s, n);
+  return cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
+  if (!g_capturing) memset(d, v, n);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+const char* cudaGetErrorString(cudaError_t) { return "fake error"; }
+cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return *s = (cudaStream_t)0x100, cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* st) {
+  return *st = cudaStreamCaptureStatusNone, cudaSuccess;
+}
+cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode) {
+  if (legacy(s)) return cudaErrorStreamCaptureUnsupported;
+  g_capturing = true;
+  return cudaSuccess;
+}
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) {
+  g_capturing = false;
+  return *g = (cudaGraph_t)0x200, cudaSuccess;
+}
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) {
+  return *e = (cudaGraphExec_t)0x300, cudaSuccess;
+}
+cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) {
+  ++g_graph_launches;
+  if (g_sc) g_sc[agca::MS_DONE] = g_sc[agca::MS_ITERS] = 1.0;
+  return cudaSuccess;
+}
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+}
+
+// ------------------------------------------------------------- fake launchers
+static int g_captured_lanczos = 0, g_fail_captured_lanczos = 0;  // which captured Lanczos step fails (0: none)
+static const double *g_copy_dst = nullptr, *g_lanczos_v = nullptr;
+
+namespace agca {
+#define OK(sig) \
+  cudaError_t sig { return cudaSuccess; }
+int dot_blocks() { return 1216; }
+int64_t compact_scratch_blocks(int64_t n) { return (n + 1023) / 1024; }
+OK(launch_check_eta(const double*, int64_t, int*, cudaStream_t))
+OK(launch_coarsen(int, int, const double*, const double*, const double*, double, double*, double*, double*, uint8_t*,
+                  cudaStream_t))
+OK(launch_mark_vertices(int, const uint8_t*, uint8_t*, cudaStream_t))
+cudaError_t launch_compact(const uint8_t*, int64_t, int32_t*, int32_t*, int32_t*, int64_t* total, cudaStream_t) {
+  return *total = 0, cudaSuccess;
+}
+OK(launch_galerkin(int, int64_t, const int32_t*, int, bool, const double*, const int32_t*, const double*, double*,
+                   cudaStream_t))
+OK(launch_stencil_assemble(int, int64_t, const int32_t*, const int32_t*, const double*, double*, cudaStream_t))
+OK(launch_stencil_to_f32(int64_t, const double*, float*, float*, cudaStream_t))
+template <typename T>
+OK(launch_edge_records(int, const T*, const int32_t*, T*, cudaStream_t))
+template <typename T>
+OK(launch_masked_coef(int64_t, const double*, const int32_t*, T*, cudaStream_t))
+OK(launch_diag(const LevelOp<double>&, double*, double*, float*, cudaStream_t))
+OK(launch_d2f(const double*, float*, int64_t, cudaStream_t, const FirstIterate<float>&))
+OK(launch_x1(const double*, const FirstIterate<double>&, int64_t, cudaStream_t))
+OK(launch_coarse_assemble(const LevelOp<double>&, double*, cudaStream_t))
+OK(launch_cholesky(double*, int, int*, cudaStream_t))
+OK(launch_trinv(const double*, int, double*, cudaStream_t))
+OK(launch_coarse_inverse(const double*, int, double*, cudaStream_t))
+OK(launch_start_vector(int, double*, cudaStream_t))
+OK(launch_pressure_mass(int, const double*, double*, double*, double*, cudaStream_t))
+OK(launch_mask_boundary(int, double*, cudaStream_t))
+OK(launch_gradient(int, const double*, const double*, const double*, double*, cudaStream_t))
+OK(launch_divergence(int, const double*, double*, cudaStream_t))
+template <typename T>
+OK(launch_coarse_solve(int, const double*, const T*, T*, cudaStream_t))
+template <typename T>
+OK(launch_gather(const LevelOp<T>&, const T*, cudaStream_t))
+template <typename T>
+OK(launch_restrict(int, int, bool, T, const T*, T*, cudaStream_t, const FirstIterate<T>&))
+template <typename T>
+OK(launch_prolong(int, int, bool, bool, const T*, T*, cudaStream_t))
+template <typename TS, typename T>
+OK(launch_stencil(int, const LevelOp<T>&, const StencilArgs<TS>&, cudaStream_t, const TileCfg*))
+template cudaError_t launch_edge_records(int, const double*, const int32_t*, double*, cudaStream_t);
+template cudaError_t launch_masked_coef(int64_t, const double*, const int32_t*, float*, cudaStream_t);
+#define BOTH(T)                                                                                                  \
+  template cudaError_t launch_coarse_solve(int, const double*, const T*, T*, cudaStream_t);                      \
+  template cudaError_t launch_gather(const LevelOp<T>&, const T*, cudaStream_t);                                 \
+  template cudaError_t launch_restrict(int, int, bool, T, const T*, T*, cudaStream_t, const FirstIterate<T>&);   \
+  template cudaError_t launch_prolong(int, int, bool, bool, const T*, T*, cudaStream_t);                         \
+  template cudaError_t launch_stencil(int, const LevelOp<T>&, const StencilArgs<T>&, cudaStream_t, const TileCfg*);
+BOTH(float)
+BOTH(double)
+template cudaError_t launch_stencil(int, const LevelOp<float>&, const StencilArgs<double>&, cudaStream_t,
+                                    const TileCfg*);
+OK(launch_sum(const double*, int64_t, double*, int*, double*, double, cudaStream_t))
+cudaError_t launch_dot(const double*, const double*, int64_t, double*, int*, double* out, double, cudaStream_t) {
+  if (!g_capturing) *out = 1.0;
+  return cudaSuccess;
+}
+cudaError_t launch_vec_op(int op, int64_t, double* y, const double*, const double*, const double*, cudaStream_t) {
+  if (op == VOP_COPY) g_copy_dst = y;
+  return cudaSuccess;
+}
+OK(launch_pdiv(int64_t, const double*, const double*, double*, double*, double*, int*, cudaStream_t))
+cudaError_t launch_minres_init(double* sc, double, cudaStream_t) {
+  g_sc = sc;
+  sc[MS_DONE] = sc[MS_ITERS] = 0.0;
+  return cudaSuccess;
+}
+cudaError_t launch_lanczos(int64_t, const double*, const double* v, double*, double*, int64_t, double*, int*,
+                           cudaStream_t) {
+  if (g_capturing) return ++g_captured_lanczos == g_fail_captured_lanczos ? cudaErrorUnknown : cudaSuccess;
+  g_lanczos_v = v;
+  return cudaSuccess;
+}
+cudaError_t launch_minres_finish(int64_t, int64_t, double*, const double*, double* sc, double*, int*, cudaStream_t) {
+  if (!g_capturing) sc[MS_DONE] = sc[MS_ITERS] = 1.0;
+  return cudaSuccess;
+}
+OK(launch_minres_update(int64_t, const double*, const double*, double*, double*, const double*, cudaStream_t))
+}  // namespace agca
+
+// ------------------------------------------------------------- scenarios
+#define REQUIRE(c)                                        \
+  do {                                                    \
+    if (!(c)) {                                           \
+      printf("line %d: %s is false\n", __LINE__, #c);     \
+      return 1;                                           \
+    }                                                     \
+  } while (0)
+
+struct Problem {
+  agca_ctx* ctx = nullptr;
+  std::vector<void*> mem;
+  double *b = nullptr, *x = nullptr;
+  void* take(size_t bytes) {
+    void* p = aligned_alloc(256, (bytes + 255) / 256 * 256 + 256);
+    memset(p, 0, bytes);
+    mem.push_back(p);
+    return p;
+  }
+  // a context with its hierarchy set up, right-hand side and solution vectors
+  bool make(int N, int L, int prec, void* stream) {
+    size_t ws = 0, gs = 0;
+    const size_t n = 2 * N, nt = 3 * (n + 1) * (n + 1) * (n + 1) + (size_t)(N + 1) * (N + 1) * (N + 1);
+    if (agca_create(N, L, prec, stream, &ctx) || agca_workspace_size(ctx, &ws)) return false;
+    if (agca_bind_workspace(ctx, take(ws), ws)) return false;
+    if (agca_set_viscosity(ctx, (double*)take(6 * n * n * n * sizeof(double))) || agca_flag(ctx, 10.0, &gs)) return false;
+    if (agca_bind_gca_store(ctx, take(gs), gs) || agca_setup(ctx)) return false;
+    b = (double*)take(nt * sizeof(double));
+    x = (double*)take(nt * sizeof(double));
+    return true;
+  }
+  ~Problem() {
+    agca_destroy(ctx);
+    for (void* p : mem) free(p);
+  }
+};
+
+// The second of the two iterations captured for a context on the default stream
+// fails: the direct launches that follow start from the vectors of a fresh MINRES
+static int second_captured_iteration_fails() {
+  Problem p;
+  REQUIRE(p.make(4, 2, AGCA_FP64, nullptr));
+  g_fail_captured_lanczos = 2;
+  int its = 0;
+  double rel = 0.0;
+  agca_solve(p.ctx, p.b, p.x, 1e-8, 1, &its, &rel);
+  REQUIRE(g_captured_lanczos == 2);
+  REQUIRE(g_lanczos_v != nullptr && g_lanczos_v == g_copy_dst);  // v = the vector that holds the residual
+  return 0;
+}
+
+int main(int argc, char** argv) {
+  const std::string s = argc > 1 ? argv[1] : "";
+  int r = 2;
+  if (s == "second_captured_iteration_fails") r = second_captured_iteration_fails();
+  if (r == 0) printf("ok\n");
+  return r;
+}
