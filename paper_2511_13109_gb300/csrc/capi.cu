@@ -487,6 +487,9 @@ agca_status vcycle_direct(agca_ctx* ctx, const double* r, double* z) {
   return AGCA_OK;
 }
 
+// the legacy default stream, under either name: it cannot be captured
+bool legacy_stream(cudaStream_t s) { return s == nullptr || s == cudaStreamLegacy; }
+
 // One V-cycle, replayed from a CUDA graph captured on first use for this
 // (r, z) pair: the cycle is a fixed sequence of ~40 launches whose
 // parameters only change at setup.  Direct launches when the stream is the
@@ -494,7 +497,7 @@ agca_status vcycle_direct(agca_ctx* ctx, const double* r, double* z) {
 // per-launch timing is on.
 agca_status vcycle_impl(agca_ctx* ctx, const double* r, double* z) {
   cudaStream_t s = ctx->stream;
-  bool graph = ctx->use_graphs && !ctx->prof && s != nullptr;
+  bool graph = ctx->use_graphs && !ctx->prof && !legacy_stream(s);
   if (graph) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CK(cudaStreamIsCapturing(s, &cs));
@@ -631,7 +634,7 @@ agca_status minres_impl(agca_ctx* ctx, const double* b, double* d, double tol_re
   // The legacy default stream cannot be captured, but a graph captured on
   // another stream runs on it: some 25 launches an iteration at small sizes
   // otherwise cost more on the host than on the GPU.
-  const bool legacy = s == nullptr || s == cudaStreamLegacy;
+  const bool legacy = legacy_stream(s);
   bool graph = ctx->use_graphs && !ctx->prof;
   if (graph && !legacy) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;

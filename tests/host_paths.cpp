@@ -196,10 +196,24 @@ static int second_captured_iteration_fails() {
   return 0;
 }
 
+// The legacy default stream by its handle: MINRES replays its graph there as on
+// the null stream (the preconditioner before it must not switch graphs off)
+static int legacy_stream_handle() {
+  for (void* stream : {(void*)nullptr, (void*)cudaStreamLegacy}) {
+    Problem p;
+    REQUIRE(p.make(4, 2, AGCA_FP64, stream));
+    g_graph_launches = 0;
+    agca_solve(p.ctx, p.b, p.x, 1e-8, 2, nullptr, nullptr);
+    REQUIRE(g_graph_launches > 0);
+  }
+  return 0;
+}
+
 int main(int argc, char** argv) {
   const std::string s = argc > 1 ? argv[1] : "";
   int r = 2;
   if (s == "second_captured_iteration_fails") r = second_captured_iteration_fails();
+  if (s == "legacy_stream_handle") r = legacy_stream_handle();
   if (r == 0) printf("ok\n");
   return r;
 }
