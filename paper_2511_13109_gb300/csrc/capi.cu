@@ -7,6 +7,7 @@
 #include <array>
 #include <fstream>
 #include <map>
+#include <optional>
 #include <sstream>
 #include <type_traits>
 #include <cstdio>
@@ -986,6 +987,15 @@ agca_status check_status(agca_ctx* ctx, const char* where) {
   return AGCA_OK;
 }
 
+// Coefficient records of a level that keeps none, for a scope: whatever way it
+// is left, the context holds no pointer to them afterwards
+struct ScopedRecords {
+  Level& lv;
+  ScopedRecords(Level& l, double* rec) : lv(l) { lv.hedge = rec; }
+  ~ScopedRecords() { lv.hedge = nullptr; }
+  ScopedRecords(const ScopedRecords&) = delete;
+};
+
 // Power iteration on D^-1 A_l from the start vector, then the two inner
 // products of the Rayleigh quotient (v^T A v) / (v^T D v) into
 // sc[kRaySlot + 2 l], sc[kRaySlot + 2 l + 1].  The quotient does not depend on
@@ -1000,33 +1010,26 @@ agca_status power_lambda(agca_ctx* ctx, int l) {
   Level& lv = ctx->lev[l];
   const int64_t n3 = 3 * lv.V;
   cudaStream_t s = ctx->stream;
-  const bool scratch = lv.hedge == nullptr && lv.n > kPointMaxN;
-  if (scratch) {
-    lv.hedge = ctx->kv[KV_Z];
-    const cudaError_t e = launch_edge_records(lv.n, lv.mean, l < ctx->L ? lv.fidx : nullptr, lv.hedge, s);
-    if (e != cudaSuccess) lv.hedge = nullptr;
-    LK(1, e);
+  std::optional<ScopedRecords> scratch;
+  if (lv.hedge == nullptr && lv.n > kPointMaxN) {
+    LK(1, launch_edge_records(lv.n, lv.mean, l < ctx->L ? lv.fidx : nullptr, ctx->kv[KV_Z], s));
+    scratch.emplace(lv, ctx->kv[KV_Z]);
   }
   double* v = ctx->kv[KV_VOLD];
   double* w = ctx->kv[KV_V];
-  auto run = [&]() -> agca_status {
-    LK(1, launch_start_vector(lv.n, v, s));
-    for (int it = 0; it < ctx->power_iters; ++it) {
-      CKS(stencil<double>(ctx, ST_POWER, l, v, nullptr, nullptr, w, 0, 0, 0));
-      std::swap(v, w);
-      if (it % 16 == 15) {
-        CKS(dot1(ctx, v, v, n3, ctx->sc + MS_TMP0));
-        LK(1, launch_vec_op(VOP_SCALE_RSQRT, n3, v, v, nullptr, ctx->sc + MS_TMP0, s));
-      }
+  LK(1, launch_start_vector(lv.n, v, s));
+  for (int it = 0; it < ctx->power_iters; ++it) {
+    CKS(stencil<double>(ctx, ST_POWER, l, v, nullptr, nullptr, w, 0, 0, 0));
+    std::swap(v, w);
+    if (it % 16 == 15) {
+      CKS(dot1(ctx, v, v, n3, ctx->sc + MS_TMP0));
+      LK(1, launch_vec_op(VOP_SCALE_RSQRT, n3, v, v, nullptr, ctx->sc + MS_TMP0, s));
     }
-    CKS(stencil<double>(ctx, ST_APPLY, l, v, nullptr, nullptr, w, 0, 0, 0));
-    CKS(dot1(ctx, v, w, n3, ctx->sc + kRaySlot + 2 * l));
-    LK(1, launch_vec_op(VOP_MUL, n3, w, v, lv.diag, nullptr, s));
-    return dot1(ctx, v, w, n3, ctx->sc + kRaySlot + 2 * l + 1);
-  };
-  const agca_status st = run();
-  if (scratch) lv.hedge = nullptr;
-  return st;
+  }
+  CKS(stencil<double>(ctx, ST_APPLY, l, v, nullptr, nullptr, w, 0, 0, 0));
+  CKS(dot1(ctx, v, w, n3, ctx->sc + kRaySlot + 2 * l));
+  LK(1, launch_vec_op(VOP_MUL, n3, w, v, lv.diag, nullptr, s));
+  return dot1(ctx, v, w, n3, ctx->sc + kRaySlot + 2 * l + 1);
 }
 
 bool valid_level(const agca_ctx* ctx, int l) { return l >= 1 && l <= ctx->L; }
@@ -1946,13 +1949,12 @@ agca_status agca_solve_fgmres(agca_ctx* ctx, const double* b_dev, double* x_dev,
   if (work_bytes < W.need) W.has_rec = false;
   if (work_bytes < W.need_bare) return ctx->fail(AGCA_ENOMEM, "FGMRES workspace too small");
   Level& lf = ctx->lev[ctx->L];
+  std::optional<ScopedRecords> records;
   if (W.has_rec) {
     LK(1, launch_edge_records(lf.n, lf.mean, nullptr, W.rec, ctx->stream));
-    lf.hedge = W.rec;
+    records.emplace(lf, W.rec);
   }
-  const agca_status st = fgmres_impl(ctx, W, restart, b_dev, x_dev, rtol, maxit, schur, z_iters, iters, relres);
-  if (W.has_rec) lf.hedge = nullptr;
-  return st;
+  return fgmres_impl(ctx, W, restart, b_dev, x_dev, rtol, maxit, schur, z_iters, iters, relres);
 }
 
 agca_status agca_element_sensitivity(agca_ctx* ctx, const double* lam_u_dev, const double* u_dev, double* g_dev) {

@@ -61,6 +61,8 @@ cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 
 // ------------------------------------------------------------- fake launchers
 static int g_captured_lanczos = 0, g_fail_captured_lanczos = 0;  // which captured Lanczos step fails (0: none)
+static bool g_throw_block_dot = false;
+static const void* g_records = nullptr;  // coefficient records of the last operator launch
 static const double *g_copy_dst = nullptr, *g_lanczos_v = nullptr;
 
 namespace agca {
@@ -104,7 +106,10 @@ OK(launch_restrict(int, int, bool, T, const T*, T*, cudaStream_t, const FirstIte
 template <typename T>
 OK(launch_prolong(int, int, bool, bool, const T*, T*, cudaStream_t))
 template <typename TS, typename T>
-OK(launch_stencil(int, const LevelOp<T>&, const StencilArgs<TS>&, cudaStream_t, const TileCfg*))
+cudaError_t launch_stencil(int, const LevelOp<T>& op, const StencilArgs<TS>&, cudaStream_t, const TileCfg*) {
+  g_records = op.hedge;
+  return cudaSuccess;
+}
 template cudaError_t launch_edge_records(int, const double*, const int32_t*, double*, cudaStream_t);
 template cudaError_t launch_masked_coef(int64_t, const double*, const int32_t*, float*, cudaStream_t);
 #define BOTH(T)                                                                                                  \
@@ -140,6 +145,10 @@ cudaError_t launch_lanczos(int64_t, const double*, const double* v, double*, dou
 }
 cudaError_t launch_minres_finish(int64_t, int64_t, double*, const double*, double* sc, double*, int*, cudaStream_t) {
   if (!g_capturing) sc[MS_DONE] = sc[MS_ITERS] = 1.0;
+  return cudaSuccess;
+}
+cudaError_t launch_block_dot(int, const double*, int64_t, const double*, int64_t, double*, double*, cudaStream_t) {
+  if (g_throw_block_dot) throw std::bad_alloc();
   return cudaSuccess;
 }
 OK(launch_minres_update(int64_t, const double*, const double*, double*, double*, const double*, cudaStream_t))
@@ -209,11 +218,33 @@ static int legacy_stream_handle() {
   return 0;
 }
 
+// FGMRES of a mixed context works on coefficient records in the caller's
+// workspace: whatever way the call ends, none of them stay in the context
+static int records_leave_with_fgmres() {
+  Problem p;
+  REQUIRE(p.make(18, 3, AGCA_MIXED, nullptr));  // 36 cubes per axis: past the point kernel
+  size_t work = 0;
+  REQUIRE(agca_fgmres_workspace_size(p.ctx, 4, &work) == AGCA_OK);
+  char* w = (char*)p.take(work);
+  g_throw_block_dot = true;
+  bool thrown = false;
+  try {
+    agca_solve_fgmres(p.ctx, p.b, p.x, 1e-8, 4, 4, 0, 1, w, work, nullptr, nullptr);
+  } catch (const std::bad_alloc&) {
+    thrown = true;
+  }
+  REQUIRE(thrown && g_records >= w && g_records < w + work);
+  REQUIRE(agca_apply(p.ctx, 3, AGCA_F64, p.b, p.x) == AGCA_OK);
+  REQUIRE(g_records == nullptr);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   const std::string s = argc > 1 ? argv[1] : "";
   int r = 2;
   if (s == "second_captured_iteration_fails") r = second_captured_iteration_fails();
   if (s == "legacy_stream_handle") r = legacy_stream_handle();
+  if (s == "records_leave_with_fgmres") r = records_leave_with_fgmres();
   if (r == 0) printf("ok\n");
   return r;
 }
