@@ -109,10 +109,13 @@ const char* agca_last_error(const agca_ctx* ctx);
 agca_status agca_set_smoother(agca_ctx* ctx, int degree, double lo, double hi, int power_iters);
 
 /* Solver options: in mixed contexts each residual-refinement step runs
- * MINRES until the preconditioned residual norm has dropped by at least
- * mixed_inner_rtol (default 1e-4; the FP32 cycle and operator limit how far
- * one inner solve can usefully go); check_every MINRES iterations pass
- * between host-side convergence checks (default 4). */
+ * MINRES until the preconditioned residual norm has dropped by
+ * mixed_inner_rtol, or by less where that ends the solve (the FP32 cycle and
+ * operator limit how far one inner solve can usefully go); check_every MINRES
+ * iterations pass between host-side convergence checks.  A context on which
+ * this call has not been made uses 1e-4, except that a step which would end
+ * the solve with up to 30 times more reduction than that runs so far, and
+ * checks every 4 iterations. */
 agca_status agca_set_solver_options(agca_ctx* ctx, double mixed_inner_rtol, int check_every);
 
 /* Coarse DCA coefficient of a coarse element from its 8 children's values

@@ -234,6 +234,8 @@ class Context:
         self._check(lib().agca_set_smoother(self._h, degree, lo, hi, power_iters), "set_smoother")
 
     def set_solver_options(self, mixed_inner_rtol: float = 1e-4, check_every: int = 4):
+        """Smallest reduction asked of one inner MINRES of the mixed refinement,
+        and the iterations between host checks (agca_set_solver_options)."""
         self._check(lib().agca_set_solver_options(self._h, float(mixed_inner_rtol), int(check_every)),
                     "set_solver_options")
 

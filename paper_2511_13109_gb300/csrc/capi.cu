@@ -71,6 +71,7 @@ struct agca_ctx {
   double cheb_lo = 0.1, cheb_hi = 1.1;
   int power_iters = 20;
   double mixed_inner = 1e-4;  // floor of the inner MINRES tolerance in mixed refinement
+  bool mixed_inner_set = false;  // by the caller
   int projection = 0;         // coarse DCA coefficient: 0 arithmetic, 1 harmonic, 2 geometric mean
   int check_every = 4;        // MINRES iterations between host convergence checks
   std::vector<Level> lev;  // 1..L
@@ -714,11 +715,15 @@ agca_status project_pressure(agca_ctx* ctx, double* x) {
 
 // Tolerance of an inner MINRES that would have to reduce the residual by `want`
 // to end a tenth below the outer one's.  Mixed refinement stops at the floor,
-// where FP32 arithmetic still converges well, and goes on from the true residual
-// -- unless a little more ends the solve: stopping just short of it, the result
+// where FP32 arithmetic still converges well, and goes on from the true residual.
+// A floor that the caller set is kept; the default one is undercut, by up to
+// kInnerReach, where that ends the solve: stopping just short of it, the result
 // lay barely below or barely above the tolerance, by chance.
-double inner_tolerance(double want, bool mixed, double floor) {
-  if (mixed && want < floor && !(30.0 * want >= floor)) want = floor;
+constexpr double kInnerReach = 30.0;
+double inner_tolerance(const agca_ctx* ctx, double want) {
+  if (ctx->prec == AGCA_MIXED && want < ctx->mixed_inner &&
+      (ctx->mixed_inner_set || kInnerReach * want < ctx->mixed_inner))
+    want = ctx->mixed_inner;
   return std::max(want, 1e-14);
 }
 
@@ -750,7 +755,7 @@ agca_status solve_impl(agca_ctx* ctx, const double* b_in, double* x, double rtol
     CKS(read_scalar(ctx, ctx->sc + MS_TMP0, &nr2));
     rel = sqrt(nr2) / nb;
     if (!(rel > rtol) || total >= maxit) break;
-    const double inner = inner_tolerance(0.1 * rtol / rel, mixed, ctx->mixed_inner);
+    const double inner = inner_tolerance(ctx, 0.1 * rtol / rel);
     int its = 0;
     CKS(minres_impl(ctx, r, d, inner, maxit - total, mixed, &its));
     total += its;
@@ -1674,6 +1679,7 @@ agca_status agca_set_solver_options(agca_ctx* ctx, double mixed_inner_rtol, int 
   if (!(mixed_inner_rtol > 0.0 && mixed_inner_rtol < 1.0) || check_every < 1 || check_every > 1000)
     return ctx->fail(AGCA_EINVAL, "solver options out of range");
   ctx->mixed_inner = mixed_inner_rtol;
+  ctx->mixed_inner_set = true;
   ctx->check_every = check_every;
   return AGCA_OK;
 }
@@ -2346,7 +2352,6 @@ agca_status agca_batch_solve(agca_batch* b, const double* const* b_devs, double*
   if (!b->setup_done) return b->fail(AGCA_ESTATE, "setup first");
   if (!(rtol > 0.0) || maxit < 1) return b->fail(AGCA_EINVAL, "rtol must be > 0 and maxit >= 1");
   const int P = b->n;
-  const bool mixed = b->prec == AGCA_MIXED;
   std::vector<double> nb(P, 0.0), rel(P, 0.0);
   std::vector<int> total(P, 0);
   std::vector<char> active(P, 0);
@@ -2402,7 +2407,7 @@ agca_status agca_batch_solve(agca_batch* b, const double* const* b_devs, double*
         continue;
       }
       budget = std::max(budget, maxit - total[p]);
-      const double inner = inner_tolerance(0.1 * rtol / rel[p], mixed, ctx->mixed_inner);
+      const double inner = inner_tolerance(ctx, 0.1 * rtol / rel[p]);
       LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_D], nullptr, nullptr, nullptr, s));
       LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_VOLD], nullptr, nullptr, nullptr, s));
       LK(1, launch_vec_op(VOP_ZERO, nt, ctx->kv[KV_WOLD], nullptr, nullptr, nullptr, s));

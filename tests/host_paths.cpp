@@ -61,6 +61,7 @@ cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 
 // ------------------------------------------------------------- fake launchers
 static int g_captured_lanczos = 0, g_fail_captured_lanczos = 0;  // which captured Lanczos step fails (0: none)
+static double g_inner = 0.0;  // tolerance of the last inner MINRES
 static bool g_throw_block_dot = false;
 static const void* g_records = nullptr;  // coefficient records of the last operator launch
 static const double *g_copy_dst = nullptr, *g_lanczos_v = nullptr;
@@ -132,8 +133,9 @@ cudaError_t launch_vec_op(int op, int64_t, double* y, const double*, const doubl
   return cudaSuccess;
 }
 OK(launch_pdiv(int64_t, const double*, const double*, double*, double*, double*, int*, cudaStream_t))
-cudaError_t launch_minres_init(double* sc, double, cudaStream_t) {
+cudaError_t launch_minres_init(double* sc, double tol_rel, cudaStream_t) {
   g_sc = sc;
+  g_inner = tol_rel;
   sc[MS_DONE] = sc[MS_ITERS] = 0.0;
   return cudaSuccess;
 }
@@ -239,12 +241,34 @@ static int records_leave_with_fgmres() {
   return 0;
 }
 
+// A mixed context's inner tolerance: never below a mixed_inner_rtol that the
+// caller set; by default 1e-4, or up to 30 times lower where that ends the solve
+static int inner_tolerance_of_the_caller() {
+  const struct {
+    double set, rtol, inner;  // the first residual is 1: MINRES would have to reach 0.1 rtol
+  } cases[] = {{0.0, 1e-3, 1e-4},  {0.0, 1e-4, 1e-5},  {0.0, 1e-5, 1e-4},  {1e-4, 1e-4, 1e-4},
+               {1e-2, 1e-2, 1e-2}, {1e-2, 1e-3, 1e-2}, {1e-2, 0.5, 0.05}, {1e-6, 1e-6, 1e-6},
+               {1e-6, 1e-4, 1e-5}};
+  for (const auto& c : cases) {
+    Problem p;
+    REQUIRE(p.make(4, 2, AGCA_MIXED, nullptr));
+    if (c.set > 0.0) REQUIRE(agca_set_solver_options(p.ctx, c.set, 4) == AGCA_OK);
+    agca_solve(p.ctx, p.b, p.x, c.rtol, 2, nullptr, nullptr);
+    if (!(g_inner > 0.999 * c.inner && g_inner < 1.001 * c.inner)) {
+      printf("set %g, rtol %g: inner tolerance %g, expected %g\n", c.set, c.rtol, g_inner, c.inner);
+      return 1;
+    }
+  }
+  return 0;
+}
+
 int main(int argc, char** argv) {
   const std::string s = argc > 1 ? argv[1] : "";
   int r = 2;
   if (s == "second_captured_iteration_fails") r = second_captured_iteration_fails();
   if (s == "legacy_stream_handle") r = legacy_stream_handle();
   if (s == "records_leave_with_fgmres") r = records_leave_with_fgmres();
+  if (s == "inner_tolerance_of_the_caller") r = inner_tolerance_of_the_caller();
   if (r == 0) printf("ok\n");
   return r;
 }

@@ -25,7 +25,7 @@ def program(tmp_path_factory):
 
 
 @pytest.mark.parametrize("scenario", ["second_captured_iteration_fails", "legacy_stream_handle",
-                                      "records_leave_with_fgmres"])
+                                      "records_leave_with_fgmres", "inner_tolerance_of_the_caller"])
 def test_host_path(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0 and r.stdout == "ok\n", r.stdout + r.stderr
