@@ -130,53 +130,40 @@ __device__ __forceinline__ RowPiece row_piece(const int nv, const int w, const i
   return RowPiece{32 * (w - row * per) + lane, row - k * nv, k};
 }
 
-// scale * P^T r at coarse vertex (I, J, K) for NC components of a fine grid with
+// scale * P^T r at coarse vertex (I, J, K) for one component of a fine grid with
 // nf cubes per axis; 0 on the coarse boundary when mask is set; with fi.x1, the
 // first Chebyshev iterate beside it.  The sum runs over d = 1 .. 7, +d before -d,
 // and a neighbour outside the grid contributes nothing.
-template <typename T, int NC>
+template <typename T>
 __device__ __forceinline__ void restrict_point(const int nf, const bool mask, const T scale, const T* __restrict__ rf,
-                                               T* __restrict__ rc, const FirstIterate<T>& fi, const RowPiece& p) {
-  const int nc = nf / 2, nvc = nc + 1, nvf = nf + 1, Vc = nvc * nvc * nvc, Vf = nvf * nvf * nvf;
-  const int I = p.i, J = p.j, K = p.k;
-  if (I >= nvc) return;
+                                               T* __restrict__ rc, const FirstIterate<T>& fi, const int I, const int J,
+                                               const int K) {
+  const int nc = nf / 2, nvc = nc + 1, nvf = nf + 1;
   const bool edge = I == 0 || J == 0 || K == 0 || I == nc || J == nc || K == nc;
-  const int f = 2 * I + nvf * (2 * J + nvf * 2 * K), c0 = I + nvc * (J + nvc * K);
-  T v[NC];
-#pragma unroll
-  for (int c = 0; c < NC; ++c) v[c] = T(0);
+  const int c0 = I + nvc * (J + nvc * K);
+  const T* r = rf + 2 * I + nvf * (2 * J + nvf * 2 * K);
+  T v = T(0);
   if (!edge) {
+    T acc = T(0);
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const T* r = rf + c * Vf + f;
-      T acc = T(0);
-#pragma unroll
-      for (int d = 1; d < 8; ++d) {
-        const int o = (d & 1) + nvf * (((d >> 1) & 1) + nvf * ((d >> 2) & 1));
-        acc += __ldg(r + o);
-        acc += __ldg(r - o);
-      }
-      v[c] = scale * (__ldg(r) + T(0.5) * acc);
+    for (int d = 1; d < 8; ++d) {
+      const int o = (d & 1) + nvf * (((d >> 1) & 1) + nvf * ((d >> 2) & 1));
+      acc += __ldg(r + o);
+      acc += __ldg(r - o);
     }
+    v = scale * (__ldg(r) + T(0.5) * acc);
   } else if (!mask) {
+    T acc = T(0);
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const T* r = rf + c * Vf + f;
-      T acc = T(0);
-#pragma unroll
-      for (int d = 1; d < 8; ++d) {
-        const int dx = d & 1, dy = (d >> 1) & 1, dz = (d >> 2) & 1, o = dx + nvf * (dy + nvf * dz);
-        if (2 * I + dx <= nf && 2 * J + dy <= nf && 2 * K + dz <= nf) acc += __ldg(r + o);
-        if (2 * I >= dx && 2 * J >= dy && 2 * K >= dz) acc += __ldg(r - o);
-      }
-      v[c] = scale * (__ldg(r) + T(0.5) * acc);
+    for (int d = 1; d < 8; ++d) {
+      const int dx = d & 1, dy = (d >> 1) & 1, dz = (d >> 2) & 1, o = dx + nvf * (dy + nvf * dz);
+      if (2 * I + dx <= nf && 2 * J + dy <= nf && 2 * K + dz <= nf) acc += __ldg(r + o);
+      if (2 * I >= dx && 2 * J >= dy && 2 * K >= dz) acc += __ldg(r - o);
     }
+    v = scale * (__ldg(r) + T(0.5) * acc);
   }
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    rc[c * Vc + c0] = v[c];
-    if (fi.x1) fi.x1[c * Vc + c0] = fi.s2 * __ldg(fi.invD + c * Vc + c0) * v[c];
-  }
+  rc[c0] = v;
+  if (fi.x1) fi.x1[c0] = fi.s2 * __ldg(fi.invD + c0) * v;
 }
 
 // P e at fine vertex (i, j, k) (added to xf when ADD) for NC components; 0 on the

@@ -1,10 +1,19 @@
-// Interpolation between Kuhn grids and its transpose (Sec. 2.1): one thread per
-// written vertex, all components at once, a warp on 32 vertices of one row.  The
-// per-point formulas are restrict_point / prolong_point in device_ops.cuh.  With
-// flat vertex indices (two integer divisions each) and a loop over the components
-// the finest FP32 level at 128^3 pressure cubes took 131 us (prolongation) and
-// 87 us (restriction with the first iterate); now 92 and 54 us, floors 64 and 41.
-// (One warp per row, looping over it, left too little in flight: 134 and 106 us.)
+// Interpolation between Kuhn grids and its transpose (Sec. 2.1); the per-point
+// formulas are restrict_point / prolong_point in device_ops.cuh.
+//
+// Prolongation: one thread per fine vertex, all components at once, a warp on 32
+// vertices of one row.  With flat vertex indices (two integer divisions each) and
+// a loop over the components the finest FP32 level at 128^3 pressure cubes took
+// 131 us, now 92; floor 64.  (One warp per row, looping over it, left too little
+// in flight: 134 us.)
+//
+// Restriction: one thread per coarse vertex and component, flat indices.  In FP64
+// it is bound by the FP64 pipe (16 operations a value: 164 us at 256^3 cubes; 18
+// with the first iterate), so lanes must not idle: rows of 32 vertices waste a fifth of them at 129 vertices
+// a row.  Measured alone, 256^3 / 128^3 / 64^3 cubes: FP64 196 / 30 / 9 us (rows of
+// 32 with all components per thread 216 / 34 / 12, flat with a loop over the
+// components 198 / 32 / 12), FP32 53 / 12 / 6 us (54 / 14 / 9, 78 / 18 / 11); with
+// the first iterate FP64 221 / 35 / 10, FP32 60 / 14 / 6 us.
 #include <stdlib.h>
 
 #include "agca_internal.cuh"
@@ -15,13 +24,27 @@ namespace agca {
 namespace {
 
 constexpr int kRowWarps = 8;
+constexpr int kRestrictThreads = 256;
 
-template <typename T, int NC>
-__global__ void __launch_bounds__(32 * kRowWarps)
+// grid (blocks of the vertices, components)
+template <typename T>
+__device__ __forceinline__ void restrict_thread(const int nf, const bool mask, const T scale, const T* rf, T* rc,
+                                                FirstIterate<T> fi, const int c) {
+  const int nvf = nf + 1, nv = nf / 2 + 1, V = nv * nv * nv, id = blockIdx.x * kRestrictThreads + threadIdx.x;
+  if (id >= V) return;
+  const int t = id / nv, K = t / nv;
+  if (fi.x1) {
+    fi.x1 += c * V;
+    fi.invD += c * V;
+  }
+  restrict_point<T>(nf, mask, scale, rf + c * (nvf * nvf * nvf), rc + c * V, fi, id - t * nv, t - K * nv, K);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kRestrictThreads)
     restrict_kernel(int nf, bool mask, T scale, const T* __restrict__ rf, T* __restrict__ rc, const FirstIterate<T> fi) {
   grid_dep_entry();
-  const int w = blockIdx.x * kRowWarps + (threadIdx.x >> 5), nv = nf / 2 + 1;
-  if (w < row_pieces(nv)) restrict_point<T, NC>(nf, mask, scale, rf, rc, fi, row_piece(nv, w, threadIdx.x & 31));
+  restrict_thread<T>(nf, mask, scale, rf, rc, fi, blockIdx.y);
 }
 
 template <typename T, int NC, bool ADD>
@@ -32,20 +55,18 @@ __global__ void __launch_bounds__(32 * kRowWarps)
   if (w < row_pieces(nv)) prolong_point<T, NC, ADD>(nf, mask, ec, xf, row_piece(nv, w, threadIdx.x & 31));
 }
 
-// many problems: grid (blocks of the largest, problems)
-template <typename T, int NC>
-__global__ void __launch_bounds__(32 * kRowWarps) restrict_batch_kernel(const XferTask* __restrict__ tasks) {
+// many problems: grid (blocks of the largest, problems, components of a restriction)
+template <typename T>
+__global__ void __launch_bounds__(kRestrictThreads) restrict_batch_kernel(const XferTask* __restrict__ tasks) {
   grid_dep_entry();
   const XferTask tk = tasks[blockIdx.y];
   if (tk.sc && tk.sc[MS_DONE] != 0.0) return;
-  const int w = blockIdx.x * kRowWarps + (threadIdx.x >> 5), nv = tk.nf / 2 + 1;
-  if (w >= row_pieces(nv)) return;
   FirstIterate<T> fi;
   fi.invD = static_cast<const T*>(tk.invD);
   fi.x1 = static_cast<T*>(tk.x1);
   fi.s2 = (T)tk.s2;
-  restrict_point<T, NC>(tk.nf, tk.mask, (T)tk.scale, static_cast<const T*>(tk.src), static_cast<T*>(tk.dst), fi,
-                        row_piece(nv, w, threadIdx.x & 31));
+  restrict_thread<T>(tk.nf, tk.mask, (T)tk.scale, static_cast<const T*>(tk.src), static_cast<T*>(tk.dst), fi,
+                     blockIdx.z);
 }
 
 template <typename T, int NC, bool ADD>
@@ -64,6 +85,8 @@ unsigned row_blocks(int n) {
   return (unsigned)((nv * nv * ((nv + 31) / 32) + kRowWarps - 1) / kRowWarps);
 }
 
+unsigned vertex_blocks(int n) { return (unsigned)((nverts(n) + kRestrictThreads - 1) / kRestrictThreads); }
+
 }  // namespace
 
 bool pdl_enabled(cudaStream_t s) {
@@ -78,10 +101,9 @@ bool pdl_enabled(cudaStream_t s) {
 template <typename T>
 cudaError_t launch_restrict(int nf, int ncomp, bool mask, T scale, const T* rf, T* rc, cudaStream_t s,
                             const FirstIterate<T>& fi) {
-  const dim3 g(row_blocks(nf / 2)), t(32 * kRowWarps);
-  if (ncomp == 3) return launch_k(restrict_kernel<T, 3>, g, t, 0, s, nf, mask, scale, rf, rc, fi);
-  if (ncomp == 1) return launch_k(restrict_kernel<T, 1>, g, t, 0, s, nf, mask, scale, rf, rc, fi);
-  return cudaErrorInvalidValue;
+  if (ncomp != 3 && ncomp != 1) return cudaErrorInvalidValue;
+  return launch_k(restrict_kernel<T>, dim3(vertex_blocks(nf / 2), (unsigned)ncomp), dim3(kRestrictThreads), 0, s, nf, mask,
+                  scale, rf, rc, fi);
 }
 
 template <typename T>
@@ -98,8 +120,8 @@ cudaError_t launch_transfer_batch(int kind, int ncomp, const XferTask* tasks, in
   const dim3 g(row_blocks(max_n), (unsigned)ntasks), t(32 * kRowWarps);
   switch (kind) {
     case XK_RESTRICT:
-      if (ncomp == 3) return launch_k(restrict_batch_kernel<T, 3>, g, t, 0, s, tasks);
-      return launch_k(restrict_batch_kernel<T, 1>, g, t, 0, s, tasks);
+      return launch_k(restrict_batch_kernel<T>, dim3(vertex_blocks(max_n), (unsigned)ntasks, (unsigned)ncomp),
+                      dim3(kRestrictThreads), 0, s, tasks);
     case XK_PROLONG_ADD: return launch_k(prolong_batch_kernel<T, 3, true>, g, t, 0, s, tasks);
     case XK_PROLONG: return launch_k(prolong_batch_kernel<T, 1, false>, g, t, 0, s, tasks);
     default: return cudaErrorInvalidValue;
