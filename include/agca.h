@@ -223,13 +223,14 @@ agca_status agca_solve(agca_ctx* ctx, const double* b_dev, double* x_dev, double
  * launches, else the call fails with AGCA_ECUDA).
  * work_dev: caller-owned device memory of agca_fgmres_workspace_size bytes
  * (256-byte aligned; holds the 2 restart + 1 Krylov vectors and Z, and in
- * mixed contexts the finest level's coefficient records, 27 doubles a vertex:
- * a workspace smaller by these also serves, with slower FP64 products).  x is
- * overwritten (initial guess 0; pressure returned mean-free).  *iters,
+ * mixed contexts the finest level's coefficient records, 27 doubles a vertex).
+ * One of agca_fgmres_workspace_min bytes, smaller by the records, also serves,
+ * with slower FP64 products.  x is overwritten (initial guess 0; pressure returned mean-free).  *iters,
  * *relres (host): iterations and the final true relative residual.
  * Synchronizes (once per iteration).  AGCA_ENOTCONV above the tolerance
  * after maxit iterations. */
 agca_status agca_fgmres_workspace_size(const agca_ctx* ctx, int restart, size_t* bytes);
+agca_status agca_fgmres_workspace_min(const agca_ctx* ctx, int restart, size_t* bytes);
 agca_status agca_solve_fgmres(agca_ctx* ctx, const double* b_dev, double* x_dev, double rtol, int maxit, int restart,
                               int schur, int z_iters, void* work_dev, size_t work_bytes, int* iters, double* relres);
 

@@ -64,6 +64,7 @@ _SIGS = {
     "agca_load_vector": ([_P, _P, _P], _I),
     "agca_solve": ([_P, _P, _P, _D, _I, ctypes.POINTER(_I), ctypes.POINTER(_D)], _I),
     "agca_fgmres_workspace_size": ([_P, _I, ctypes.POINTER(_SZ)], _I),
+    "agca_fgmres_workspace_min": ([_P, _I, ctypes.POINTER(_SZ)], _I),
     "agca_solve_fgmres": ([_P, _P, _P, _D, _I, _I, _I, _I, _P, _SZ, ctypes.POINTER(_I), ctypes.POINTER(_D)], _I),
     "agca_element_sensitivity": ([_P, _P, _P, _P], _I),
     "agca_adjoint_gradient": ([_P, _P, _P, _P, _D, _I, ctypes.POINTER(_I)], _I),
@@ -349,7 +350,15 @@ class Context:
         x = torch.empty_like(b) if x is None else x
         sz = _SZ()
         self._check(lib().agca_fgmres_workspace_size(self._h, int(restart), ctypes.byref(sz)), "fgmres_workspace_size")
-        work = torch.empty(int(sz.value), dtype=torch.uint8, device=self.device)
+        try:
+            work = torch.empty(int(sz.value), dtype=torch.uint8, device=self.device)
+        except torch.cuda.OutOfMemoryError:  # without the coefficient records of a mixed context
+            full = sz.value
+            self._check(lib().agca_fgmres_workspace_min(self._h, int(restart), ctypes.byref(sz)),
+                        "fgmres_workspace_min")
+            if sz.value == full:
+                raise
+            work = torch.empty(int(sz.value), dtype=torch.uint8, device=self.device)
         its, rel = _I(), _D()
         st = lib().agca_solve_fgmres(self._h, _ptr(b), _ptr(x), float(rtol), int(maxit), int(restart),
                                      {"mass": 0, "bfbt": 1}[schur], int(z_iters), _ptr(work), sz.value,

@@ -1944,6 +1944,12 @@ agca_status agca_fgmres_workspace_size(const agca_ctx* ctx, int restart, size_t*
   return AGCA_OK;
 }
 
+agca_status agca_fgmres_workspace_min(const agca_ctx* ctx, int restart, size_t* bytes) {
+  if (!ctx || !bytes || restart < 1 || restart > 500) return AGCA_EINVAL;
+  *bytes = fgmres_layout(ctx, restart, nullptr).need_bare;
+  return AGCA_OK;
+}
+
 agca_status agca_solve_fgmres(agca_ctx* ctx, const double* b_dev, double* x_dev, double rtol, int maxit, int restart,
                               int schur, int z_iters, void* work_dev, size_t work_bytes, int* iters, double* relres) {
   if (!ctx || !b_dev || !x_dev || !work_dev) return AGCA_EINVAL;

@@ -3,7 +3,7 @@ grid transfers between such levels."""
 import pytest
 import torch
 
-from synth import random_vector
+from synth import random_vector, sphere_sinkers
 
 pytestmark = pytest.mark.gpu
 
@@ -35,3 +35,29 @@ def test_restriction_bit_exact(N, levels, dtype):
         ref = torch.zeros_like(got)
         ref[:, 1:-1, 1:-1, 1:-1] = at(0, 0, 0) + 0.5 * acc
         assert torch.equal(got, ref), l
+
+
+# A mixed context's coefficient records are the part of the FGMRES workspace that
+# it can do without: a device that has no room for them still solves
+@pytest.mark.parametrize("prec", [pkg.MIXED, pkg.FP64])
+def test_fgmres_where_the_records_do_not_fit(prec, monkeypatch):
+    p = sphere_sinkers(18, 3, 0.15, 0.03, 1e2)  # 36 cubes per axis: past the point kernel
+    c = pkg.Context(18, None, prec, device=DEV)
+    c.prepare(torch.from_numpy(p.eta).to(DEV), 10.0)
+    b = c.load_vector(torch.from_numpy(p.fbar.ravel()).to(DEV))
+    empty, sizes = torch.empty, []
+
+    def no_room_for_the_first(*a, **k):
+        if k.get("dtype") is torch.uint8:
+            sizes.append(a[0])
+            if len(sizes) == 1:
+                raise torch.cuda.OutOfMemoryError("out of memory")
+        return empty(*a, **k)
+
+    monkeypatch.setattr(torch, "empty", no_room_for_the_first)
+    if prec == pkg.FP64:  # nothing to leave out
+        with pytest.raises(torch.cuda.OutOfMemoryError):
+            c.solve_fgmres(b, 1e-6, 400, 20)
+        return
+    x, its, rel = c.solve_fgmres(b, 1e-6, 400, 20)
+    assert rel <= 1e-6 and sizes[0] - sizes[1] >= 27 * 8 * c.V[c.L]
