@@ -270,13 +270,14 @@ agca_status agca_adjoint_gradient(agca_ctx* ctx, const double* x_dev, const doub
 agca_status agca_stokes_apply_static(int N, const double* eta_dev, const double* x_dev, double* y_dev,
                                      void* cuda_stream);
 
-/* Autotuner: for every level >= 2 and V-cycle stencil mode (0 apply,
- * 1 residual, 2 first and 3 later Chebyshev steps, 4 pre-smoothing step from
- * zero), time the candidate tile shapes (8 block rows; z-chunks 1..64 and
- * those that fill whole waves) with CUDA events on the context stream, reps
- * launches each, and keep the fastest for the context's later launches.
- * cache_path (nullable): text file of earlier results, read first and
- * rewritten.  Uses the cycle vectors as scratch.  Synchronizes. */
+/* Autotuner: for every level of more than 32 cubes per axis (smaller ones run
+ * no tiles) and V-cycle stencil mode (1 residual, 2 first and 3 later
+ * Chebyshev steps, 4 pre-smoothing step from zero), time the candidate tile
+ * shapes (8 block rows; z-chunks 1..64 and those that fill whole waves) with
+ * CUDA events on the context stream, reps launches each, and keep the fastest
+ * for the context's later launches.  cache_path (nullable): text file of
+ * earlier results, read first and rewritten.  Uses the cycle vectors as
+ * scratch.  Synchronizes. */
 agca_status agca_autotune(agca_ctx* ctx, int reps, const char* cache_path);
 /* The tile shape in use for (level, mode): block rows and z-chunk (0 = automatic). */
 agca_status agca_tile_config(const agca_ctx* ctx, int level, int mode, int* by, int* zch);

@@ -1046,33 +1046,26 @@ bool valid_level(const agca_ctx* ctx, int l) { return l >= 1 && l <= ctx->L; }
 template <typename T>
 agca_status tune_level(agca_ctx* ctx, int l, int reps, std::map<std::string, TileCfg>& cache) {
   Level& lv = ctx->lev[l];
+  if (lv.n <= kPointMaxN) return AGCA_OK;  // no tiles there
   const int64_t n3 = 3 * lv.V;
   cudaStream_t s = ctx->stream;
   for (void* p : {lv.vb, lv.vx, lv.vt, lv.vr}) CK(cudaMemsetAsync(p, 0, n3 * sizeof(T), s));
   const bool f32 = sizeof(T) == 4;
-  // the edge form (every FP64 level) has one tile shape
-  const bool edge = !f32;
-  const std::vector<int> bys = {8};  // the tile kernels have one tile shape; the small levels no tiles
-  auto tiles = [&](int zr, int slots) { return edge ? edge_tiles(lv.n, zr, slots) : f32_tiles(lv.n, zr, slots); };
+  auto tiles = [&](int zr, int slots) { return f32 ? f32_tiles(lv.n, zr, slots) : edge_tiles(lv.n, zr, slots); };
   const int nv = lv.n + 1;
   int dev = 0, sms = 152;
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  // z-chunk candidates: a fixed ladder plus, per block-row count, the chunks
-  // whose block count fills k = 1..16 whole waves of resident blocks (no
-  // partly filled last wave)
-  auto candidates = [&](int by) {
-    std::vector<int> zs = {0, 1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
-    (void)by;
-    const int per_z = tiles(1, 0).per_z();
-    for (int k = 1; k <= 16; ++k) {
-      const int gz = std::max(1, 2 * k * sms / per_z);
-      zs.push_back((nv + gz - 1) / gz);
-    }
-    std::sort(zs.begin() + 1, zs.end());
-    zs.erase(std::unique(zs.begin() + 1, zs.end()), zs.end());
-    return zs;
-  };
+  // z-chunk candidates: a fixed ladder plus the chunks whose block count fills
+  // k = 1..16 whole waves of resident blocks (no partly filled last wave)
+  std::vector<int> chunks = {0, 1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
+  const int per_z = tiles(1, 0).per_z();
+  for (int k = 1; k <= 16; ++k) {
+    const int gz = std::max(1, 2 * k * sms / per_z);
+    chunks.push_back((nv + gz - 1) / gz);
+  }
+  std::sort(chunks.begin() + 1, chunks.end());
+  chunks.erase(std::unique(chunks.begin() + 1, chunks.end()), chunks.end());
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
@@ -1088,44 +1081,40 @@ agca_status tune_level(agca_ctx* ctx, int l, int reps, std::map<std::string, Til
     }
     TileCfg best;
     float best_ms = 1e30f;
-    for (int by : bys) {
-      int last_zch = -1;
-      for (int zr : candidates(by)) {
-        if (zr > nv) continue;
-        const int zch = tiles(zr, 2 * sms).zch;
-        if (zch == last_zch) continue;
-        last_zch = zch;
-        TileCfg c;
-        c.by = by;
-        c.zch = zch;
-        ctx->tune[l][mode] = c;
-        T* X = static_cast<T*>(lv.vx);
-        T* Bv = static_cast<T*>(lv.vb);
-        T* Tb = static_cast<T*>(lv.vt);
-        T* R = static_cast<T*>(lv.vr);
-        auto once = [&]() -> agca_status {
-          switch (mode) {
-            case ST_CHEB_PRE: return stencil<T>(ctx, mode, l, Tb, Bv, nullptr, X, 0.5, 0.5, 0.5);
-            case ST_RESID: return stencil<T>(ctx, mode, l, X, Bv, nullptr, R, 0, 0, 0);
-            case ST_CHEB_FIRST: return stencil<T>(ctx, mode, l, X, Bv, nullptr, Tb, 0.5, 0, 0);
-            default: return stencil<T>(ctx, mode, l, Tb, Bv, X, X, 0.5, 0.5, 0);
-          }
-        };
-        if ((st = once()) != AGCA_OK) break;
-        if ((st = once()) != AGCA_OK) break;
-        if (cudaEventRecord(e0, s) != cudaSuccess) break;
-        for (int r = 0; r < reps && st == AGCA_OK; ++r) st = once();
-        if (st != AGCA_OK) break;
-        cudaEventRecord(e1, s);
-        cudaEventSynchronize(e1);
-        float ms = 0.0f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best_ms) {
-          best_ms = ms;
-          best = c;
+    int last_zch = -1;
+    for (int zr : chunks) {
+      if (zr > nv) continue;
+      const int zch = tiles(zr, 2 * sms).zch;
+      if (zch == last_zch) continue;
+      last_zch = zch;
+      TileCfg c;
+      c.zch = zch;
+      ctx->tune[l][mode] = c;
+      T* X = static_cast<T*>(lv.vx);
+      T* Bv = static_cast<T*>(lv.vb);
+      T* Tb = static_cast<T*>(lv.vt);
+      T* R = static_cast<T*>(lv.vr);
+      auto once = [&]() -> agca_status {
+        switch (mode) {
+          case ST_CHEB_PRE: return stencil<T>(ctx, mode, l, Tb, Bv, nullptr, X, 0.5, 0.5, 0.5);
+          case ST_RESID: return stencil<T>(ctx, mode, l, X, Bv, nullptr, R, 0, 0, 0);
+          case ST_CHEB_FIRST: return stencil<T>(ctx, mode, l, X, Bv, nullptr, Tb, 0.5, 0, 0);
+          default: return stencil<T>(ctx, mode, l, Tb, Bv, X, X, 0.5, 0.5, 0);
         }
-      }
+      };
+      if ((st = once()) != AGCA_OK) break;
+      if ((st = once()) != AGCA_OK) break;
+      if (cudaEventRecord(e0, s) != cudaSuccess) break;
+      for (int r = 0; r < reps && st == AGCA_OK; ++r) st = once();
       if (st != AGCA_OK) break;
+      cudaEventRecord(e1, s);
+      cudaEventSynchronize(e1);
+      float ms = 0.0f;
+      cudaEventElapsedTime(&ms, e0, e1);
+      if (ms < best_ms) {
+        best_ms = ms;
+        best = c;
+      }
     }
     if (st != AGCA_OK) break;
     ctx->tune[l][mode] = best;

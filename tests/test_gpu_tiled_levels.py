@@ -61,3 +61,13 @@ def test_fgmres_where_the_records_do_not_fit(prec, monkeypatch):
         return
     x, its, rel = c.solve_fgmres(b, 1e-6, 400, 20)
     assert rel <= 1e-6 and sizes[0] - sizes[1] >= 27 * 8 * c.V[c.L]
+
+
+# levels of up to 32 cubes per axis run no tiles: the autotuner has nothing to time there
+def test_autotuner_leaves_small_levels(tmp_path):
+    cache = tmp_path / "tiles.txt"
+    c = pkg.Context(16, None, pkg.MIXED, device=DEV)
+    c.prepare(torch.from_numpy(sphere_sinkers(16, 3, 0.15, 0.03, 1e2).eta).to(DEV), 10.0)
+    n = c.launch_count()
+    assert set(c.autotune(2, str(cache)).values()) == {(8, 0)}
+    assert c.launch_count() == n and cache.read_text() == ""
