@@ -263,8 +263,8 @@ constexpr int kF32BatchTasks = 120;
 cudaError_t launch_stencil_f32_batch(int mode, bool sten, bool wide, const StencilTask<float, float>* tasks, int ntasks,
                                      cudaStream_t s);
 // whether a step of this kind runs the edge form: every level of an FP64
-// context (its coefficient records exist on every level); the FP32 cycle and
-// the Stokes operator run the per-cube kernel
+// context (its coefficient records exist on every level); the FP32 cycle runs
+// its own tiles, the FP32-arithmetic Stokes operator the per-cube kernel
 template <typename TS, typename T>
 constexpr bool edge_form_step(int mode, bool coarse) {
   (void)coarse;
@@ -403,13 +403,11 @@ enum KBatchOp { KB_DOT = 0, KB_SUM, KB_LANCZOS, KB_UPDATE, KB_SCALARS, KB_PDIV, 
 cudaError_t launch_krylov_batch(int op, const KTask* tasks, int ntasks, int64_t max_n, double* partials,
                                 cudaStream_t s);
 cudaError_t launch_mask_boundary(int n, double* x, cudaStream_t s);
-// FGMRES pieces: out[i] = w . V_i (i < nvec, V_i = V + i ld); w += sign sum_i coef[i] V_i;
-// y = a * s or a / s (s on the device)
+// FGMRES pieces: out[i] = w . V_i (i < nvec, V_i = V + i ld); w += sign sum_i coef[i] V_i
 cudaError_t launch_block_dot(int nvec, const double* V, int64_t ld, const double* w, int64_t n, double* partials,
                              double* out, cudaStream_t s);
 cudaError_t launch_block_axpy(int nvec, const double* V, int64_t ld, const double* coef, double sign, double* w,
                               int64_t n, cudaStream_t s);
-cudaError_t launch_scale(int64_t n, double* y, const double* a, const double* s_dev, bool recip, cudaStream_t s);
 // assembled Z = B W^-1 B^T on the pressure grid as per-vertex stencils over
 // the ZSTENCIL offsets that are sums of two Kuhn offsets, SoA [ZSTENCIL][V]
 constexpr int ZSTENCIL = 65;

@@ -115,54 +115,15 @@ __global__ void vec_batch_kernel(const KTask* __restrict__ tasks, int op) {
   }
 }
 
-// MINRES scalar recurrence, one thread per problem (as minres_scalar_kernel)
-__device__ void scalars_one(double* sc) {
-  if (sc[MS_DONE] != 0.0) {
-    sc[MS_UPD_SKIP] = 1.0;
-    return;
-  }
-  const double g = sc[MS_GAMMA];
-  const double delta = sc[MS_DOT_KZZ] / (g * g);
-  const double gn2 = sc[MS_DOT_ZV];
-  const double gn = gn2 > 0.0 ? sqrt(gn2) : 0.0;
-  const double c = sc[MS_C], co = sc[MS_C_OLD], s = sc[MS_S], so = sc[MS_S_OLD];
-  const double a0 = c * delta - co * s * g;
-  const double a1 = sqrt(a0 * a0 + gn * gn);
-  const double a2 = s * delta + co * c * g;
-  const double a3 = so * g;
-  const double eta = sc[MS_ETA];
-  if (!(a1 > 0.0) || !isfinite(a1)) {
-    sc[MS_DONE] = 2.0;
-    sc[MS_UPD_SKIP] = 1.0;
-    return;
-  }
-  const double cn = a0 / a1, sn = gn / a1;
-  sc[MS_A1] = a1;
-  sc[MS_A2] = a2;
-  sc[MS_A3] = a3;
-  sc[MS_XCOEF] = cn * eta;
-  sc[MS_INV_GAMMA_PREV] = 1.0 / g;
-  sc[MS_UPD_SKIP] = 0.0;
-  sc[MS_ETA] = -sn * eta;
-  sc[MS_C_OLD] = c;
-  sc[MS_C] = cn;
-  sc[MS_S_OLD] = s;
-  sc[MS_S] = sn;
-  sc[MS_GAMMA_OLD] = g;
-  sc[MS_GAMMA] = gn;
-  sc[MS_ITERS] += 1.0;
-  if (fabs(sc[MS_ETA]) <= sc[MS_TOL_ABS] || !(gn > 0.0)) sc[MS_DONE] = 1.0;
-}
-
+// MINRES scalar recurrence, one thread per problem
 __global__ void scalars_batch_kernel(const KTask* __restrict__ tasks, int ntasks) {
   grid_dep_entry();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= ntasks) return;
   double* sc = tasks[p].sc;
-  scalars_one(sc);
+  minres_scalars(sc);
   if (tasks[p].c) tasks[p].c[0] = sc[MS_DONE];  // contiguous copy of the done flags for the host
 }
-
 
 inline unsigned chunks(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 

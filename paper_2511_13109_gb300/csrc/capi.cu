@@ -1143,9 +1143,9 @@ struct BatchStep {
   size_t off;      // byte offset of the task array in the task table
   int ntasks;
   int64_t work;    // tiles (stencil), max count (xfer), max n (krylov)
-  int max_m;       // coarsest solve size; transfers: cubes per axis of the largest
-                   // grid written; FP32 tiles: results widened to FP64
+  int largest = 0; // transfers: cubes per axis of the largest grid written; coarsest solves: most unknowns
   int ncomp = 0;   // components (transfers)
+  bool wide = false;  // FP32 tiles: results widened to FP64
 };
 
 }  // namespace
@@ -1224,7 +1224,7 @@ template <typename T>
 void push_gather(std::vector<BatchStep>& steps, const std::vector<StencilTask<T, T>>& t, size_t off, int prec) {
   int64_t mx = 0;
   for (const auto& tk : t) mx = std::max(mx, tk.op.sten ? tk.op.n_sv : 0);
-  if (mx > 0) steps.push_back(BatchStep{5, 0, prec, true, off, (int)t.size(), mx, 0});
+  if (mx > 0) steps.push_back(BatchStep{5, 0, prec, true, off, (int)t.size(), mx});
 }
 
 template <typename TS, typename T>
@@ -1237,7 +1237,7 @@ void push_stencil(agca_batch* b, std::vector<BatchStep>& steps, int mode, bool c
       if (!small.empty()) {
         int64_t mx = 0;
         for (const auto& tk : small) mx = std::max<int64_t>(mx, tk.op.n);
-        steps.push_back(BatchStep{3, mode, prec, coarse, push_tasks(b, small), (int)small.size(), mx, 0});
+        steps.push_back(BatchStep{3, mode, prec, coarse, push_tasks(b, small), (int)small.size(), mx});
       }
       t.swap(large);
     }
@@ -1273,7 +1273,7 @@ void push_stencil(agca_batch* b, std::vector<BatchStep>& steps, int mode, bool c
       }
       const size_t off = push_tasks(b, u);
       push_gather(steps, u, off, prec);
-      steps.push_back(BatchStep{4, mode, prec, sten, off, (int)u.size(), tiles, u[0].a.out64 ? 1 : 0});
+      steps.push_back(BatchStep{4, mode, prec, sten, off, (int)u.size(), tiles, 0, 0, u[0].a.out64 != nullptr});
     }
     return;
   }
@@ -1295,7 +1295,7 @@ void push_stencil(agca_batch* b, std::vector<BatchStep>& steps, int mode, bool c
   if constexpr (std::is_same<TS, T>::value) {
     if (coarse) push_gather(steps, t, off, prec);
   }
-  BatchStep st{0, mode, prec, coarse, off, (int)t.size(), tiles, 0};
+  BatchStep st{0, mode, prec, coarse, off, (int)t.size(), tiles};
   steps.push_back(st);
 }
 
@@ -1317,7 +1317,7 @@ void push_krylov(agca_batch* b, std::vector<BatchStep>& steps, int op, const std
   if (t.empty()) return;
   int64_t mx = 0;
   for (auto& tk : t) mx = std::max(mx, tk.n);
-  BatchStep st{2, op, 0, false, push_tasks(b, t), (int)t.size(), mx, 0};
+  BatchStep st{2, op, 0, false, push_tasks(b, t), (int)t.size(), mx};
   steps.push_back(st);
 }
 
@@ -1325,7 +1325,6 @@ void push_krylov(agca_batch* b, std::vector<BatchStep>& steps, int op, const std
 template <typename T>
 void build_cycle(agca_batch* b, std::vector<BatchStep>& steps, const std::vector<const double*>& r,
                  const std::vector<double*>& z, bool skip_done) {
-  const int P = b->n;
   const int pr = std::is_same<T, float>::value ? 1 : 0;
   const bool mixed = std::is_same<T, float>::value;
   int maxL = 0;
@@ -1571,15 +1570,15 @@ agca_status run_steps(agca_batch* b, const std::vector<BatchStep>& steps, int64_
         BCK(launch_gather_batch<float>((const StencilTask<float, float>*)t, st.ntasks, st.work, s));
       *launches += 1;
     } else if (st.kind == 4) {
-      BCK(launch_stencil_f32_batch(st.mode, st.coarse, st.max_m != 0,
+      BCK(launch_stencil_f32_batch(st.mode, st.coarse, st.wide,
                                    reinterpret_cast<const StencilTask<float, float>*>(b->host_tab.data() + st.off),
                                    st.ntasks, s));
       *launches += st.ntasks <= 24 ? 1 : (st.ntasks + kF32BatchTasks - 1) / kF32BatchTasks;
     } else if (st.kind == 1) {
       if (st.prec == 1)
-        BCK(launch_xfer_batch<float>(st.mode, st.ncomp, (const XferTask*)t, st.ntasks, st.work, st.max_m, s));
+        BCK(launch_xfer_batch<float>(st.mode, st.ncomp, (const XferTask*)t, st.ntasks, st.work, st.largest, s));
       else
-        BCK(launch_xfer_batch<double>(st.mode, st.ncomp, (const XferTask*)t, st.ntasks, st.work, st.max_m, s));
+        BCK(launch_xfer_batch<double>(st.mode, st.ncomp, (const XferTask*)t, st.ntasks, st.work, st.largest, s));
       *launches += 1;
     } else {
       BCK(launch_krylov_batch(st.mode, (const KTask*)t, st.ntasks, st.work, b->partials, s));

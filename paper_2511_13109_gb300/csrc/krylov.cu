@@ -10,6 +10,7 @@
 #include <cooperative_groups.h>
 
 #include "agca_internal.cuh"
+#include "device_ops.cuh"
 
 namespace agca {
 
@@ -164,44 +165,6 @@ __global__ void __launch_bounds__(kRedThreads) pdiv_kernel(int64_t n, const doub
         acc += v;
       });
   if (grid_sum(acc, partials, counter, &total)) sc[MS_TMP1] = total / (double)n;
-}
-
-__device__ void minres_scalars(double* sc) {
-  if (sc[MS_DONE] != 0.0) {
-    sc[MS_UPD_SKIP] = 1.0;  // iterations past convergence change nothing
-    return;
-  }
-  const double g = sc[MS_GAMMA];
-  const double delta = sc[MS_DOT_KZZ] / (g * g);
-  const double gn2 = sc[MS_DOT_ZV];
-  const double gn = gn2 > 0.0 ? sqrt(gn2) : 0.0;
-  const double c = sc[MS_C], co = sc[MS_C_OLD], s = sc[MS_S], so = sc[MS_S_OLD];
-  const double a0 = c * delta - co * s * g;
-  const double a1 = sqrt(a0 * a0 + gn * gn);
-  const double a2 = s * delta + co * c * g;
-  const double a3 = so * g;
-  const double eta = sc[MS_ETA];
-  if (!(a1 > 0.0) || !isfinite(a1)) {  // exact convergence or breakdown
-    sc[MS_DONE] = 2.0;
-    sc[MS_UPD_SKIP] = 1.0;
-    return;
-  }
-  const double cn = a0 / a1, sn = gn / a1;
-  sc[MS_A1] = a1;
-  sc[MS_A2] = a2;
-  sc[MS_A3] = a3;
-  sc[MS_XCOEF] = cn * eta;
-  sc[MS_INV_GAMMA_PREV] = 1.0 / g;
-  sc[MS_UPD_SKIP] = 0.0;
-  sc[MS_ETA] = -sn * eta;
-  sc[MS_C_OLD] = c;
-  sc[MS_C] = cn;
-  sc[MS_S_OLD] = s;
-  sc[MS_S] = sn;
-  sc[MS_GAMMA_OLD] = g;
-  sc[MS_GAMMA] = gn;
-  sc[MS_ITERS] += 1.0;
-  if (fabs(sc[MS_ETA]) <= sc[MS_TOL_ABS] || !(gn > 0.0)) sc[MS_DONE] = 1.0;
 }
 
 // z_p -= sc[MS_TMP1] (entries n3 and on), then z . v and the recurrence's scalars
@@ -415,17 +378,6 @@ __global__ void __launch_bounds__(kRedThreads) block_axpy_kernel(int nvec, const
   }
 }
 
-// y = a * s (s on the device)
-__global__ void scale_kernel(int64_t n, double* __restrict__ y, const double* __restrict__ a,
-                             const double* __restrict__ s, int recip) {
-  grid_dep_entry();
-  const double f = recip ? 1.0 / s[0] : s[0];
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-    y[q] = a[q] * f;
-}
-
-// conjugate-gradient vector updates on the device scalars sc: x += alpha p,
-// r -= alpha q with alpha = sc[0] / sc[1]; p = z + beta p with beta = sc[2] / sc[0]
 // Assembled Z = B W^-1 B^T on the pressure grid (np cubes per axis).  A
 // pressure hat and a velocity hat overlap only where their Kuhn
 // neighbourhoods meet, so Z couples pressure vertices whose offset is a sum
@@ -646,11 +598,6 @@ cudaError_t launch_block_dot(int nvec, const double* V, int64_t ld, const double
 cudaError_t launch_block_axpy(int nvec, const double* V, int64_t ld, const double* coef, double sign, double* w,
                               int64_t n, cudaStream_t s) {
   KL(launch_k(block_axpy_kernel, dim3(kRedBlocks), dim3(kRedThreads), 0, s, nvec, V, ld, coef, sign, w, n));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_scale(int64_t n, double* y, const double* a, const double* s_dev, bool recip, cudaStream_t s) {
-  KL(launch_k(scale_kernel, dim3(kRedBlocks), dim3(kRedThreads), 0, s, n, y, a, s_dev, recip ? 1 : 0));
   return cudaGetLastError();
 }
 
