@@ -221,7 +221,9 @@ __global__ void galerkin_kernel(const RefineTables rt, int nc, int64_t n_flag, c
                                 const int32_t* __restrict__ fidx_f, const double* __restrict__ gca_f,
                                 double* __restrict__ gca_c) {
   grid_dep_entry();
-  constexpr int R = 128;  // |4 P^T K' P| <= 4 * 16 * max |K'| is far below
+  // 2 P^T takes the child's scaled gradients to the parent's, whose entries are
+  // -1, 0 or 1: |4 P^T K' P| <= 3; products of two weights (2 P) are at most 4
+  constexpr int R = 4;
   __shared__ int8_t kp[6][144], pk[6][8][16], ct[6][8];
   __shared__ double quarter[2 * R + 1];  // i / 4
   __shared__ double w[8];

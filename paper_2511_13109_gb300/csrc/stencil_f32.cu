@@ -12,11 +12,11 @@
 // residual.  60 to 96 bytes a vertex at the copy rate leave an SM 90 to 140
 // cycles for each 32 vertices; the per-cube kernel this replaces issued 533
 // instructions a vertex, this one about 320.
-// Measured at 256^3 cubes (per-cube kernel -> this): residual 368 -> 216 us
-// (method's bytes / time: 0.69 of the measured copy rate), first step
-// 392 -> 251 us (0.84), later step with FP64 result 414 -> 326 us, step from
-// zero 444 -> 251 us with x1 written by the producer of b (+36 us there); at
-// 128^3 cubes 66-82 -> 34-46 us.
+// Measured at 256^3 cubes (per-cube kernel -> this; in brackets the method's
+// bytes over the time, of the measured copy rate): residual 368 -> 216 us (0.69),
+// first step 392 -> 251 us (0.72), later step with FP64 result 414 -> 325 us
+// (0.74), step from zero 444 -> 251 us (0.60; 0.72 with its first iterate, which
+// the producer of b writes in 36 us); at 128^3 cubes 66-82 -> 34-46 us.
 //
 // Tiling: a CTA owns 32 x 16 vertex columns starting at vertex (1, 1) and
 // marches a chunk of z-planes; n a multiple of 32 then wastes no lane.  Eight
@@ -136,8 +136,8 @@ __device__ __forceinline__ void f32_block(const LevelOp<float>& op, const Stenci
   // this thread's pieces of a cube layer: the rows start at column x0 - 1, a
   // multiple of 32, and n is even, so they are 16-byte aligned.  A piece that
   // begins beyond the last column or row is not copied: those cubes enter
-  // only Dirichlet outputs.  (The last piece of a row may end 8 bytes past it,
-  // in the next row or the next array of the workspace.)
+  // only Dirichlet outputs.  (A piece that begins within a row ends within it: a
+  // row holds 6 (n - x0 + 1) values from its start, a multiple of four.)
   unsigned cg[(CQ + FNT - 1) / FNT];
 #pragma unroll
   for (int i = 0; i < (CQ + FNT - 1) / FNT; ++i) {

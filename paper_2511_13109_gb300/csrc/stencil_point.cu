@@ -1,18 +1,23 @@
 // Operator application on the small levels (Eq. 2.9), eight lanes per vertex,
 // fused with the smoother and residual epilogues.
 //
-// A level of up to 33^3 vertices does not fill the chip and is bound by the
-// length of its dependency chain: a tile marching z-planes pays a copy wait
+// A tile marching z-planes over a level of up to 33^3 vertices, which does not
+// fill the chip, is bound by the length of its dependency chain: a copy wait
 // and two block barriers per plane (12 to 16 us a launch in FP32, 26 to 60 us
 // in FP64, whatever the level's size).  Here nothing is staged and nothing
-// waits on a barrier.  The operator at a vertex is the difference of the
+// waits on a barrier.  What bounds this kernel is load latency, except in FP64
+// from about 17^3 vertices on: every flux is formed at both its ends and the
+// sums by shuffles add in all lanes, some 35 FP64 warp instructions per four
+// vertices, four times the tiles' arithmetic a vertex, so that at 33^3 vertices
+// the FP64 pipe takes 24 to 26 us a launch (39 for the step from zero, which
+// forms its input on the fly) where FP32 takes 7 (9.5).  The operator at a vertex is the difference of the
 // fluxes along its six axis edges (edge form, see stencil_edge.cu), and lane
 // 2 m + s of a vertex's eight computes one of them: the edge of axis m that
 // ends (s = 0) or starts (s = 1) at the vertex.  All six follow one formula:
 // with c < k the other two axes and S the edge's start vertex,
 //   F[m] = 2 H d[m],   F[c] = H d[c] + sum of four differences along c of
 //   component m, at S + e_m, S - e_c, S + e_m + e_k and S - e_c - e_k,
-// so a lane's 18 vector values and 6 coefficients (or 9 record values) are
+// so a lane's 12 vector values and 6 coefficients (or 9 record values) are
 // independent loads, and three shuffles add the fluxes as
 //   ((F_x- - F_x+) + (F_y- - F_y+)) + (F_z- - F_z+),
 // the order of the tile kernels of stencil_edge.cu: in FP64 with coefficient

@@ -8,12 +8,12 @@
 // (-B_f^T q)_c at an interior vertex is the same combination of q.  The
 // velocity is zero on the boundary and counts as zero outside it, so the
 // stencil holds at every vertex.  P^T B_f at a pressure vertex K is again one
-// stencil, over 64 offsets of [-2, 2]^3 around 2K (sums of two Kuhn offsets),
-// odd in the offset: 32 differences a component.
+// stencil around 2K, over sums of two Kuhn offsets and odd in the offset: 26
+// differences with a non-zero weight a component.
 //
 // Per tetrahedron, with the coupling recomputed for every element, this took
 // some 190 FP64 operations a vertex (665 us at 128^3 cubes, 0.60 of the
-// operator's time); here they are 21 for the gradient and 24 for the
+// operator's time); here they are 22 for the gradient and 20 for the
 // divergence, and the divergence is formed where the pressure lives, without
 // a fine-grid vector and its restriction: 119 + 94 us, the operator at 64^3
 // pressure cubes 1105 -> 650 us (FP64 pipe-bound, as the viscous part).
@@ -66,6 +66,7 @@ constexpr HalfStencil make_half() {
   return h;
 }
 constexpr HalfStencil kHalf = make_half();
+static_assert(kHalf.n == 26, "differences a component of the divergence");
 
 // sum_q w_q (at(o_q) - at(-o_q)), in the order of q
 template <typename F, int... Q>
