@@ -718,7 +718,9 @@ agca_status project_pressure(agca_ctx* ctx, double* x) {
 // where FP32 arithmetic still converges well, and goes on from the true residual.
 // A floor that the caller set is kept; the default one is undercut, by up to
 // kInnerReach, where that ends the solve: stopping just short of it, the result
-// lay barely below or barely above the tolerance, by chance.
+// lay barely below or barely above the tolerance, by chance.  Over 34 solves of
+// contrasts 1e2 to 1e6 to 1e-5 .. 1e-10, a reach of 30 changes the iterations by
+// -9 to +8 % (mean 0), 100 by -17 to +20 % and 1000 costs 2.4 % on average.
 constexpr double kInnerReach = 30.0;
 double inner_tolerance(const agca_ctx* ctx, double want) {
   if (ctx->prec == AGCA_MIXED && want < ctx->mixed_inner &&
